@@ -356,11 +356,6 @@ __device__ __forceinline__ void block_sum(double (&v)[N], double *out) {
 //   J = 4: explicit Euler comparison scheme, f^{n+1} = f^n + dt (Gamma^a + Gamma^c), into fs_out
 // The accumulator inputs are read through (pointer, row stride, column): a1 is f^n (J = 1),
 // B (J = 2) or C (J = 3); a2 is C (J = 2).  Outputs go to global memory at cell i.
-//   FN_FROM_F1: unless fn_read, f^n is not read but recovered from f^(1) = [f^n + z/4 f^eq] /
-//   (1 + z/4) as f^n = f^(1) - dt/4 Gamma^c(1) (same moments, so f^eq(1) follows from f^(1));
-//   the recovery multiplies the rounding of f^(1) by z/4, so with large z (local time steps)
-//   the caller sets fn_read and f^n is read from fn at cell i instead;
-//   frel (if given): at J = 3, laminar instances also store f^(1) of the next step.
 // The collision terms are formed from differences that are not scaled by z: with
 // f^(J) = (X + zJ f^eq) / (1 + zJ), dt Gamma^c(J) = dt/tau (f^eq - X) / (1 + zJ) exactly, so a
 // rounding of X or f^eq is multiplied by dt/tau / (1 + zJ) <= 1/m_JJ instead of dt/tau.
@@ -388,8 +383,8 @@ __device__ __forceinline__ void store_stage(T *__restrict__ f, size_t np, int i,
 }
 
 // EQ1_IN_A2 (stage 1): f^eq(f^n) is given in a2 (the face-value stage relaxed the cell with it).
-template <class T, int STAGE, bool STATS, int NT, bool FN_FROM_F1 = false, bool ROWS = false,
-          bool EQ1_IN_A2 = false>
+// ROWS also leaves out C_0, which is 0 (e_0 carries no flux).
+template <class T, int STAGE, bool STATS, int NT, bool ROWS = false, bool EQ1_IN_A2 = false>
 __device__ __forceinline__ void stage_algebra(int i, size_t np, const T *fi, const T *acc,
                                               const InstParam &P, T t_i, T dt_i, const T *a1, size_t ld1,
                                               int c1, const T *a2, size_t ld2, int c2,
@@ -397,9 +392,7 @@ __device__ __forceinline__ void stage_algebra(int i, size_t np, const T *fi, con
                                               T *__restrict__ Bacc, T *__restrict__ Cacc,
                                               T *__restrict__ mac, double *__restrict__ partial,
                                               const T *__restrict__ area,
-                                              T *__restrict__ frel = nullptr,
-                                              bool fn_read = false, T t1_i = T(0),
-                                              T *macv = nullptr) {
+                                              T t1_i = T(0), T *macv = nullptr) {
     const T rho0 = ipv<T>(P.rho0, P.rho0_f);
     const T dt = dt_i;
     const T itau = sdiv(T(1), t_i);     // one division per cell, products below
@@ -411,17 +404,9 @@ __device__ __forceinline__ void stage_algebra(int i, size_t np, const T *fi, con
         const T z = dt * itau;
         const T zq = z * T(0.25);
         const T inv = sdiv(T(1), T(1) + zq);
-        if (FN_FROM_F1 && !fn_read) {
-            moments(fi, rho0, dr, r, u, v);
-            feq_dev(dr, r, u, v, eq);
+        {
 #pragma unroll
-            for (int a = 0; a < kQ; ++a) {
-                dgc1[a] = (eq[a] - fi[a]) * z;
-                f0[a] = fi[a] - T(0.25) * dgc1[a];
-            }
-        } else {
-#pragma unroll
-            for (int a = 0; a < kQ; ++a) f0[a] = FN_FROM_F1 ? fn[a * np + i] : a1[a * ld1 + c1];
+            for (int a = 0; a < kQ; ++a) f0[a] = a1[a * ld1 + c1];
             if constexpr (EQ1_IN_A2) {
 #pragma unroll
                 for (int a = 0; a < kQ; ++a) eq[a] = a2[a * ld2 + c2];
@@ -450,7 +435,7 @@ __device__ __forceinline__ void stage_algebra(int i, size_t np, const T *fi, con
             f2[a] = (X[a] + zq * eq[a]) * inv;
             const T dgc2 = (eq[a] - X[a]) * s2;  // dt Gamma^c(2)
             Bacc[a * np + i] = X[a] + T(1.0 / 3.0) * (dgc1[a] + dgc2);
-            Cacc[a * np + i] = dt6 * acc[a];
+            if (!ROWS || a > 0) Cacc[a * np + i] = dt6 * acc[a];
         }
         store_stage<T, ROWS>(fs_out, np, i, f2);
     } else if (STAGE == 2) {
@@ -464,7 +449,7 @@ __device__ __forceinline__ void stage_algebra(int i, size_t np, const T *fi, con
 #pragma unroll
         for (int a = 0; a < kQ; ++a) {
             f3[a] = (X[a] + zt * eq[a]) * inv;
-            Cacc[a * np + i] = a2[a * ld2 + c2] + dt6 * acc[a];
+            if (!ROWS || a > 0) Cacc[a * np + i] = a2[a * ld2 + c2] + dt6 * acc[a];
         }
         store_stage<T, ROWS>(fs_out, np, i, f3);
     } else if (STAGE == 4) {
@@ -490,7 +475,8 @@ __device__ __forceinline__ void stage_algebra(int i, size_t np, const T *fi, con
     } else {
         T fnew[kQ], dr, r, u, v;
 #pragma unroll
-        for (int a = 0; a < kQ; ++a) fnew[a] = fi[a] + a1[a * ld1 + c1] - dt3 * acc[a];
+        for (int a = 0; a < kQ; ++a)
+            fnew[a] = ROWS && a == 0 ? fi[a] : fi[a] + a1[a * ld1 + c1] - dt3 * acc[a];
         store9(fn, np, i, fnew);
         moments(fnew, rho0, dr, r, u, v);
         if (STATS) {
@@ -509,10 +495,6 @@ __device__ __forceinline__ void stage_algebra(int i, size_t np, const T *fi, con
             macv[1] = u;
             macv[2] = v;
         }
-        if (frel != nullptr && !P.sst) {  // laminar: tau is constant, relax for the next step
-            relax9(fnew, rho0, dt, t_i);
-            store9(frel, np, i, fnew);
-        }
     }
 }
 
@@ -526,7 +508,7 @@ __device__ __forceinline__ void stage_update(int i, size_t np, const T *fi, cons
                                              const T *__restrict__ area, T dt_i, T t1_i) {
     const T *a1 = STAGE == 1 ? fn : (STAGE == 2 ? Bacc : Cacc);
     stage_algebra<T, STAGE, STATS, NT>(i, np, fi, acc, P, tau[i], dt_i, a1, np, i, Cacc, np, i, fs_out,
-                                       fn, Bacc, Cacc, mac, partial, area, nullptr, false, t1_i);
+                                       fn, Bacc, Cacc, mac, partial, area, t1_i);
 }
 
 // ------------------------------------------------------------------ flux + stage solve
@@ -578,33 +560,14 @@ __global__ void __launch_bounds__(kTile)
                                          (STAGE == 1 && tau1 != nullptr) ? tau1[i] : T(0));
 }
 
-// ------------------------------------------------------------------ fused stage kernel
-// Per block of kBlock consecutive cells (compact patch, see the host renumbering): the ring-1
-// and ring-2 halo cells are listed on the host; the local adjacency of block and ring-1 cells
-// is stored with 16-bit local indices.  Encoding of one adjacency word: kAdjNone (no face),
-// kAdjBnd | global boundary face, or local index | back slot << 16 | (neighbour is a
-// triangle) << 18.
-constexpr int kFusedSmemCap = 200 * 1024;  // dynamic shared memory cap of the fused kernel
-constexpr unsigned kAdjNone = 0xFFFFFFFFu;
-constexpr unsigned kAdjBnd = 0x80000000u;
+// ------------------------------------------------------------------ fused stages: shared pieces
 constexpr long long kWaitLimit = 1ll << 26;  // bounded spin on the staging barrier
 
-struct Halo {
-    const int *__restrict__ halo_ptr;   // [nblk + 1] offsets into halo
-    const int *__restrict__ halo;       // global ids: ring 1 then ring 2, per block
-    const int *__restrict__ r1;         // [nblk] ring-1 count
-    const int *__restrict__ adj_ptr;    // [nblk + 1] offsets (cells) into adj / 4
-    const unsigned *__restrict__ adj;   // per block [4][kBlock + r1] adjacency words
-    int *__restrict__ err;              // set to 1 if a staging wait gave up
-    int emax, gmax;                     // smem row strides: max ext cells, max gradient cells
-    long long wait_first;               // polls of the first staging wait (fvlbm_set_wait_limit)
-};
-
-// Compact geometry of the fused kernels: per cell the node positions relative to the centroid
-// (gq, face m joins nodes m and m+1) and, per face slot, d_m = neighbour centroid (periodic
-// shift included) or face midpoint, minus the own centroid.  Everything else is derived:
-// area and n dl / A from gq, the face offset r_m = face midpoint - centroid from gq, the
-// neighbour's offset r_m - d_m, and the least-squares weights M^{-1} d_m.
+// Compact geometry of the SST kernels beside the fused stages: per cell the node positions
+// relative to the centroid (gq, face m joins nodes m and m+1) and, per face slot, d_m = neighbour
+// centroid (periodic shift included) or face midpoint, minus the own centroid.  Everything else
+// is derived: area and n dl / A from gq, the face offset r_m = face midpoint - centroid from gq
+// and the neighbour's offset r_m - d_m.
 template <class T>
 struct CompactGeo {
     const T *__restrict__ gq;    // [8 np]
@@ -681,235 +644,6 @@ __device__ __forceinline__ int4 ld_keep(const int4 *a, unsigned long long pol) {
         : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
         : "l"(a), "l"(pol));
     return v;
-}
-
-// Face m of a cell whose node positions (relative to its centroid) are q[(2k + c) * ld]:
-// midpoint r = (q_m + q_{m+1}) / 2 and edge vector e = q_{m+1} - q_m.
-template <class T>
-__device__ __forceinline__ void face_geo_s(const T *q, int ld, int m, int nv, T &rx, T &ry,
-                                           T &exv, T &eyv) {
-    const int m1 = (m + 1 == nv) ? 0 : m + 1;
-    const T x0 = q[(2 * m) * ld], y0 = q[(2 * m + 1) * ld];
-    const T x1 = q[(2 * m1) * ld], y1 = q[(2 * m1 + 1) * ld];
-    rx = T(0.5) * (x0 + x1);
-    ry = T(0.5) * (y0 + y1);
-    exv = x1 - x0;
-    eyv = y1 - y0;
-}
-
-// Shared-memory layout of the fused kernel (element offsets, every row 16-byte aligned):
-//   sf  [9][emax]   f^(J) of block, ring-1 and ring-2 cells
-//   sg  [gmax][17]  gradients (alpha = 1..8; x, y) of block and ring-1 cells, cell-major
-//   sD  [8][gmax]   neighbour-centroid offsets d_m of block and ring-1 cells
-//   adj [4 gmax] words, then one 8-byte mbarrier
-
-// Gradients in shared memory are cell-major, 16 values (alpha = 1..8, x and y) in a row of 17
-// words: one base address per cell serves all 16 reads (immediate offsets), and the odd row
-// length keeps consecutive cells in distinct banks.
-constexpr int kGradStride = 17;
-
-template <class T>
-struct FusedSmem {
-    static __host__ __device__ size_t elems(int emax, int gmax) {
-        return size_t(kQ) * emax + size_t(kGradStride) * gmax + 8u * gmax;
-    }
-    static __host__ __device__ size_t bytes(int emax, int gmax) {
-        return elems(emax, gmax) * sizeof(T) + 4u * gmax * sizeof(unsigned) + 16;
-    }
-};
-
-// One IMEX stage for a block of BLK cells (BLK = 128 or 256), one thread per cell.  Staging: the block's own
-// rows (contiguous in every SoA array) arrive by bulk copies on one mbarrier; halo rows are
-// gathered with cp.async; each thread's accumulators, tau and face normals go straight into
-// registers; nothing is waited for until everything has been issued.  Then: least-squares
-// gradients of block + ring-1 cells, and per block cell the flux of Eq. (advection) and the
-// local stage algebra.  No gradient array goes through HBM.  alpha = 0 has e = 0: no gradient
-// and no flux.  Stage 1 stages f^(1), which the previous step (laminar instances) or the SST
-// update (turbulent instances, with the new tau) has already relaxed from f^n; stage 3 writes
-// f^(1) of the next step for laminar instances into frel.
-template <class T, int STAGE, bool STATS, int BLK>
-__global__ void __launch_bounds__(BLK, sizeof(T) == 4 ? (768 / BLK) : 1)
-    k_fused_stage(const T *__restrict__ fin, T *__restrict__ fs_out, T *__restrict__ fn,
-                  T *__restrict__ Bacc, T *__restrict__ Cacc, const T *__restrict__ tau,
-                  T *__restrict__ mac, double *__restrict__ partial, Geo<T> G, Halo H,
-                  T *__restrict__ frel, CompactGeo<T> CG) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    const int E0 = H.emax, G0 = H.gmax;
-    T *sf = reinterpret_cast<T *>(smem_raw);
-    T *sg = sf + kQ * E0;
-    T *sD = sg + kGradStride * G0;
-    unsigned *sAdj = reinterpret_cast<unsigned *>(sD + 8 * G0);
-    unsigned long long *bar = reinterpret_cast<unsigned long long *>(sAdj + 4 * G0);
-
-    const int b = blockIdx.x, t = threadIdx.x;
-    const int base = b * BLK;
-    const int i = base + t;
-    const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[b * (BLK / kTile)]];
-    const T rho0 = ipv<T>(P.rho0, P.rho0_f);
-    const int h0 = H.halo_ptr[b], nh = H.halo_ptr[b + 1] - h0, nr1 = H.r1[b];
-    const int E = BLK + nh, NG = BLK + nr1;
-    const unsigned *__restrict__ adj_g = H.adj + 4 * static_cast<size_t>(H.adj_ptr[b]);
-
-    // 1. issue every copy of the block's data, then wait once
-    if (t == 0) mbar_init(bar);
-    __syncthreads();
-    if (t == 0) {
-        constexpr unsigned row = BLK * sizeof(T);
-        const unsigned adj_bytes = 4u * NG * sizeof(unsigned);
-        mbar_expect_tx(bar, row * (kQ + 8) + adj_bytes);
-        for (int a = 0; a < kQ; ++a) bulk_g2s(sf + a * E0, fin + a * np + base, row, bar);
-        for (int k = 0; k < 8; ++k) bulk_g2s(sD + k * G0, CG.dv + k * np + base, row, bar);
-        bulk_g2s(sAdj, adj_g, adj_bytes, bar);
-    }
-    for (int e = BLK + t; e < E; e += BLK) {  // halo rows
-        const int gid = H.halo[h0 + e - BLK];
-#pragma unroll
-        for (int a = 0; a < kQ; ++a) cp_async<sizeof(T)>(sf + a * E0 + e, fin + a * np + gid);
-        if (e < NG) {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) cp_async<sizeof(T)>(sD + k * G0 + e, CG.dv + k * np + gid);
-        }
-    }
-    // this thread's accumulators, tau and node positions, straight into registers
-    T a1[kQ], a2[kQ], q[8];
-    const T tau_i = tau[i];
-    {
-        if (STAGE != 1) {
-            const T *p1 = STAGE == 2 ? Bacc : Cacc;
-#pragma unroll
-            for (int a = 0; a < kQ; ++a) a1[a] = p1[a * np + i];
-        }
-        if (STAGE == 2) {
-#pragma unroll
-            for (int a = 0; a < kQ; ++a) a2[a] = Cacc[a * np + i];
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) q[k] = CG.gq[k * np + i];
-    }
-    cp_async_wait_all();
-    {
-        long long it = 0;
-        // (a limit of 0 gives up at once, without polling: the diagnostic of the error path)
-        bool done = H.wait_first > 0 && mbar_try_wait(bar, 0);
-        while (!done && ++it < H.wait_first) done = mbar_try_wait(bar, 0);
-        // the block leaves together if any thread gave up: flag it, wait once more (bounded)
-        if (__syncthreads_or(!done)) {
-            if (t == 0) atomicExch(H.err, 1);
-            for (long long k = 0; k < kWaitLimit && !mbar_try_wait(bar, 0); ++k) {
-            }
-            return;
-        }
-    }
-
-    // 2. least-squares gradients (alpha = 1..8) of block and ring-1 cells (Step 2)
-    for (int c = t; c < NG; c += BLK) {
-        T fc[kQ], gx[kQ], gy[kQ];
-#pragma unroll
-        for (int a = 0; a < kQ; ++a) {
-            fc[a] = sf[a * E0 + c];
-            gx[a] = gy[a] = T(0);
-        }
-        // least-squares matrix M = sum_m d_m d_m^T of this cell, inverted once
-        T mxx = 0, mxy = 0, myy = 0;
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            if (sAdj[m * NG + c] == kAdjNone) continue;
-            const T dx = sD[(2 * m) * G0 + c], dy = sD[(2 * m + 1) * G0 + c];
-            mxx += dx * dx;
-            mxy += dx * dy;
-            myy += dy * dy;
-        }
-        const T idet = T(1) / (mxx * myy - mxy * mxy);
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const unsigned w = sAdj[m * NG + c];
-            if (w == kAdjNone) continue;
-            const T dx = sD[(2 * m) * G0 + c], dy = sD[(2 * m + 1) * G0 + c];
-            const T wx = (myy * dx - mxy * dy) * idet, wy = (mxx * dy - mxy * dx) * idet;
-            if (w & kAdjBnd) {
-                const int bf = static_cast<int>(w & ~kAdjBnd);
-                // outward face normal (n dl / A) for the far-field upwind choice
-                const int gid = c < BLK ? base + c : H.halo[h0 + c - BLK];
-                const T nx = G.sn[(2 * m) * np + gid], ny = G.sn[(2 * m + 1) * np + gid];
-                T dr, r, u, v, fb[kQ];
-                moments(fc, rho0, dr, r, u, v);
-                boundary_values(G.btype[bf], G.bval + bf, 0, G.nbt, nx, ny, fc, dr, r, u, v, rho0,
-                                fb);
-#pragma unroll
-                for (int a = 1; a < kQ; ++a) {
-                    const T d = fb[a] - fc[a];
-                    gx[a] += wx * d;
-                    gy[a] += wy * d;
-                }
-            } else {
-                const int j = static_cast<int>(w & 0xFFFFu);
-#pragma unroll
-                for (int a = 1; a < kQ; ++a) {
-                    const T d = sf[a * E0 + j] - fc[a];
-                    gx[a] += wx * d;
-                    gy[a] += wy * d;
-                }
-            }
-        }
-#pragma unroll
-        for (int a = 1; a < kQ; ++a) {
-            sg[c * kGradStride + 2 * a - 2] = gx[a];
-            sg[c * kGradStride + 2 * a - 1] = gy[a];
-        }
-    }
-    __syncthreads();
-
-    // 3. flux of block cell t (Eq. (advection)), then the stage algebra
-    T fi[kQ], acc[kQ];
-#pragma unroll
-    for (int a = 0; a < kQ; ++a) {
-        fi[a] = sf[a * E0 + t];
-        acc[a] = T(0);
-    }
-    const bool tri = sAdj[3 * NG + t] == kAdjNone;
-    // end node of face m (m compile-time): node m + 1, wrapping to node 0 after the last face
-    auto end_x = [&](int m) { return m == 3 ? q[0] : (m == 2 && tri ? q[0] : q[2 * m + 2]); };
-    auto end_y = [&](int m) { return m == 3 ? q[1] : (m == 2 && tri ? q[1] : q[2 * m + 3]); };
-    T a2x = T(0);  // twice the area (shoelace on centroid-relative nodes)
-#pragma unroll
-    for (int m = 0; m < 4; ++m)
-        if (m < 3 || !tri) a2x += q[2 * m] * end_y(m) - end_x(m) * q[2 * m + 1];
-    const T inv_a = a2x > T(0) ? sdiv(T(2), a2x) : T(0);  // padding cells have no faces
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const unsigned w = sAdj[m * NG + t];
-        if (w == kAdjNone) continue;
-        const T x1 = end_x(m), y1 = end_y(m);
-        const T snx = (y1 - q[2 * m + 1]) * inv_a;   // n dl / A
-        const T sny = -(x1 - q[2 * m]) * inv_a;
-        if (w & kAdjBnd) {
-            const int bf = static_cast<int>(w & ~kAdjBnd);
-            T dr, r, u, v, fb[kQ];
-            moments(fi, rho0, dr, r, u, v);
-            boundary_values(G.btype[bf], G.bval + bf, 0, G.nbt, snx, sny, fi, dr, r, u, v, rho0, fb);
-#pragma unroll
-            for (int a = 1; a < kQ; ++a) acc[a] += edot<T>(a, snx, sny) * fb[a];
-        } else {
-            const int j = static_cast<int>(w & 0xFFFFu);
-            // face offsets from this cell's centroid and from the neighbour's
-            const T rox = T(0.5) * (q[2 * m] + x1), roy = T(0.5) * (q[2 * m + 1] + y1);
-            const T rnx = rox - sD[(2 * m) * G0 + t], rny = roy - sD[(2 * m + 1) * G0 + t];
-#pragma unroll
-            for (int a = 1; a < kQ; ++a) {
-                const T en = edot<T>(a, snx, sny);
-                const bool own = en >= T(0);           // upwind side, branch free
-                const int src = own ? t : j;
-                const T rx = own ? rox : rnx, ry = own ? roy : rny;
-                const T *gs = sg + src * kGradStride;
-                const T fv = sf[a * E0 + src] + gs[2 * a - 2] * rx + gs[2 * a - 1] * ry;
-                acc[a] += en * fv;
-            }
-        }
-    }
-    stage_algebra<T, STAGE, STATS, BLK, true>(i, np, fi, acc, P, tau_i, cell_dt(G, P, i), a1, 1, 0, a2, 1,
-                                                        0, fs_out, fn, Bacc, Cacc, mac, partial,
-                                                        G.area, frel, P.local != 0);  // local steps: read f^n
 }
 
 // Sum per-block partials into per-instance totals (one block per instance).
@@ -1276,7 +1010,7 @@ __global__ void __launch_bounds__(kTile)
     }
 }
 
-// The k / omega update and the new relaxation time (and, on the fused path, f^(1)).  In
+// The k / omega update and the new relaxation time.  In
 // float, 5 blocks of 128 per SM (96 registers, a few spilled) run faster than 4 (120).
 // NONORTH compiles the SST reading variants in (2: non-orthogonal diffusion correction, 8:
 // production limiter); without them the kernel keeps the register count (and occupancy) of
@@ -1287,7 +1021,7 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
                  const T *__restrict__ nut, const T *__restrict__ grads,
                  const T *__restrict__ f1a, T *__restrict__ k_out, T *__restrict__ w_out,
                  T *__restrict__ nut_out, T *__restrict__ tau, Geo<T> G,
-                 const T *__restrict__ fn, T *__restrict__ frel, CompactGeo<T> CG,
+                 CompactGeo<T> CG,
                  const T *__restrict__ rec8, const T *__restrict__ rec2, int tile0) {
     const int tile = tile0 + static_cast<int>(blockIdx.x);
     const int i = tile * kTile + threadIdx.x;
@@ -1383,12 +1117,6 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
     w_out[i] = wn;
     nut_out[i] = ntn;
     tau[i] = tnew;
-    if (frel != nullptr) {  // fused path: stage 1's f^(1) with the new relaxation time
-        T f[kQ];
-        load9(fn, np, i, f);
-        relax9(f, ipv<T>(P.rho0, P.rho0_f), dt_i, tnew);
-        store9(frel, np, i, f);
-    }
 }
 
 // ------------------------------------------------------------------ state I/O kernels
@@ -1481,11 +1209,10 @@ __global__ void k_gather_f_all(const T *__restrict__ f, const int *__restrict__ 
 // State input: internal cells [i0, i0 + n), each reading its record at input position
 // inv[i] - po of the concatenated input order (padding cells: inv = -1, left as they are).
 // IN = double: absolute f; IN = float: the FP32 deviation f - w_alpha rho0.  Writes f^n, the
-// macros and f^(1) of the coming step (relaxed like k_stage1, for the fused stages).
+// macros.
 template <class T, class IN>
-__global__ void k_scatter_state(T *__restrict__ f, T *__restrict__ mac, T *__restrict__ frel,
-                                const T *__restrict__ tau, const int *__restrict__ inv, int i0, int n,
-                                int po, Geo<T> G, const IN *__restrict__ in) {
+__global__ void k_scatter_state(T *__restrict__ f, T *__restrict__ mac, const int *__restrict__ inv, int i0,
+                                int n, int po, Geo<T> G, const IN *__restrict__ in) {
     // one thread per internal cell i (the state arrays are written coalesced; the input record
     // of the cell, 9 consecutive values, is read where the input order puts it)
     const int i = i0 + static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
@@ -1513,17 +1240,12 @@ __global__ void k_scatter_state(T *__restrict__ f, T *__restrict__ mac, T *__res
     mac[i] = r;
     mac[np + i] = u;
     mac[2 * np + i] = v;
-    if (frel != nullptr) {  // f^(1) of the coming step, for the forms that stage it
-        relax9(d, ipv<T>(P.rho0, P.rho0_f), cell_dt(G, P, i), tau[i]);
-        store9(frel, np, i, d);
-    }
 }
 
 // The same for a list of cells: position j < n of the input takes internal cell map[j] (the
 // cell lists of fvlbm_set_cells).
 template <class T, class IN>
-__global__ void k_scatter_list(T *__restrict__ f, T *__restrict__ mac, T *__restrict__ frel,
-                               const T *__restrict__ tau, const int *__restrict__ map, int n,
+__global__ void k_scatter_list(T *__restrict__ f, T *__restrict__ mac, const int *__restrict__ map, int n,
                                Geo<T> G, const IN *__restrict__ in) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
@@ -1546,10 +1268,6 @@ __global__ void k_scatter_list(T *__restrict__ f, T *__restrict__ mac, T *__rest
     mac[i] = r;
     mac[np + i] = u;
     mac[2 * np + i] = v;
-    if (frel != nullptr) {
-        relax9(d, ipv<T>(P.rho0, P.rho0_f), cell_dt(G, P, i), tau[i]);
-        store9(frel, np, i, d);
-    }
 }
 
 // Cell lists of one instance (halo exchange of a partitioned mesh): map[j] = the internal id
@@ -1622,11 +1340,10 @@ __global__ void k_pack_cells(const T *__restrict__ f, const T *__restrict__ kk, 
     v[11] = value_of(nut[i]);
 }
 
-// The reverse: f^n (deviation), the macros and, where kept, f^(1) of the coming step (as
-// fvlbm_set_f writes them), k, omega and nu_t of cell map[j] from row j of vals.
+// The reverse: f^n (deviation) and the macros (as fvlbm_set_f writes them), k, omega and nu_t of
+// cell map[j] from row j of vals.
 template <class T>
-__global__ void k_unpack_cells(T *__restrict__ f, T *__restrict__ mac, T *__restrict__ frel,
-                               const T *__restrict__ tau, T *__restrict__ kk, T *__restrict__ ww,
+__global__ void k_unpack_cells(T *__restrict__ f, T *__restrict__ mac, T *__restrict__ kk, T *__restrict__ ww,
                                T *__restrict__ nut, const int *__restrict__ map, int n, Geo<T> G,
                                const double *__restrict__ vals) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1649,10 +1366,6 @@ __global__ void k_unpack_cells(T *__restrict__ f, T *__restrict__ mac, T *__rest
     kk[i] = T(v[9]);
     ww[i] = T(v[10]);
     nut[i] = T(v[11]);
-    if (frel != nullptr) {
-        relax9(d, ipv<T>(P.rho0, P.rho0_f), cell_dt(G, P, i), tau[i]);
-        store9(frel, np, i, d);
-    }
 }
 
 // Output fields[q][j] for the fields q (rho, u, v, k, omega, nu_t) selected by mask bit q.
@@ -1766,25 +1479,19 @@ struct fvlbm_handle {
     int *d_back = nullptr;      // FP64 handles: slot of each face at its neighbour [4 np] (adjoint)
     size_t adj_budget = 0;      // device bytes the adjoint may keep stage values in (0: half the free)
     int total_nc = 0, total_nb = 0;
-    // fused path: per-block halo lists and local adjacency, for each fused block size
-    struct HaloSet {
-        bool ok = false;
-        int blk = 0, nblk = 0, emax = 0, gmax = 0;
-        size_t smem = 0;
-        int *d_halo_ptr = nullptr, *d_halo = nullptr, *d_r1 = nullptr, *d_adj_ptr = nullptr;
-        int *d_inst_blk0 = nullptr;
-        unsigned *d_adj = nullptr;
-    } hs[2];                // [0]: 256-cell blocks, [1]: 128-cell blocks
     struct FvSet {          // work items of the face-value fused kernel (config 3)
         bool ok = false;
+        int it = 0;                             // cells per item (FvShape)
         int nitem = 0, n_split = 0, n_ovf = 0;  // items; blocks split; items using the overflow
         int4 *d_hdr = nullptr;
         int *d_halo = nullptr, *d_ovf = nullptr, *d_inst_item0 = nullptr;
         uint4 *d_adj = nullptr;
+        uint2 *d_cut = nullptr;
+        int4 *d_ghost = nullptr;
+        void *geo = nullptr, *cutc = nullptr;   // geometry of the cells, coefficients of the cuts
     } fv;
     bool fused = false;     // fused kernels available (IMEX scheme, kernel_path 0 or 2)
-    int config = 2;         // 0: fused 256, 1: fused 128, 2: two-pass, 3: face-value fused
-                            // (see fvlbm_autotune)
+    int config = 2;         // 2: two-pass, 3: face-value fused (see fvlbm_autotune)
     int scheme = 0;         // 0: IMEX Runge-Kutta; 1: explicit Euler (comparison scheme)
     int kernel_path = 0;    // as requested at create (fvlbm_params.kernel_path)
     bool limit_f = false;   // an instance uses the limiter variant (two-pass kernels only)
@@ -1807,14 +1514,12 @@ struct fvlbm_handle {
     int *d_err = nullptr;   // device error flag (a staging wait gave up)
     long long wait_first = kWaitLimit;  // polls of the fused kernels' first staging wait
     void *gq = nullptr;     // fused path: node positions minus centroid [8 np]
-    void *geo16 = nullptr;  // face-value path: per cell q[8] then least-squares W[8] [np][16]
     void *dvec = nullptr;   // fused path: neighbour-centroid offsets d_m [8 np]
     InstParam *d_ip = nullptr;
     void *sn = nullptr, *lsq = nullptr, *rown = nullptr, *rnbr = nullptr, *dinv = nullptr;
     void *area = nullptr, *wdist = nullptr, *bval = nullptr, *bnrm = nullptr, *blen = nullptr;
     void *fn = nullptr, *s0 = nullptr, *s1 = nullptr, *bacc = nullptr, *cacc = nullptr;
     void *grad = nullptr, *tau = nullptr, *mac = nullptr;
-    void *frel = nullptr;   // fused path: f^(1) of the coming step (relaxed f^n)
     void *dtc = nullptr;    // local time stepping: dt of each cell (NULL: every instance global)
     void *kk[2] = {nullptr, nullptr}, *ww[2] = {nullptr, nullptr}, *nut[2] = {nullptr, nullptr};
     void *sgrad = nullptr, *f1 = nullptr;
@@ -1893,13 +1598,13 @@ int dalloc(fvlbm_handle *h, void **p, size_t bytes) {
 }
 
 // The device arrays that make up the state a step reads (everything else is scratch):
-// f^n, f^(1) of the coming step, the macros, tau and both k / omega / nu_t ping-pong buffers.
+// f^n, the macros, tau and both k / omega / nu_t ping-pong buffers.
 std::vector<std::pair<void *, size_t>> state_regions(const fvlbm_handle *h) {
     size_t ts = 0;
     dispatch(h->precision, [&](auto z_) { ts = sizeof(z_); });
     const size_t np = h->np;
     std::vector<std::pair<void *, size_t>> st = {
-        {h->fn, kQ * np * ts}, {h->frel, kQ * np * ts}, {h->mac, 3 * np * ts}, {h->tau, np * ts}};
+        {h->fn, kQ * np * ts}, {h->mac, 3 * np * ts}, {h->tau, np * ts}};
     for (int b = 0; b < 2; ++b) {
         st.push_back({h->kk[b], np * ts});
         st.push_back({h->ww[b], np * ts});
@@ -1976,73 +1681,47 @@ enum KernelId {
     K_FUSED1, K_FUSED2, K_FUSED3, K_EULER, K_MACROS
 };
 
-// The three fused stages with BLK-cell blocks (halo set S).
-template <class T, int BLK>
-void enqueue_fused(fvlbm_handle *h, bool stats, const fvlbm_handle::HaloSet &S) {
+// The three stages in the face-value form (config 3): stage 1 reads f^n and writes f^(2) in
+// cell-major rows into s1, stage 2 reads them and writes f^(3) likewise into s0.
+// With stats, stage 3 also writes the items' FP64 partial sums (the caller reduces them).
+template <class T, int IT>
+void fv_stages(fvlbm_handle *h, bool stats) {
     Geo<T> G = geo_of<T>(h);
     cudaStream_t s = h->stream;
     T *fn = static_cast<T *>(h->fn), *s0 = static_cast<T *>(h->s0), *s1 = static_cast<T *>(h->s1);
     T *B = static_cast<T *>(h->bacc), *C = static_cast<T *>(h->cacc);
     T *tau = static_cast<T *>(h->tau), *mac = static_cast<T *>(h->mac);
-    T *fr = static_cast<T *>(h->frel);
-    const Halo H{S.d_halo_ptr, S.d_halo, S.d_r1, S.d_adj_ptr, S.d_adj, h->d_err, S.emax, S.gmax,
-                 h->wait_first};
-    const CompactGeo<T> CG{static_cast<const T *>(h->gq), static_cast<const T *>(h->dvec)};
-    const dim3 fg(S.nblk), fb(BLK);
-    const size_t sm = S.smem;
+    const auto &F = h->fv;
+    const FvItems W{F.d_hdr, F.d_halo, F.d_ovf, F.d_adj, F.d_cut, F.d_ghost, h->d_err, h->wait_first};
+    const T *geo = static_cast<const T *>(F.geo), *cc = static_cast<const T *>(F.cutc);
+    const T *bn = static_cast<const T *>(h->bnrm);
+    const dim3 fg(static_cast<unsigned>(F.nitem)), fb(FvShape<IT>::nt);
+    const size_t sm = FvSmem<T, IT>::bytes;
     launch(h, K_FUSED1, "fused_stage1", [&] {
-        k_fused_stage<T, 1, false, BLK><<<fg, fb, sm, s>>>(fr, s1, fn, B, C, tau, mac, nullptr, G, H, fr, CG);
+        k_fused_fv<T, 1, false, IT><<<fg, fb, sm, s>>>(fn, s1, fn, B, C, tau, mac, nullptr, G, W, geo, cc, bn);
     });
     launch(h, K_FUSED2, "fused_stage2", [&] {
-        k_fused_stage<T, 2, false, BLK><<<fg, fb, sm, s>>>(s1, s0, fn, B, C, tau, mac, nullptr, G, H, fr, CG);
-    });
-    if (stats) {
-        launch(h, K_FUSED3, "fused_stage3", [&] {
-            k_fused_stage<T, 3, true, BLK><<<fg, fb, sm, s>>>(s0, s1, fn, B, C, tau, mac, h->d_partial, G, H, fr,
-                                                              CG);
-        });
-        launch(h, K_REDUCE, "reduce", [&] {
-            k_reduce_instances<<<h->ninst, kTile, 0, s>>>(h->d_partial, S.d_inst_blk0, h->d_inst_sums);
-        });
-    } else {
-        launch(h, K_FUSED3, "fused_stage3", [&] {
-            k_fused_stage<T, 3, false, BLK><<<fg, fb, sm, s>>>(s0, s1, fn, B, C, tau, mac, nullptr, G, H, fr, CG);
-        });
-    }
-}
-
-// The three stages in the face-value form (config 3): stage 1 reads f^n and writes f^(2) in
-// cell-major rows into s1, stage 2 reads them and writes f^(3) likewise into s0.
-// The three face-value stages over items [item0, item0 + nitem) on stream s; with stats,
-// stage 3 also writes the items' FP64 partial sums (the caller reduces them).
-template <class T>
-void fv_stages(fvlbm_handle *h, bool stats, int item0, int nitem, cudaStream_t s) {
-    Geo<T> G = geo_of<T>(h);
-    T *fn = static_cast<T *>(h->fn), *s0 = static_cast<T *>(h->s0), *s1 = static_cast<T *>(h->s1);
-    T *B = static_cast<T *>(h->bacc), *C = static_cast<T *>(h->cacc);
-    T *tau = static_cast<T *>(h->tau), *mac = static_cast<T *>(h->mac);
-    const FvItems W{h->fv.d_hdr, h->fv.d_halo, h->fv.d_ovf, h->fv.d_adj, h->d_err, h->wait_first, item0};
-    const T *geo = static_cast<const T *>(h->geo16);
-    const dim3 fg(static_cast<unsigned>(nitem)), fb(kFvThreads);
-    const size_t sm = FvSmem<T>::bytes;
-    launch(h, K_FUSED1, "fused_stage1", [&] {
-        k_fused_fv<T, 1, false><<<fg, fb, sm, s>>>(fn, s1, fn, B, C, tau, mac, nullptr, G, W, geo);
-    });
-    launch(h, K_FUSED2, "fused_stage2", [&] {
-        k_fused_fv<T, 2, false><<<fg, fb, sm, s>>>(s1, s0, fn, B, C, tau, mac, nullptr, G, W, geo);
+        k_fused_fv<T, 2, false, IT><<<fg, fb, sm, s>>>(s1, s0, fn, B, C, tau, mac, nullptr, G, W, geo, cc, bn);
     });
     launch(h, K_FUSED3, "fused_stage3", [&] {
         if (stats)
-            k_fused_fv<T, 3, true><<<fg, fb, sm, s>>>(s0, s1, fn, B, C, tau, mac, h->d_partial, G, W, geo);
+            k_fused_fv<T, 3, true, IT><<<fg, fb, sm, s>>>(s0, s1, fn, B, C, tau, mac, h->d_partial, G, W, geo, cc, bn);
         else
-            k_fused_fv<T, 3, false><<<fg, fb, sm, s>>>(s0, s1, fn, B, C, tau, mac, nullptr, G, W, geo);
+            k_fused_fv<T, 3, false, IT><<<fg, fb, sm, s>>>(s0, s1, fn, B, C, tau, mac, nullptr, G, W, geo, cc, bn);
     });
+}
+
+// f(std::integral_constant<int, IT>) for the handle's item size.
+template <class F>
+auto fv_dispatch(int it, F &&f) {
+    if (it == 256) return f(std::integral_constant<int, 256>());
+    return f(std::integral_constant<int, 64>());
 }
 
 template <class T>
 void enqueue_fused_fv(fvlbm_handle *h, bool stats) {
     cudaStream_t s = h->stream;
-    fv_stages<T>(h, stats, 0, h->fv.nitem, s);
+    fv_dispatch(h->fv.it, [&](auto it) { fv_stages<T, decltype(it)::value>(h, stats); });
     if (stats)
         launch(h, K_REDUCE, "reduce", [&] {
             k_reduce_instances<<<h->ninst, kTile, 0, s>>>(h->d_partial, h->fv.d_inst_item0, h->d_inst_sums);
@@ -2082,10 +1761,10 @@ void sst_update_twopass(const fvlbm_handle *h, const T *mac, const T *kc, const 
     for_sst_runs(h, [&](dim3 g, int t0) {
         if (h->nonorth)
             k_sst_update<T, false, true><<<g, kTile, 0, h->stream>>>(mac, kc, wc, nc, sg, f1, kn, wn, nn, tau_out,
-                                                                     G, nullptr, nullptr, CG, nullptr, nullptr, t0);
+                                                                     G, CG, nullptr, nullptr, t0);
         else
             k_sst_update<T, false, false><<<g, kTile, 0, h->stream>>>(mac, kc, wc, nc, sg, f1, kn, wn, nn, tau_out,
-                                                                      G, nullptr, nullptr, CG, nullptr, nullptr, t0);
+                                                                      G, CG, nullptr, nullptr, t0);
     });
 }
 
@@ -2106,7 +1785,7 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
         T *sg = static_cast<T *>(h->sgrad), *f1 = static_cast<T *>(h->f1);
         const CompactGeo<T> CG{static_cast<const T *>(h->gq), static_cast<const T *>(h->dvec)};
         if constexpr (kHasFused<T>) {
-            if (h->config != 2) {  // compact geometry, and stage 1's f^(1) with the new tau
+            if (h->config != 2) {  // compact geometry, packed records
                 T *r8 = static_cast<T *>(h->sst_rec8), *r2 = static_cast<T *>(h->sst_rec2);
                 launch(h, K_SST_GRAD, "sst_grad", [&] {
                     for_sst_runs(h, [&](dim3 sg_grid, int t0) {
@@ -2115,16 +1794,13 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
                     });
                 });
                 launch(h, K_SST_UPDATE, "sst_update", [&] {
-                    // the face-value stages relax f^n themselves; the other fused form reads
-                    // stage 1's f^(1), relaxed here with the new tau
-                    T *fr = h->config == 3 ? nullptr : static_cast<T *>(h->frel);
                     for_sst_runs(h, [&](dim3 sg_grid, int t0) {
                         if (h->nonorth)
                             k_sst_update<T, true, true><<<sg_grid, block, 0, s>>>(
-                                mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, fn, fr, CG, r8, r2, t0);
+                                mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
                         else
                             k_sst_update<T, true, false><<<sg_grid, block, 0, s>>>(
-                                mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, fn, fr, CG, r8, r2, t0);
+                                mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
                     });
                 });
             }
@@ -2200,14 +1876,6 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
             enqueue_fused_fv<T>(h, stats);
             return;
         }
-        if (h->config == 0) {
-            enqueue_fused<T, 256>(h, stats, h->hs[0]);
-            return;
-        }
-        if (h->config == 1) {
-            enqueue_fused<T, 128>(h, stats, h->hs[1]);
-            return;
-        }
     }
     launch(h, K_STAGE1, "stage1", [&] { k_stage1<T><<<grid, block, 0, s>>>(fn, s0, tau, G); });
     launch(h, K_GRAD, "grad_f", [&] { grad_f<T>(h, grid, block, s, s0, g, G); });
@@ -2262,113 +1930,29 @@ int build_graph(fvlbm_handle *h, int nsteps, cudaGraphExec_t *out) {
     return FVLBM_OK;
 }
 
-// Per block of blk cells: ring-1 and ring-2 halo lists and the local adjacency of block and
-// ring-1 cells.  The set is marked unusable (ok = false) when a block's halo does not fit the
-// 16-bit local index or the shared-memory budget; the two-pass kernels then serve.
-template <class T>
-int build_halos(fvlbm_handle *h, fvlbm_handle::HaloSet &S, int blk, const std::vector<int> &nbr,
-                const std::vector<int> &back, const std::vector<int> &nface,
-                const std::vector<int> &inst_tile0) {
-    const size_t np = h->np;
-    S.blk = blk;
-    S.nblk = static_cast<int>(np / blk);
-    std::vector<int> local(np, -1), halo_ptr(1, 0), halo, r1n, adj_ptr(1, 0);
-    std::vector<unsigned> adj;
-    int emax = 0, gmax = 0;
-    std::vector<int> ring1, ring2;
-    for (int b = 0; b < S.nblk; ++b) {
-        const int base = b * blk;
-        for (int c = 0; c < blk; ++c) local[base + c] = c;
-        ring1.clear();
-        ring2.clear();
-        int next = blk;
-        for (int c = 0; c < blk; ++c)
-            for (int m = 0; m < 4; ++m) {
-                const int v = nbr[m * np + base + c];
-                if (v >= 0 && local[v] < 0) { local[v] = next++; ring1.push_back(v); }
-            }
-        for (int g : ring1)
-            for (int m = 0; m < 4; ++m) {
-                const int v = nbr[m * np + g];
-                if (v >= 0 && local[v] < 0) { local[v] = next++; ring2.push_back(v); }
-            }
-        const int E = next, NG = blk + static_cast<int>(ring1.size());
-        emax = std::max(emax, E);
-        gmax = std::max(gmax, NG);
-        halo.insert(halo.end(), ring1.begin(), ring1.end());
-        halo.insert(halo.end(), ring2.begin(), ring2.end());
-        halo_ptr.push_back(static_cast<int>(halo.size()));
-        r1n.push_back(static_cast<int>(ring1.size()));
-        const size_t a0 = adj.size();
-        adj.resize(a0 + 4 * static_cast<size_t>(NG), kAdjNone);
-        for (int c = 0; c < NG; ++c) {
-            const int g = c < blk ? base + c : ring1[c - blk];
-            for (int m = 0; m < 4; ++m) {
-                const int v = nbr[m * np + g];
-                unsigned w = kAdjNone;
-                if (v == kNone) {
-                    w = kAdjNone;
-                } else if (v < 0) {
-                    w = kAdjBnd | static_cast<unsigned>(-v - 1);
-                } else {
-                    w = static_cast<unsigned>(local[v]) | (static_cast<unsigned>(back[m * np + g]) << 16) |
-                        (nface[v] == 3 ? (1u << 18) : 0u);
-                }
-                adj[a0 + static_cast<size_t>(m) * NG + c] = w;
-            }
-        }
-        adj_ptr.push_back(adj_ptr.back() + NG);
-        for (int c = 0; c < blk; ++c) local[base + c] = -1;
-        for (int g : ring1) local[g] = -1;
-        for (int g : ring2) local[g] = -1;
-    }
-    emax = (emax + 3) / 4 * 4;  // 16-byte aligned shared-memory rows
-    gmax = (gmax + 3) / 4 * 4;
-    const size_t smem = FusedSmem<T>::bytes(emax, gmax);
-    if (emax >= 65536 || smem > static_cast<size_t>(kFusedSmemCap)) return FVLBM_OK;  // not usable
-    S.emax = emax;
-    S.gmax = gmax;
-    S.smem = smem;
-    int rc;
-    std::vector<int> inst_blk0(inst_tile0.size());
-    for (size_t q = 0; q < inst_tile0.size(); ++q) inst_blk0[q] = inst_tile0[q] / (blk / kTile);
-    if ((rc = upload_raw(h, &S.d_inst_blk0, inst_blk0))) return rc;
-    if ((rc = upload_raw(h, &S.d_halo_ptr, halo_ptr))) return rc;
-    if (halo.empty()) halo.push_back(0);
-    if ((rc = upload_raw(h, &S.d_halo, halo))) return rc;
-    if ((rc = upload_raw(h, &S.d_r1, r1n))) return rc;
-    if ((rc = upload_raw(h, &S.d_adj_ptr, adj_ptr))) return rc;
-    if ((rc = upload_raw(h, &S.d_adj, adj))) return rc;
-    // The attribute is per function and process-wide, shared by every handle: always raise it
-    // to the library's cap so that a handle with a smaller halo never lowers another's limit.
-    const int cap = kFusedSmemCap;
-    if (blk == 256) {
-        CK(cudaFuncSetAttribute(k_fused_stage<T, 1, false, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-        CK(cudaFuncSetAttribute(k_fused_stage<T, 2, false, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-        CK(cudaFuncSetAttribute(k_fused_stage<T, 3, false, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-        CK(cudaFuncSetAttribute(k_fused_stage<T, 3, true, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-    } else {
-        CK(cudaFuncSetAttribute(k_fused_stage<T, 1, false, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-        CK(cudaFuncSetAttribute(k_fused_stage<T, 2, false, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-        CK(cudaFuncSetAttribute(k_fused_stage<T, 3, false, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-        CK(cudaFuncSetAttribute(k_fused_stage<T, 3, true, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-    }
-    S.ok = true;
-    return FVLBM_OK;
-}
+// Cells per item of the face-value kernels for a handle of np padded cells: items of 256 cells
+// where there are enough of them to fill the 152 SMs several times over, 64 below that, so that
+// a small mesh spreads over the chip.  Both sides measured, us per step, 256 against 64 cells:
+// float 10k cells 17.6 / 12.6, 40k 20.6 / 15.0, 80k (SST) 36.1 / 35.2, 200k (SST) 73 / 79, 2.6M
+// (sweep) 657 / 852; double 4k 80 / 52, 50k (SST) 259 / 250, 640k (SST) 1744 / 1969.
+int fv_item_cells(size_t np) { return np <= 90000 ? 64 : 256; }
 
-// Work items of the face-value kernel: every 256-cell block whose ring-1 + ring-2 halo and
-// ring-1 count fit its shared memory (kFvEcap, kFvGcap) is one item; a block that does not fit
-// is split into halves, and a half that does not fit into quarters.  Per item: the ring lists,
-// the adjacency words (cell-major) of item and ring-1 cells, and per face which member of each
-// direction pair leaves the cell through it -- decided once per face from the FP64 normal of
-// one side (e_alpha . n >= 0, the upwind rule of Eq. (advection)) and complemented on the
-// other side, so that both sides always agree.  The ring lists and the adjacency sit at fixed
-// strides per item (FvItems).  The set is left unusable (ok = false) if a quarter block still
-// does not fit.
-template <class T>
-int build_fv_items(fvlbm_handle *h, const std::vector<int> &nbr, const std::vector<int> &back,
-                   const std::vector<double> &sn, const std::vector<int> &inst_tile0) {
+// Work items of the face-value kernel: every block of IT cells whose rows (cells, ring-1 and
+// ring-2 halo, ghosts) and cut faces fit its shared memory (FvShape) is one item; a block that does
+// not fit is split into halves, and so on down to eighths.  Per item: the ring lists, the
+// adjacency words of its cells, the cut faces (interior faces between an item cell and a
+// ring cell: the ring cell's row, the rows of its face data, its coefficients and outgoing
+// bits) and the ghosts (boundary faces of item and ring-1 cells).  Which member of each
+// direction pair leaves the cell through a face is decided once per face from the FP64 normal
+// of one side (e_alpha . n >= 0, the upwind rule of Eq. (advection)) and complemented on the
+// other side, so that both sides always agree.  The ring lists sit at a fixed stride per item
+// (FvItems).  The set is left unusable (ok = false) if an eighth of a block still does not fit.
+template <class T, int IT>
+int build_fv_items_it(fvlbm_handle *h, const std::vector<int> &nbr, const std::vector<int> &back,
+                      const std::vector<double> &sn, const std::vector<double> &lsq,
+                      const std::vector<double> &rown, const std::vector<double> &gq, const std::vector<int> &bowner,
+                      const std::vector<int> &inst_tile0) {
+    using S = FvShape<IT>;
     const size_t np = h->np;
     // outgoing bits of every (cell, face slot)
     std::vector<unsigned char> pbits(4 * np, 0);
@@ -2388,121 +1972,200 @@ int build_fv_items(fvlbm_handle *h, const std::vector<int> &nbr, const std::vect
             }
             pbits[m * np + g] = static_cast<unsigned char>(owner ? bits : (~bits & 15u));
         }
+    // A_mk = W_k . r_m of cell g
+    auto coef = [&](size_t g, int m, int k) {
+        return lsq[(2 * k) * np + g] * rown[(2 * m) * np + g] + lsq[(2 * k + 1) * np + g] * rown[(2 * m + 1) * np + g];
+    };
     std::vector<int4> hdr;
     std::vector<int> halo, ovf, item_inst;
-    std::vector<uint4> adj;
-    std::vector<int> local(np, -1), ring1, ring2;
+    std::vector<uint4> adj(np, make_uint4(kFvNone, kFvNone, kFvNone, kFvNone));
+    std::vector<uint2> cut;
+    std::vector<int4> ghost;
+    std::vector<double> cutc;
+    // float: node positions minus centroid as the kernels read them, and the offset of face m
+    // formed from them in float
+    auto node = [&](size_t g, int m, int c) { return static_cast<float>(gq[(2 * m + c) * np + g]); };
+    auto mid = [&](size_t g, int m, int c) {
+        const int nv = nbr[3 * np + g] == kNone ? 3 : 4;
+        return 0.5f * (node(g, m, c) + node(g, m + 1 == nv ? 0 : m + 1, c));
+    };
+    std::vector<int> local(np, -1), ring;   // ring: ring-1 cells, then ring-2 cells
+    std::vector<int> grow(std::max(h->nbt, 1), -1), gface;  // ghost row of a boundary face
     int n_split = 0, n_ovf = 0;
-    bool fits_all = true;
-    // try one item of cnt cells at base (instance inst); returns false if it does not fit
-    auto try_item = [&](int base, int cnt, int inst, bool commit) -> bool {
+    // one item of cnt cells at base (instance inst); returns false, adding nothing, if it does
+    // not fit
+    auto try_item = [&](int base, int cnt, int inst) -> bool {
         for (int c = 0; c < cnt; ++c) local[base + c] = c;
-        ring1.clear();
-        ring2.clear();
-        int next = cnt;
-        for (int c = 0; c < cnt; ++c)
-            for (int m = 0; m < 4; ++m) {
-                const int v = nbr[m * np + base + c];
-                if (v >= 0 && local[v] < 0) { local[v] = next++; ring1.push_back(v); }
-            }
-        for (int g : ring1)
+        ring.clear();
+        gface.clear();
+        int ncut = 0;
+        auto ghosts_of = [&](size_t g) {
             for (int m = 0; m < 4; ++m) {
                 const int v = nbr[m * np + g];
-                if (v >= 0 && local[v] < 0) { local[v] = next++; ring2.push_back(v); }
+                if (v < 0 && v != kNone) gface.push_back(-v - 1);
             }
-        const int E = next, NG = cnt + static_cast<int>(ring1.size());
-        const bool fit = E <= kFvEcap && NG <= kFvGcap && E - cnt <= 2 * kFvHs;
-        if (fit && commit) {
-            // halo ids: kFvHs slots per item, the rest (split items only: E <= kFvEcap and
-            // cnt >= 64 leave at most 2 kFvHs) in a kFvHs-slot chunk of the overflow table
-            const int nh = E - cnt;
+        };
+        auto visit = [&](size_t g) {
+            for (int m = 0; m < 4; ++m) {
+                const int v = nbr[m * np + g];
+                if (v >= 0 && local[v] < 0) {
+                    local[v] = cnt + static_cast<int>(ring.size());
+                    ring.push_back(v);
+                }
+            }
+        };
+        for (int c = 0; c < cnt; ++c) {
+            visit(base + c);
+            ghosts_of(base + c);
+            for (int m = 0; m < 4; ++m) {
+                const int v = nbr[m * np + base + c];
+                if (v >= 0 && local[v] >= cnt) ++ncut;
+            }
+        }
+        const size_t n1 = ring.size();
+        for (size_t r = 0; r < n1; ++r) {
+            visit(ring[r]);
+            ghosts_of(ring[r]);
+        }
+        const int nh = static_cast<int>(ring.size()), ngh = static_cast<int>(gface.size());
+        const bool fit = cnt + nh + ngh <= S::ecap && nh <= 2 * S::hs && ncut <= S::ccap;
+        if (fit) {
+            for (int q = 0; q < ngh; ++q) grow[gface[q]] = cnt + nh + q;
             const size_t h0 = halo.size();
-            halo.resize(h0 + kFvHs, -1);
+            halo.resize(h0 + S::hs, -1);
             int ovf0 = -1;
-            if (nh > kFvHs) {
+            if (nh > S::hs) {
                 ++n_ovf;
                 ovf0 = static_cast<int>(ovf.size());
-                ovf.resize(ovf.size() + kFvHs, -1);
+                ovf.resize(ovf.size() + S::hs, -1);
             }
             for (int r = 0; r < nh; ++r) {
-                const int g = r < static_cast<int>(ring1.size()) ? ring1[r] : ring2[r - ring1.size()];
-                if (r < kFvHs)
-                    halo[h0 + r] = g;
+                if (r < S::hs)
+                    halo[h0 + r] = ring[r];
                 else
-                    ovf[ovf0 + r - kFvHs] = g;
+                    ovf[ovf0 + r - S::hs] = ring[r];
             }
-            hdr.push_back(make_int4(base, cnt | (static_cast<int>(ring1.size()) << 16), inst, ovf0));
-            const size_t a0 = adj.size();
-            adj.resize(a0 + kFvGcap, make_uint4(kFvNone, kFvNone, kFvNone, kFvNone));
-            for (int c = 0; c < NG; ++c) {
-                const int g = c < cnt ? base + c : ring1[c - cnt];
+            hdr.push_back(make_int4(base, cnt | (ncut << 16), inst, ovf0));
+            hdr.push_back(make_int4(nh, ngh, static_cast<int>(ghost.size()), static_cast<int>(cut.size())));
+            for (int q = 0; q < ngh; ++q) {
+                const int o = bowner[gface[q]];
+                int m = 0;
+                while (nbr[m * np + o] != -gface[q] - 1) ++m;
+                ghost.push_back(make_int4(local[o], gface[q], o, m));
+            }
+            // the staged row of face datum m of cell g (its own row where it has no such face)
+            auto row_of = [&](size_t g, int m) {
+                const int v = nbr[m * np + g];
+                return static_cast<unsigned>(v == kNone ? local[g] : (v < 0 ? grow[-v - 1] : local[v]));
+            };
+            int q = 0;
+            for (int c = 0; c < cnt; ++c) {
+                const size_t g = base + c;
                 unsigned w[4];
                 for (int m = 0; m < 4; ++m) {
                     const int v = nbr[m * np + g];
-                    if (v == kNone)
+                    if (v == kNone) {
                         w[m] = kFvNone;
-                    else if (v < 0)
-                        w[m] = kFvBnd | static_cast<unsigned>(-v - 1);
-                    else
-                        w[m] = static_cast<unsigned>(local[v]) | (static_cast<unsigned>(back[m * np + g]) << 16) |
-                               (static_cast<unsigned>(pbits[m * np + g]) << 18);
+                    } else if (v < 0) {
+                        w[m] = kFvBnd | row_of(g, m);
+                    } else {
+                        const int b = back[m * np + g];
+                        unsigned vrow;
+                        if (local[v] < cnt) {
+                            vrow = 4u * local[v] + (b ^ ((local[v] >> 1) & 3));
+                        } else {  // a cut face: the ring cell's values at its face b
+                            vrow = 4u * IT + q++;
+                            const size_t o = v;
+                            cut.push_back(make_uint2(
+                                static_cast<unsigned>(local[v]) | (row_of(o, 0) << 9) | (row_of(o, 1) << 18),
+                                row_of(o, 2) | (row_of(o, 3) << 9) | (static_cast<unsigned>(pbits[b * np + o]) << 18)));
+                            if constexpr (sizeof(T) == 4) {
+                                for (int k = 0; k < 8; ++k)
+                                    cutc.push_back(nbr[k / 2 * np + o] == kNone ? 0.0 : lsq[k * np + o]);
+                                for (int k = 0; k < 2; ++k) cutc.push_back(mid(o, b, k));
+                                cutc.resize(cutc.size() + 2, 0.0);
+                            } else {
+                                for (int k = 0; k < 4; ++k)
+                                    cutc.push_back(nbr[k * np + o] == kNone ? 0.0 : coef(o, b, k));
+                            }
+                        }
+                        w[m] = static_cast<unsigned>(local[v]) | (vrow << 9) |
+                               (static_cast<unsigned>(pbits[m * np + g]) << 20);
+                    }
                 }
-                adj[a0 + c] = make_uint4(w[0], w[1], w[2], w[3]);
+                adj[g] = make_uint4(w[0], w[1], w[2], w[3]);
             }
+            item_inst.push_back(inst);
         }
         for (int c = 0; c < cnt; ++c) local[base + c] = -1;
-        for (int g : ring1) local[g] = -1;
-        for (int g : ring2) local[g] = -1;
+        for (int g : ring) local[g] = -1;
         return fit;
     };
     std::vector<int> tile_inst_of(np / kTile);
     for (size_t q = 0; q + 1 < inst_tile0.size(); ++q)
         for (int tt = inst_tile0[q]; tt < inst_tile0[q + 1]; ++tt) tile_inst_of[tt] = static_cast<int>(q);
-    constexpr int IT = kFvThreads, HALF = IT / 2, QUART = IT / 4;
-    const int nblk = static_cast<int>(np / IT);
-    for (int b = 0; b < nblk && fits_all; ++b) {
-        const int base = b * IT;
-        int inst = tile_inst_of[base / kTile];
-        if (try_item(base, IT, inst, true)) {
-            item_inst.push_back(inst);
-            continue;
-        }
-        ++n_split;
-        for (int half = 0; half < 2 && fits_all; ++half) {
-            const int hb = base + HALF * half;
-            if (try_item(hb, HALF, inst, true)) {
-                item_inst.push_back(inst);
-                continue;
-            }
-            for (int qq = 0; qq < 2 && fits_all; ++qq) {
-                if (try_item(hb + QUART * qq, QUART, inst, true))
-                    item_inst.push_back(inst);
-                else
-                    fits_all = false;
-            }
-        }
+    std::vector<std::pair<int, int>> todo;  // (base, cells), the next one last
+    for (size_t b = np / IT; b-- > 0;) todo.push_back({static_cast<int>(b * IT), IT});
+    while (!todo.empty()) {
+        const auto [base, cnt] = todo.back();
+        todo.pop_back();
+        if (try_item(base, cnt, tile_inst_of[base / kTile])) continue;
+        if (cnt == IT) ++n_split;
+        if (cnt <= IT / 8 || cnt <= 8) return FVLBM_OK;  // not usable
+        todo.push_back({base + cnt / 2, cnt / 2});
+        todo.push_back({base, cnt / 2});
     }
-    if (!fits_all || hdr.empty() || ovf.size() >= (1u << 31)) return FVLBM_OK;  // not usable
-    const int nitem = static_cast<int>(hdr.size());
+    const int nitem = static_cast<int>(item_inst.size());
+    if (nitem == 0 || ovf.size() >= (1u << 31) || cut.size() >= (1u << 29)) return FVLBM_OK;
     std::vector<int> inst_item0(h->ninst + 1, nitem);
     for (int k = nitem - 1; k >= 0; --k) inst_item0[item_inst[k]] = k;
     for (int q = h->ninst - 1; q >= 0; --q)  // instances without items (none in practice)
         if (inst_item0[q] > inst_item0[q + 1]) inst_item0[q] = inst_item0[q + 1];
+    std::vector<double> geo(kFvGeo<T> * np, 0.0);
+    for (size_t g = 0; g < np; ++g) {
+        auto at = [&](int v) -> double & { return geo[fv_geo_at<T>(g, v)]; };
+        if constexpr (sizeof(T) == 4) {
+            for (int c = 0; c < 8; ++c) {
+                at(c) = gq[c * np + g];
+                at(8 + c) = lsq[c * np + g];
+            }
+            continue;
+        }
+        const bool tri = nbr[3 * np + g] == kNone;
+        const int nv = tri ? 3 : 4;
+        for (int m = 0; m < nv; ++m)
+            for (int k = 0; k < nv; ++k)
+                if (nbr[m * np + g] != kNone && nbr[k * np + g] != kNone) at(4 * m + k) = coef(g, m, k);
+        static const int tri_at[6] = {3, 7, 11, 12, 13, 14};
+        for (int c = 0; c < 2 * nv; ++c) at(tri ? tri_at[c] : 16 + c) = sn[c * np + g];
+    }
     if (ovf.empty()) ovf.push_back(-1);
+    if (cut.empty()) {
+        cut.push_back(make_uint2(0, 0));
+        cutc.assign(kFvCut<T>, 0.0);
+    }
+    if (ghost.empty()) ghost.push_back(make_int4(0, 0, 0, 0));
     int rc;
     if ((rc = upload_raw(h, &h->fv.d_hdr, hdr))) return rc;
     if ((rc = upload_raw(h, &h->fv.d_halo, halo))) return rc;
     if ((rc = upload_raw(h, &h->fv.d_ovf, ovf))) return rc;
     if ((rc = upload_raw(h, &h->fv.d_adj, adj))) return rc;
+    if ((rc = upload_raw(h, &h->fv.d_cut, cut))) return rc;
+    if ((rc = upload_raw(h, &h->fv.d_ghost, ghost))) return rc;
     if ((rc = upload_raw(h, &h->fv.d_inst_item0, inst_item0))) return rc;
-    CK(cudaFuncSetAttribute(k_fused_fv<T, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            static_cast<int>(FvSmem<T>::bytes)));
-    CK(cudaFuncSetAttribute(k_fused_fv<T, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            static_cast<int>(FvSmem<T>::bytes)));
-    CK(cudaFuncSetAttribute(k_fused_fv<T, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            static_cast<int>(FvSmem<T>::bytes)));
-    CK(cudaFuncSetAttribute(k_fused_fv<T, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            static_cast<int>(FvSmem<T>::bytes)));
+    if ((rc = upload_as<T>(h, &h->fv.geo, geo))) return rc;
+    if ((rc = upload_as<T>(h, &h->fv.cutc, cutc))) return rc;
+    if (nitem > h->ntiles) {  // stage 3's partial sums: one row per item
+        h->d_partial = nullptr;
+        if ((rc = dalloc(h, reinterpret_cast<void **>(&h->d_partial), 4 * sizeof(double) * nitem))) return rc;
+    }
+    // (the attribute is per function and process-wide; every handle sets the same value)
+    constexpr int smem = static_cast<int>(FvSmem<T, IT>::bytes);
+    CK(cudaFuncSetAttribute(k_fused_fv<T, 1, false, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CK(cudaFuncSetAttribute(k_fused_fv<T, 2, false, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CK(cudaFuncSetAttribute(k_fused_fv<T, 3, false, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CK(cudaFuncSetAttribute(k_fused_fv<T, 3, true, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    h->fv.it = IT;
     h->fv.nitem = nitem;
     h->fv.n_split = n_split;
     h->fv.n_ovf = n_ovf;
@@ -2510,13 +2173,13 @@ int build_fv_items(fvlbm_handle *h, const std::vector<int> &nbr, const std::vect
     return FVLBM_OK;
 }
 
-// f^(1) of the coming step from the current f^n and tau, for every cell (after create and
-// set_f); the fused stage-1 kernel reads it.
 template <class T>
-void relax_all(fvlbm_handle *h) {
-    k_stage1<T><<<h->ntiles, kTile, 0, h->stream>>>(static_cast<const T *>(h->fn),
-                                                   static_cast<T *>(h->frel),
-                                                   static_cast<const T *>(h->tau), geo_of<T>(h));
+int build_fv_items(fvlbm_handle *h, const std::vector<int> &nbr, const std::vector<int> &back,
+                   const std::vector<double> &sn, const std::vector<double> &lsq, const std::vector<double> &rown,
+                   const std::vector<double> &gq, const std::vector<int> &bowner, const std::vector<int> &inst_tile0) {
+    return fv_dispatch(fv_item_cells(h->np), [&](auto it) {
+        return build_fv_items_it<T, decltype(it)::value>(h, nbr, back, sn, lsq, rown, gq, bowner, inst_tile0);
+    });
 }
 
 template <class T>
@@ -2525,7 +2188,7 @@ int allocate_state(fvlbm_handle *h, const std::vector<const Prepared *> &P,
     const size_t np = h->np;
     int rc;
     const size_t ts = sizeof(T);
-    for (void **p : {&h->fn, &h->s0, &h->s1, &h->bacc, &h->cacc, &h->frel})
+    for (void **p : {&h->fn, &h->s0, &h->s1, &h->bacc, &h->cacc})
         if ((rc = dalloc(h, p, kQ * np * ts))) return rc;
     if ((rc = dalloc(h, &h->grad, 2 * kQ * np * ts))) return rc;
     if ((rc = dalloc(h, &h->tau, np * ts))) return rc;
@@ -2653,23 +2316,8 @@ int allocate_state(fvlbm_handle *h, const std::vector<const Prepared *> &P,
     }
     if constexpr (kHasFused<T>) {
         if (h->fused) {
-            if ((rc = build_halos<T>(h, h->hs[0], 256, nbr, back, nface, inst_tile0))) return rc;
-            if ((rc = build_halos<T>(h, h->hs[1], 128, nbr, back, nface, inst_tile0))) return rc;
-            if ((rc = build_fv_items<T>(h, nbr, back, sn, inst_tile0))) return rc;
-            if (h->fv.ok) {  // cell-major geometry of the face-value kernels (64 B per cell)
-                std::vector<double> g16(16 * np);
-                for (size_t k = 0; k < np; ++k)
-                    for (int c = 0; c < 8; ++c) {
-                        g16[16 * k + c] = gq[c * np + k];
-                        g16[16 * k + 8 + c] = lsq[c * np + k];
-                    }
-                if ((rc = upload_as<T>(h, &h->geo16, g16))) return rc;
-            }
-            h->config = h->hs[0].ok ? 0 : (h->hs[1].ok ? 1 : 2);
-            if (h->fv.ok && (h->kernel_path == 2 || h->config == 2)) h->config = 3;
-            // FP32: only the forms whose least-squares weights come from the host in FP64 (the
-            // 256- and 128-cell forms invert M on chip, in FP32 a few digits on y+ ~ 1 cells)
-            if (h->precision == FVLBM_FP32_DEV) h->config = h->fv.ok ? 3 : 2;
+            if ((rc = build_fv_items<T>(h, nbr, back, sn, lsq, rown, gq, bowner, inst_tile0))) return rc;
+            if (h->fv.ok) h->config = 3;
             if (h->config == 2) h->fused = false;
         }
     }
@@ -2695,8 +2343,6 @@ int allocate_state(fvlbm_handle *h, const std::vector<const Prepared *> &P,
     Geo<T> G = geo_of<T>(h);
     k_init_state<T><<<h->ntiles, kTile, 0, h->stream>>>(static_cast<T *>(h->fn), static_cast<T *>(h->mac),
                                                        d_init, d_init + np, d_init + 2 * np, G);
-    CK(cudaGetLastError());
-    relax_all<T>(h);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(h->stream));
     return FVLBM_OK;
@@ -2894,12 +2540,8 @@ size_t io_cells(const fvlbm_handle *h, int instance) {
     return instance == -1 ? static_cast<size_t>(h->total_nc) : static_cast<size_t>(h->inst[instance].nc);
 }
 
-// f^(1) of the coming step is kept only for the 256- and 128-cell fused forms (configurations
-// 0, 1); a switch to them (the autotuner) or a load relaxes it again from f^n.
-void *frel_target(const fvlbm_handle *h) { return h->config == 0 || h->config == 1 ? h->frel : nullptr; }
-
 // The state from a DEVICE buffer (input cell order, [cells][9]; IN = double: absolute f,
-// float: FP32 deviations) into f^n, the macros and f^(1) of the coming step; handle's stream.
+// float: FP32 deviations) into f^n and the macros; handle's stream.
 template <class IN>
 void scatter_state_dev(fvlbm_handle *h, int instance, const IN *src) {
     // the internal cells of the instance (all instances: every cell), padding included
@@ -2909,8 +2551,7 @@ void scatter_state_dev(fvlbm_handle *h, int instance, const IN *src) {
     dispatch(h->precision, [&](auto z_) {
         using T = decltype(z_);
         k_scatter_state<T, IN><<<(n + 255) / 256, 256, 0, h->stream>>>(
-            static_cast<T *>(h->fn), static_cast<T *>(h->mac), static_cast<T *>(frel_target(h)),
-            static_cast<const T *>(h->tau), h->d_all_inv, i0, n, po, geo_of<T>(h), src);
+            static_cast<T *>(h->fn), static_cast<T *>(h->mac), h->d_all_inv, i0, n, po, geo_of<T>(h), src);
     });
 }
 
@@ -3273,10 +2914,9 @@ int fvlbm_set_cells(fvlbm_handle *h, int instance, int n, const int *cells, cons
     dispatch(h->precision, [&](auto z_) {
         using T = decltype(z_);
         const int c = h->turb;
-        if (f)  // f^n, the macros and f^(1) of the coming step, as fvlbm_set_f
+        if (f)  // f^n and the macros, as fvlbm_set_f
             k_scatter_list<T, double><<<(n + 255) / 256, 256, 0, h->stream>>>(
-                static_cast<T *>(h->fn), static_cast<T *>(h->mac), static_cast<T *>(frel_target(h)),
-                static_cast<const T *>(h->tau), d_map, n, geo_of<T>(h), d_f);
+                static_cast<T *>(h->fn), static_cast<T *>(h->mac), d_map, n, geo_of<T>(h), d_f);
         if (turb)
             k_set_turb<T><<<(n + 255) / 256, 256, 0, h->stream>>>(static_cast<T *>(h->kk[c]),
                                                                  static_cast<T *>(h->ww[c]),
@@ -3357,8 +2997,7 @@ int fvlbm_unpack_cells_dev(fvlbm_handle *h, int list_id, const double *vals) {
         using T = decltype(z_);
         const int c = h->turb;
         k_unpack_cells<T><<<(L.n + 255) / 256, 256, 0, h->stream>>>(
-            static_cast<T *>(h->fn), static_cast<T *>(h->mac), static_cast<T *>(frel_target(h)),
-            static_cast<const T *>(h->tau), static_cast<T *>(h->kk[c]), static_cast<T *>(h->ww[c]),
+            static_cast<T *>(h->fn), static_cast<T *>(h->mac), static_cast<T *>(h->kk[c]), static_cast<T *>(h->ww[c]),
             static_cast<T *>(h->nut[c]), L.d_map, L.n, geo_of<T>(h), vals);
     });
     CK(cudaGetLastError());
@@ -3729,7 +3368,7 @@ int fvlbm_autotune(fvlbm_handle *h, int trial_steps, int *chosen, double *ms_per
     CK(cudaSetDevice(h->device));
     if (ms_per_step)
         for (int c = 0; c < 4; ++c) ms_per_step[c] = -1.0;
-    if (h->scheme != 0 || (!h->hs[0].ok && !h->hs[1].ok && !h->fv.ok)) {  // nothing to choose
+    if (h->scheme != 0 || !h->fv.ok) {  // nothing to choose
         if (chosen) *chosen = h->config;
         return FVLBM_OK;
     }
@@ -3758,9 +3397,7 @@ int fvlbm_autotune(fvlbm_handle *h, int trial_steps, int *chosen, double *ms_per
     double best = 1e300;
     int best_c = h->config;
     cudaError_t err = cudaSuccess;
-    for (int c = 0; c < 4 && err == cudaSuccess; ++c) {
-        if (c < 2 && (!h->hs[c].ok || h->precision == FVLBM_FP32_DEV)) continue;  // see create
-        if (c == 3 && !h->fv.ok) continue;
+    for (int c = 2; c < 4 && err == cudaSuccess; ++c) {  // two-pass, face-value
         h->config = c;
         for (int k = 0; k < 2; ++k) enqueue(h, false);  // warm-up
         cudaEventRecord(e0, h->stream);
@@ -3784,11 +3421,6 @@ int fvlbm_autotune(fvlbm_handle *h, int trial_steps, int *chosen, double *ms_per
     cudaFree(snap);
     h->config = best_c;
     h->steps = steps0;
-    // The two-pass kernels do not keep f^(1) of the coming step: if they ran before this call,
-    // the restored snapshot holds a stale one.  Relax it again from f^n for the fused stages
-    // (bitwise what stage 3 writes for laminar instances; SST instances redo it every step).
-    if (best_c != 2 && err == cudaSuccess)
-        dispatch(h->precision, [&](auto z_) { relax_all<decltype(z_)>(h); });
     for (int k = 0; k < 3; ++k)  // captured graphs bake the old configuration
         if (h->graph[k]) {
             cudaGraphExecDestroy(h->graph[k]);
@@ -3812,7 +3444,7 @@ int fvlbm_save_state(fvlbm_handle *h, void *buf, long long bytes) {
     CK(cudaSetDevice(h->device));
     StateHeader hd{};
     std::memcpy(hd.magic, "FVLBMST", 8);
-    hd.version = 1;
+    hd.version = 2;
     hd.precision = h->precision;
     hd.np = h->np;
     hd.ninst = h->ninst;
@@ -3834,9 +3466,13 @@ int fvlbm_load_state(fvlbm_handle *h, const void *buf, long long bytes) {
     if (!h || !buf || bytes < static_cast<long long>(sizeof(StateHeader))) return FVLBM_ERR_BAD_PARAM;
     StateHeader hd;
     std::memcpy(&hd, buf, sizeof(hd));
-    if (std::memcmp(hd.magic, "FVLBMST", 8) != 0 || hd.version != 1 || hd.precision != h->precision ||
+    // version 1 blobs also carry f^(1) of the coming step after f^n, which no kernel reads now
+    size_t skip = 0;
+    if (hd.version == 1)
+        dispatch(h->precision, [&](auto z_) { skip = kQ * static_cast<size_t>(h->np) * sizeof(z_); });
+    if (std::memcmp(hd.magic, "FVLBMST", 8) != 0 || (hd.version != 1 && hd.version != 2) || hd.precision != h->precision ||
         hd.np != h->np || hd.ninst != h->ninst || hd.order_hash != h->order_hash ||
-        hd.payload != state_bytes(h) || bytes < static_cast<long long>(sizeof(hd) + hd.payload)) {
+        hd.payload != state_bytes(h) + skip || bytes < static_cast<long long>(sizeof(hd) + hd.payload)) {
         fprintf(stderr, "fvlbm_load_state: the blob does not match this handle\n");
         return FVLBM_ERR_BAD_PARAM;
     }
@@ -3845,13 +3481,8 @@ int fvlbm_load_state(fvlbm_handle *h, const void *buf, long long bytes) {
     for (auto &e : state_regions(h)) {
         CK(cudaMemcpyAsync(e.first, src, e.second, cudaMemcpyHostToDevice, h->stream));
         src += e.second;
+        if (e.first == h->fn) src += skip;
     }
-    // a blob saved under the face-value configuration holds no f^(1) of the coming step: the
-    // other fused configurations relax it from f^n again (bitwise what they would have stored)
-    if (h->config == 0 || h->config == 1)
-        dispatch(h->precision, [&](auto z_) {
-            if constexpr (kHasFused<decltype(z_)>) relax_all<decltype(z_)>(h);
-        });
     CK(cudaStreamSynchronize(h->stream));
     h->steps = hd.steps;
     h->turb = hd.turb;
