@@ -612,9 +612,7 @@ __device__ __forceinline__ void fv_flux(int t, const T *sn, const unsigned *w, c
 // writes f^{n+1}; geo: the geometry rows, cutc: the cut faces' coefficients.
 template <class T, int STAGE, bool STATS, int IT>
 __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ? 4 : 1) : (IT == 256 ? 2 : 1))
-    k_fused_fv(const T *__restrict__ fin, T *__restrict__ fs_out, T *__restrict__ fn,
-               T *__restrict__ Bacc, T *__restrict__ Cacc, const T *__restrict__ tau,
-               T *__restrict__ mac, double *__restrict__ partial, Geo<T> G, FvItems W,
+    k_fused_fv(const T *fin, T *__restrict__ fs_out, T *__restrict__ fn, T *Bacc, T *Cacc, const T *tau, T *mac, double *__restrict__ partial, Geo<T> G, FvItems W,
                const T *__restrict__ geo, const T *__restrict__ cutc, const T *__restrict__ bnrm) {
     using PV = FvPair<T>;
     using V = typename PV::V;
@@ -628,6 +626,7 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
     T *sacc = reinterpret_cast<T *>(smem_raw + L::sacc);
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem_raw + L::bar);
 
+    dep_launch();
     const int t = threadIdx.x;
     const int it = static_cast<int>(blockIdx.x);
     // halo slot t of the fixed-stride table and the header, loaded together (kept in L2)
@@ -644,13 +643,39 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
     const int i = base + t;
     const T *fa0 = fin + 8 * np;  // stages 2, 3: f_0 of every cell after the cell-major rows
 
-    // 1. staging, issued before any wait
+    // 1. staging, issued before any wait: first what is fixed at create, beside the last blocks of
+    // the kernel before; then the copies.
     // The bulk copies are shared out over the lanes 0 of the warps, so that no warp issues
     // more than a few of them: each such lane arrives on the mbarrier (count: the warps) with the
     // bytes of its own copies, then issues them.
     constexpr int kWarps = NT / 32;
     if (t == 0) mbar_init(bar, kWarps);
     __syncthreads();
+    static_assert(sizeof(InstParam) % 16 == 0 && L::ip % 16 == 0, "16-byte copies of the parameters");
+    if (t < static_cast<int>(sizeof(InstParam) / 16))  // (device arrays of InstParam: 16-byte aligned rows)
+        cp_async<16>(smem_raw + L::ip + 16 * t, reinterpret_cast<const unsigned char *>(Pp) + 16 * t);
+    // the item cell's adjacency and coefficients, the thread's first cut face and ghost
+    unsigned w[4] = {kFvNone, kFvNone, kFvNone, kFvNone};
+    T A[16];
+    if (mine) {
+        const uint4 w4 = W.adj[i];
+        w[0] = w4.x; w[1] = w4.y; w[2] = w4.z; w[3] = w4.w;
+#pragma unroll
+        for (int k = 0; k < 16; k += 4) fv_load_geo4(geo, i, k, A + k);
+    }
+    // cut units: (cut face, half), over the threads that hold no cell where there are any
+    constexpr int CB = NT > IT ? IT : 0, CS = NT - CB;
+    const int cu = t - CB;
+    const bool cut0 = cu >= 0 && cu < 2 * ncut;
+    uint2 cr = make_uint2(0, 0);
+    T ca[kFvCut<T>];
+    auto load_cut = [&](int c) {
+        cr = W.cut[hx.w + c];
+#pragma unroll
+        for (int k = 0; k < kFvCut<T>; k += 4) fv_load4(cutc + kFvCut<T> * static_cast<size_t>(hx.w + c) + k, ca + k);
+    };
+    if (cut0) load_cut(cu >> 1);
+    dep_wait();  // f, the accumulators and tau of the kernels before
     if ((t & 31) == 0) {
         const unsigned row = static_cast<unsigned>(cnt * sizeof(T));
         // copies: (stages 2, 3) the item's f rows and f_0, then the accumulator rows (stage 1:
@@ -703,30 +728,6 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
             cp_async<sizeof(T)>(sf0 + e, fa0 + gid);
         }
     }
-    static_assert(sizeof(InstParam) % 16 == 0 && L::ip % 16 == 0, "16-byte copies of the parameters");
-    if (t < static_cast<int>(sizeof(InstParam) / 16))  // (device arrays of InstParam: 16-byte aligned rows)
-        cp_async<16>(smem_raw + L::ip + 16 * t, reinterpret_cast<const unsigned char *>(Pp) + 16 * t);
-    // the item cell's adjacency and coefficients, the thread's first cut face and ghost
-    unsigned w[4] = {kFvNone, kFvNone, kFvNone, kFvNone};
-    T A[16];
-    if (mine) {
-        const uint4 w4 = W.adj[i];
-        w[0] = w4.x; w[1] = w4.y; w[2] = w4.z; w[3] = w4.w;
-#pragma unroll
-        for (int k = 0; k < 16; k += 4) fv_load_geo4(geo, i, k, A + k);
-    }
-    // cut units: (cut face, half), over the threads that hold no cell where there are any
-    constexpr int CB = NT > IT ? IT : 0, CS = NT - CB;
-    const int cu = t - CB;
-    const bool cut0 = cu >= 0 && cu < 2 * ncut;
-    uint2 cr = make_uint2(0, 0);
-    T ca[kFvCut<T>];
-    auto load_cut = [&](int c) {
-        cr = W.cut[hx.w + c];
-#pragma unroll
-        for (int k = 0; k < kFvCut<T>; k += 4) fv_load4(cutc + kFvCut<T> * static_cast<size_t>(hx.w + c) + k, ca + k);
-    };
-    if (cut0) load_cut(cu >> 1);
     cp_async_wait_all();
     // stage 1: each thread relaxes the halo cells it staged (its own copies have landed)
     if (STAGE == 1) {

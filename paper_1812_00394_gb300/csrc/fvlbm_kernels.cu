@@ -607,13 +607,26 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned by
 }
 template <int BYTES>
 __device__ __forceinline__ void cp_async(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst)), "l"(src),
-                 "n"(BYTES)
-                 : "memory");
+    if constexpr (BYTES == 16)  // (.ca is the only form below 16 bytes)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst)), "l"(src), "n"(BYTES)
+                     : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
+
+// Programmatic dependent launch of a step's kernels: a kernel lets its successor start as soon as
+// its own blocks have all started (dep_launch), and the successor reads nothing that a kernel
+// writes before dep_wait, which returns when every earlier kernel has finished and its stores are
+// visible.  Until then it may read the tables and geometry fixed at create, so its launch, its
+// block start-up and those loads run beside the predecessor's last blocks.  (A kernel finishes
+// only after its own dep_wait, so a chain of early starts never overtakes a kernel two back.)
+// What a kernel writes is read through pointers that are not const __restrict__: such loads
+// may be taken for loop-invariant and moved above dep_wait.
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Loads of small tables that every launch reads once per item (the face-value items' headers
 // and halo ids), marked evict-last in L2 so that the streamed state does not push them out
@@ -908,7 +921,7 @@ __device__ __forceinline__ void sst_store_rec(T *__restrict__ rec8, T *__restric
     }
 }
 template <class T>
-__device__ __forceinline__ void sst_load_rec(const T *__restrict__ rec8, const T *__restrict__ rec2, int i, T *v8,
+__device__ __forceinline__ void sst_load_rec(const T *rec8, const T *rec2, int i, T *v8,
                                              T &f1, T &nut) {
     const T *r = rec8 + 8 * static_cast<size_t>(i);
     if constexpr (std::is_same<T, float>::value) {
@@ -931,16 +944,15 @@ __device__ __forceinline__ void sst_load_rec(const T *__restrict__ rec8, const T
 // its own cell at once, without waiting for the instance parameters first.
 template <class T, bool COMPACT>
 __global__ void __launch_bounds__(kTile)
-    k_sst_grad(const T *__restrict__ mac, const T *__restrict__ kk, const T *__restrict__ ww,
-               T *__restrict__ grads, T *__restrict__ f1out, Geo<T> G, CompactGeo<T> CG,
-               const T *__restrict__ nut, T *__restrict__ rec8, T *__restrict__ rec2, bool inv_only,
+    k_sst_grad(const T *mac, const T *kk, const T *ww, T *__restrict__ grads, T *__restrict__ f1out, Geo<T> G,
+               CompactGeo<T> CG, const T *nut, T *__restrict__ rec8, T *__restrict__ rec2, bool inv_only,
                int tile0) {
+    dep_launch();
     const int tile = tile0 + static_cast<int>(blockIdx.x);
     const int i = tile * kTile + threadIdx.x;
     const size_t np = G.np;
     const InstParam P = G.ip[G.tile_inst[tile]];
     const T nu = ipv<T>(P.nu, P.nu_f);
-    const T own[4] = {mac[np + i], mac[2 * np + i], kk[i], ww[i]};
     const T di = G.wdist[i];
     bool has[4];
     int nbs[4];
@@ -977,6 +989,8 @@ __global__ void __launch_bounds__(kTile)
             R[2 * m + 1] = G.rown[(2 * m + 1) * np + i];
         }
     }
+    dep_wait();
+    const T own[4] = {mac[np + i], mac[2 * np + i], kk[i], ww[i]};
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
         const int nb = nbs[m];
@@ -1017,43 +1031,17 @@ __global__ void __launch_bounds__(kTile)
 // the default reading.
 template <class T, bool COMPACT, bool NONORTH>
 __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
-    k_sst_update(const T *__restrict__ mac, const T *__restrict__ kk, const T *__restrict__ ww,
-                 const T *__restrict__ nut, const T *__restrict__ grads,
-                 const T *__restrict__ f1a, T *__restrict__ k_out, T *__restrict__ w_out,
-                 T *__restrict__ nut_out, T *__restrict__ tau, Geo<T> G,
-                 CompactGeo<T> CG,
-                 const T *__restrict__ rec8, const T *__restrict__ rec2, int tile0) {
+    k_sst_update(const T *mac, const T *kk, const T *ww, const T *nut, const T *grads, const T *f1a,
+                 T *__restrict__ k_out, T *__restrict__ w_out, T *__restrict__ nut_out, T *__restrict__ tau,
+                 Geo<T> G, CompactGeo<T> CG, const T *rec8, const T *rec2, int tile0) {
+    dep_launch();
     const int tile = tile0 + static_cast<int>(blockIdx.x);
     const int i = tile * kTile + threadIdx.x;
     const size_t np = G.np;
     const InstParam P = G.ip[G.tile_inst[tile]];
     const T nu = ipv<T>(P.nu, P.nu_f);
     const bool packed = COMPACT && rec8 != nullptr;
-    T ui, vi, ki, wi, nti, f1i;
-    T g[8], lgi[4];
-    if (packed) {
-        T v8[8];
-        sst_load_rec(rec8, rec2, i, v8, f1i, nti);
-        ui = v8[0]; vi = v8[1]; ki = v8[2]; wi = v8[3];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) lgi[c] = v8[4 + c];
-    } else {
-        ui = mac[np + i]; vi = mac[2 * np + i]; ki = kk[i]; wi = ww[i]; nti = nut[i];
-        f1i = f1a[i];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) lgi[c] = grads[(8 + c) * np + i];
-    }
     const T di = G.wdist[i];
-    T SS, dv, kw;
-    if (packed && !NONORTH) {  // the grad kernel stored the invariants alone
-        SS = grads[i];
-        dv = grads[np + i];
-        kw = grads[2 * np + i];
-    } else {
-#pragma unroll
-        for (int c = 0; c < 8; ++c) g[c] = grads[c * np + i];
-        sst_invariants(g, SS, dv, kw);
-    }
     SstFace<T> F[4];
     int nbs[4];
     bool has[4];
@@ -1075,6 +1063,31 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
             RN[2 * m] = G.rnbr[(2 * m) * np + i]; RN[2 * m + 1] = G.rnbr[(2 * m + 1) * np + i];
             DI[m] = G.dinv[m * np + i];
         }
+    }
+    dep_wait();
+    T ui, vi, ki, wi, nti, f1i;
+    T g[8], lgi[4];
+    if (packed) {
+        T v8[8];
+        sst_load_rec(rec8, rec2, i, v8, f1i, nti);
+        ui = v8[0]; vi = v8[1]; ki = v8[2]; wi = v8[3];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) lgi[c] = v8[4 + c];
+    } else {
+        ui = mac[np + i]; vi = mac[2 * np + i]; ki = kk[i]; wi = ww[i]; nti = nut[i];
+        f1i = f1a[i];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) lgi[c] = grads[(8 + c) * np + i];
+    }
+    T SS, dv, kw;
+    if (packed && !NONORTH) {  // the grad kernel stored the invariants alone
+        SS = grads[i];
+        dv = grads[np + i];
+        kw = grads[2 * np + i];
+    } else {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) g[c] = grads[c * np + i];
+        sst_invariants(g, SS, dv, kw);
     }
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
@@ -1670,6 +1683,23 @@ void launch(fvlbm_handle *h, int id, const char *name, F &&fn) {
     nvtxRangePop();
 }
 
+// A kernel of the step with programmatic dependent launch (see dep_wait); only kernels that call
+// dep_wait before they touch what other kernels write are launched this way.
+template <class... P, class... A>
+void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // NVTX range for the lifetime of a scope (entry points with several returns).
 struct NvtxScope {
     explicit NvtxScope(const char *name) { nvtxRangePushA(name); }
@@ -1698,16 +1728,16 @@ void fv_stages(fvlbm_handle *h, bool stats) {
     const dim3 fg(static_cast<unsigned>(F.nitem)), fb(FvShape<IT>::nt);
     const size_t sm = FvSmem<T, IT>::bytes;
     launch(h, K_FUSED1, "fused_stage1", [&] {
-        k_fused_fv<T, 1, false, IT><<<fg, fb, sm, s>>>(fn, s1, fn, B, C, tau, mac, nullptr, G, W, geo, cc, bn);
+        launch_dep(k_fused_fv<T, 1, false, IT>, fg, fb, sm, s, fn, s1, fn, B, C, tau, mac, nullptr, G, W, geo, cc, bn);
     });
     launch(h, K_FUSED2, "fused_stage2", [&] {
-        k_fused_fv<T, 2, false, IT><<<fg, fb, sm, s>>>(s1, s0, fn, B, C, tau, mac, nullptr, G, W, geo, cc, bn);
+        launch_dep(k_fused_fv<T, 2, false, IT>, fg, fb, sm, s, s1, s0, fn, B, C, tau, mac, nullptr, G, W, geo, cc, bn);
     });
     launch(h, K_FUSED3, "fused_stage3", [&] {
         if (stats)
-            k_fused_fv<T, 3, true, IT><<<fg, fb, sm, s>>>(s0, s1, fn, B, C, tau, mac, h->d_partial, G, W, geo, cc, bn);
+            launch_dep(k_fused_fv<T, 3, true, IT>, fg, fb, sm, s, s0, s1, fn, B, C, tau, mac, h->d_partial, G, W, geo, cc, bn);
         else
-            k_fused_fv<T, 3, false, IT><<<fg, fb, sm, s>>>(s0, s1, fn, B, C, tau, mac, nullptr, G, W, geo, cc, bn);
+            launch_dep(k_fused_fv<T, 3, false, IT>, fg, fb, sm, s, s0, s1, fn, B, C, tau, mac, nullptr, G, W, geo, cc, bn);
     });
 }
 
@@ -1789,18 +1819,18 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
                 T *r8 = static_cast<T *>(h->sst_rec8), *r2 = static_cast<T *>(h->sst_rec2);
                 launch(h, K_SST_GRAD, "sst_grad", [&] {
                     for_sst_runs(h, [&](dim3 sg_grid, int t0) {
-                        k_sst_grad<T, true><<<sg_grid, block, 0, s>>>(mac, kc, wc, sg, f1, G, CG, nc, r8, r2,
+                        launch_dep(k_sst_grad<T, true>, sg_grid, block, 0, s, mac, kc, wc, sg, f1, G, CG, nc, r8, r2,
                                                                       !h->nonorth, t0);
                     });
                 });
                 launch(h, K_SST_UPDATE, "sst_update", [&] {
                     for_sst_runs(h, [&](dim3 sg_grid, int t0) {
                         if (h->nonorth)
-                            k_sst_update<T, true, true><<<sg_grid, block, 0, s>>>(
-                                mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
+                            launch_dep(
+                                k_sst_update<T, true, true>, sg_grid, block, 0, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
                         else
-                            k_sst_update<T, true, false><<<sg_grid, block, 0, s>>>(
-                                mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
+                            launch_dep(
+                                k_sst_update<T, true, false>, sg_grid, block, 0, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
                     });
                 });
             }
