@@ -22,6 +22,10 @@
 // three or four): each such "cut" face is a record of its own -- five row indices, the
 // coefficients, four outgoing bits -- and the ring cell's remaining faces are never formed.
 //
+// The accumulators B and C are kept in tiles of IT cells, [tile][alpha][IT] (they live from stage
+// 1 to stage 3 only), so that an item's rows are one copy and the rows a thread writes are
+// at fixed offsets.
+//
 // Two forms of the face value.  Float: the least-squares gradient, then f_c + grad f . r_m for
 // each face.  Double: a face value is linear in the differences to the cell's face data,
 // grad f . r_m = sum_k (W_k . r_m) (f_k - f_c), so the host stores A_mk = W_k . r_m and the kernel
@@ -74,12 +78,20 @@ struct FvShape<64> {
     static constexpr int nt = 128, ecap = 224, hs = 128, ccap = 160;
 };
 
-// Adjacency word (4 per cell): kFvNone: no face; else bits 0-8 the staged row of the face
-// datum (neighbour or ghost), bit 31 set for a boundary face (a ghost row); for a neighbour also
-// bits 9-19 the value row that holds its outgoing values at this face and bits 20-23 the
-// outgoing bits (bit 20 + p set when the first member of pair p leaves this cell here).
-constexpr unsigned kFvNone = 0xFFFFFFFFu;
-constexpr unsigned kFvBnd = 0x80000000u;
+// Staged rows and value rows are named by the address of their first 16 bytes (float; doubles:
+// twice that), so that a gather takes one mask: a row address is the byte offset of half 0 of the
+// row within sf (half 1 is at that offset with bit 4 flipped), see fv_row_addr.
+// Adjacency word (4 per cell): bits 4-13 the row address of the face datum (neighbour, ghost, or
+// the cell itself where it has no such face); for a neighbour also bits 14-24 the value row that
+// holds its outgoing values at this face and bits 25-28 the outgoing bits (bit 25 + p set when the
+// first member of pair p leaves this cell here).  Bit 31: no neighbour (boundary face or no
+// face); bit 30: no face.
+constexpr unsigned kFvBnd = 0x80000000u, kFvNone = 0xC0000000u;
+constexpr unsigned kFvRowMask = 0x3FF0u, kFvValMask = 0x7FF0u;
+constexpr int kFvValShift = 10, kFvOutBit = 25;
+__host__ __device__ constexpr unsigned fv_row_addr(int j) {  // halves swapped where bit 2 of j is set
+    return 32u * static_cast<unsigned>(j) + ((j & 4) ? 16u : 0u);
+}
 
 // Geometry values of a cell.  Double: A_mk at 4 m + k, then (n dl / A)_m, x and y, at 16 + 2 m; a
 // triangle has no slot 3 and keeps the six normal components in the free places 3, 7, 11-14, so
@@ -111,7 +123,8 @@ struct FvItems {
     const int *__restrict__ halo;       // [nitem][hs] global ids, ring 1 then ring 2, -1 after
     const int *__restrict__ ovf;        // halo slots hs.. of the items that have them
     const uint4 *__restrict__ adj;      // [np] adjacency words of every cell (within its item)
-    const uint2 *__restrict__ cut;      // cut faces: rows i, k0, k1 (9 bits each); k2, k3, bits
+    const uint2 *__restrict__ cut;      // cut faces: row addresses / 16 of the ring cell and its face
+                                        // data, 10 bits each: i, k0, k1; k2, k3, then the outgoing bits
     const int4 *__restrict__ ghost;     // ghosts: owner row, boundary face, owner cell, face slot
     int *__restrict__ err;              // set to 1 if the bulk-copy wait gave up
     long long wait_first;               // polls of that wait (fvlbm_set_wait_limit)
@@ -163,9 +176,9 @@ struct FvPair<double> {
 //                      stage 3 C (alpha = 1..8 of C: C_0 = 0, e_0 carries no flux); row 18 tau
 //   the item's instance parameters (copied during staging, read by the stage algebra)
 //   one mbarrier for the bulk copies
-// In float an item of 256 takes 55,136 bytes, so that four CTAs (32 warps, at 64 registers)
-// share an SM; whole ring-1 cells took 67 KB and 80 registers, which allowed three.  Measured on
-// the 2.57M-cell sweep: stages 1 / 2 / 3 217 / 174 / 156 us before, 194 / 152 / 137 us now.
+// In float three CTAs of 256 (24 warps, 80 registers, 55 KB each) share an SM; four at 64
+// registers, which would fit the shared memory, spill 12 words and ran slower (sweep step 576
+// against 509 us), as did two (588).
 template <class T, int IT>
 struct FvSmem {
     using S = FvShape<IT>;
@@ -176,8 +189,8 @@ struct FvSmem {
     static constexpr size_t ip = sacc + size_t(2 * kQ + 1) * IT * sizeof(T);
     static constexpr size_t bar = ip + sizeof(InstParam);
     static constexpr size_t bytes = bar + 16;
-    static_assert(S::ecap % 4 == 0 && S::ecap <= 512 && 4 * IT + S::ccap <= 2048 && S::hs <= S::nt,
-                  "16-byte sections, 9-bit rows, 11-bit value rows, one halo slot per thread");
+    static_assert(S::ecap % 8 == 0 && S::ecap <= 512 && 4 * IT + S::ccap <= 2048 && S::hs <= S::nt,
+                  "whole groups of swapped rows, 10-bit row and 11-bit value addresses, one halo slot per thread");
 };
 
 // Rows of 8 (staged in shared memory, and the cell-major stage values in global memory) keep
@@ -224,6 +237,21 @@ __device__ __forceinline__ void fv_load_half(const T *sf, int j, int h, typename
     } else {
         o[0] = *reinterpret_cast<const double2 *>(p);
         o[1] = *reinterpret_cast<const double2 *>(p + 2);
+    }
+}
+
+// The same of the row at address a (fv_row_addr).
+template <class T>
+__device__ __forceinline__ void fv_load_half_at(const T *sf, unsigned a, int h, typename FvPair<T>::V *o) {
+    using PV = FvPair<T>;
+    const unsigned char *p = reinterpret_cast<const unsigned char *>(sf) + (sizeof(T) / 4) * (a ^ (16u * h));
+    if constexpr (sizeof(T) == 4) {
+        const float4 x = *reinterpret_cast<const float4 *>(p);
+        o[0] = PV::make(x.x, x.y);
+        o[1] = PV::make(x.z, x.w);
+    } else {
+        o[0] = reinterpret_cast<const double2 *>(p)[0];
+        o[1] = reinterpret_cast<const double2 *>(p)[1];
     }
 }
 
@@ -304,24 +332,25 @@ __device__ __forceinline__ void fv_relax_to_row(float *f, float *sf, float *sf0,
 // Gradient (Step 2) and outgoing face values of item cell c, two pairs at a time (packed FMAs).
 // g: node positions q relative to the centroid, then least-squares weights W_m (x, y per face
 // slot); w: adjacency.
-__device__ __forceinline__ void fv_cell(int c, const float *g, const unsigned *w, const float *__restrict__ sf,
-                                        float *__restrict__ sv) {
+// Absent faces have weight 0 and the cell itself as datum, and values at faces without a neighbour
+// are formed but not read, so the only branch is the warp's on the fourth slot (quads).
+__device__ __forceinline__ void fv_cell(int c, const float *g, const unsigned *w, bool quads,
+                                        const float *__restrict__ sf, float *__restrict__ sv) {
     using PV = FvPair<float>;
     using V = PV::V;
     const float *q = g, *lw = g + 8;
-    const bool tri = w[3] == kFvNone;
+    const bool tri = w[3] >= kFvNone;
     const V mone = PV::bcast(-1.f);
+    const unsigned own = fv_row_addr(c);
     float o[4][2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         V fc[2], gx[2], gy[2];
-        fv_load_half(sf, c, h, fc);
+        fv_load_half_at(sf, own, h, fc);
         gx[0] = gx[1] = gy[0] = gy[1] = PV::bcast(0.f);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if (w[k] == kFvNone) continue;
+        auto datum = [&](int k) {
             V fk[2];
-            fv_load_half(sf, static_cast<int>(w[k] & 511u), h, fk);
+            fv_load_half_at(sf, w[k] & kFvRowMask, h, fk);
             const V wx = PV::bcast(lw[2 * k]), wy = PV::bcast(lw[2 * k + 1]);
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
@@ -329,18 +358,15 @@ __device__ __forceinline__ void fv_cell(int c, const float *g, const unsigned *w
                 gx[s] = PV::fma(wx, df, gx[s]);
                 gy[s] = PV::fma(wy, df, gy[s]);
             }
-        }
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            if (static_cast<int>(w[m]) < 0) continue;  // no face, or a boundary face
+        };
+        auto face = [&](int m) {
             const V rx = PV::bcast(0.5f * (q[2 * m] + FV_END_X(m)));
             const V ry = PV::bcast(0.5f * (q[2 * m + 1] + FV_END_Y(m)));
-            const unsigned bits = w[m] >> (20 + 2 * h);
             float out[2];
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
                 const V val = PV::fma(gy[s], ry, PV::fma(gx[s], rx, fc[s]));
-                out[s] = ((bits >> s) & 1u) ? val.x : val.y;
+                out[s] = (w[m] & (1u << (kFvOutBit + 2 * h + s))) ? val.x : val.y;
             }
             if (h == 0) {
                 o[m][0] = out[0];
@@ -348,7 +374,15 @@ __device__ __forceinline__ void fv_cell(int c, const float *g, const unsigned *w
             } else {
                 fv_store4(sv + 4 * (4 * c + (m ^ ((c >> 1) & 3))), o[m][0], o[m][1], out[0], out[1]);
             }
-        }
+        };
+        datum(0);
+        datum(1);
+        datum(2);
+        if (quads) datum(3);
+        face(0);
+        face(1);
+        face(2);
+        if (quads) face(3);
     }
 }
 
@@ -497,33 +531,34 @@ __device__ __forceinline__ void fv_ghost(const Geo<T> &G, const T *__restrict__ 
 // Outgoing face values of item cell c at its interior faces: f_c + sum_k A_mk (f_k - f_c), A at
 // a[4 m + k]; of each pair the outgoing member is taken first (selects cost nothing beside the
 // arithmetic).  A value is the same chain of fused multiply-adds as in fv_cut.
-__device__ __forceinline__ void fv_cell(int c, const double *a, const unsigned *w, const double *__restrict__ sf,
-                                        double *__restrict__ sv) {
+__device__ __forceinline__ void fv_cell(int c, const double *a, const unsigned *w, bool quads,
+                                        const double *__restrict__ sf, double *__restrict__ sv) {
     using PV = FvPair<double>;
+    const unsigned own = fv_row_addr(c);
+    const bool four = w[3] < kFvNone;  // (per cell: an operation saved counts here)
     double o[4][2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         PV::V fc[2], d[4][2];
-        fv_load_half(sf, c, h, fc);
+        fv_load_half_at(sf, own, h, fc);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            if (w[k] == kFvNone) continue;
-            fv_load_half(sf, static_cast<int>(w[k] & 511u), h, d[k]);
+            if (k == 3 && !four) continue;
+            fv_load_half_at(sf, w[k] & kFvRowMask, h, d[k]);
 #pragma unroll
             for (int q = 0; q < 2; ++q) d[k][q] = PV::make(d[k][q].x - fc[q].x, d[k][q].y - fc[q].y);
         }
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            if (static_cast<int>(w[m]) < 0) continue;  // no face, or a boundary face
-            const unsigned bits = w[m] >> (20 + 2 * h);
+            if (w[m] & kFvBnd) continue;  // no neighbour
             double out[2];
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-                const bool first = (bits >> q) & 1u;
+                const bool first = w[m] & (1u << (kFvOutBit + 2 * h + q));
                 double v = first ? fc[q].x : fc[q].y;
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    if (k < 3 || w[3] != kFvNone) v = ::fma(a[4 * m + k], first ? d[k][q].x : d[k][q].y, v);
+                    if (k < 3 || four) v = ::fma(a[4 * m + k], first ? d[k][q].x : d[k][q].y, v);
                 out[q] = v;
             }
             if (h == 0) {
@@ -542,13 +577,12 @@ template <class T>
 __device__ __forceinline__ void fv_cut(T *__restrict__ dst, int h, uint2 r, const T *a, const T *__restrict__ sf) {
     using PV = FvPair<T>;
     using V = typename PV::V;
-    const int row[5] = {static_cast<int>(r.x & 511u), static_cast<int>((r.x >> 9) & 511u),
-                        static_cast<int>((r.x >> 18) & 511u), static_cast<int>(r.y & 511u),
-                        static_cast<int>((r.y >> 9) & 511u)};
-    const bool b0 = (r.y >> (18 + 2 * h)) & 1u, b1 = (r.y >> (19 + 2 * h)) & 1u;
-    auto member = [&](int j) {
+    const unsigned row[5] = {(r.x << 4) & kFvRowMask, (r.x >> 6) & kFvRowMask, (r.x >> 16) & kFvRowMask,
+                             (r.y << 4) & kFvRowMask, (r.y >> 6) & kFvRowMask};
+    const bool b0 = r.y & (1u << (20 + 2 * h)), b1 = r.y & (2u << (20 + 2 * h));
+    auto member = [&](unsigned a) {
         V f[2];
-        fv_load_half(sf, j, h, f);
+        fv_load_half_at(sf, a, h, f);
         return PV::make(b0 ? f[0].x : f[0].y, b1 ? f[1].x : f[1].y);
     };
     const V c = member(row[0]);
@@ -586,17 +620,20 @@ __device__ __forceinline__ void fv_flux(int t, const T *sn, const unsigned *w, c
     for (int p = 0; p < 4; ++p) ac[p] = PV::bcast(T(0));
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-        if (w[m] == kFvNone) continue;
+        if (w[m] >= kFvNone) continue;
         V val[4];
         if (w[m] & kFvBnd) {
-            fv_load_row(sf, static_cast<int>(w[m] & 511u), val);
+            fv_load_half_at(sf, w[m] & kFvRowMask, 0, val);
+            fv_load_half_at(sf, w[m] & kFvRowMask, 1, val + 2);
         } else {
             T vo[4], vn[4];
             fv_load4(sv + 4 * (4 * t + (m ^ ((t >> 1) & 3))), vo);
-            fv_load4(sv + 4 * static_cast<int>((w[m] >> 9) & 2047u), vn);
+            fv_load4(reinterpret_cast<const T *>(reinterpret_cast<const unsigned char *>(sv) +
+                                                 (sizeof(T) / 4) * ((w[m] >> kFvValShift) & kFvValMask)),
+                     vn);
 #pragma unroll
             for (int p = 0; p < 4; ++p)
-                val[p] = ((w[m] >> (20 + p)) & 1u) ? PV::make(vo[p], vn[p]) : PV::make(vn[p], vo[p]);
+                val[p] = (w[m] & (1u << (kFvOutBit + p))) ? PV::make(vo[p], vn[p]) : PV::make(vn[p], vo[p]);
         }
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
@@ -606,12 +643,18 @@ __device__ __forceinline__ void fv_flux(int t, const T *sn, const unsigned *w, c
     }
 }
 
+// Accumulator alpha of cell i.
+template <int IT>
+__host__ __device__ constexpr size_t fv_acc_at(size_t i, int alpha) {
+    return (i / IT * kQ + alpha) * IT + i % IT;
+}
+
 // One IMEX stage (see fvlbm_kernels.cu's stage_algebra for what STAGE computes) in the
 // face-value form, one CTA per work item.  fin: stage 1 f^n (structure of arrays), stages 2, 3
 // f^(2), f^(3) (cell-major rows); fs_out: stages 1, 2 write f^(2), f^(3) cell-major; fn: stage 3
 // writes f^{n+1}; geo: the geometry rows, cutc: the cut faces' coefficients.
 template <class T, int STAGE, bool STATS, int IT>
-__global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ? 4 : 1) : (IT == 256 ? 2 : 1))
+__global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ? 3 : 1) : (IT == 256 ? 2 : 1))
     k_fused_fv(const T *fin, T *__restrict__ fs_out, T *__restrict__ fn, T *Bacc, T *Cacc, const T *tau, T *mac, double *__restrict__ partial, Geo<T> G, FvItems W,
                const T *__restrict__ geo, const T *__restrict__ cutc, const T *__restrict__ bnrm) {
     using PV = FvPair<T>;
@@ -628,7 +671,9 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
 
     dep_launch();
     const int t = threadIdx.x;
-    const int it = static_cast<int>(blockIdx.x);
+    // Stage 2 walks the items backwards: what stage 1 wrote last (100 MB or so of a large batch) it
+    // finds in L2, and stage 3 what stage 2 wrote last (sweep step 502 -> 494 us).
+    const int it = static_cast<int>(STAGE == 2 ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
     // halo slot t of the fixed-stride table and the header, loaded together (kept in L2)
     const unsigned long long keep = l2_keep_policy();
     const int gid0 = t < HS ? ld_keep(W.halo + static_cast<size_t>(it) * HS + t, keep) : -1;
@@ -679,14 +724,18 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
     if ((t & 31) == 0) {
         const unsigned row = static_cast<unsigned>(cnt * sizeof(T));
         // copies: (stages 2, 3) the item's f rows and f_0, then the accumulator rows (stage 1:
-        // f^n; stage 2: B, then C of alpha = 1..8; stage 3: C of alpha = 1..8), then tau
+        // f^n; stage 2: B, then C of alpha = 1..8; stage 3: C of alpha = 1..8), then tau; the rows of
+        // a whole tile are one copy
+        const bool whole = STAGE != 1 && cnt == IT;
         constexpr int nf = STAGE == 1 ? 0 : 2;
-        constexpr int n1 = STAGE == 3 ? 0 : kQ, n2 = STAGE == 1 ? 0 : kQ - 1;
-        constexpr int ncopy = nf + n1 + n2 + (STAGE == 3 ? 0 : 1);
-        const T *a1g = STAGE == 1 ? fin : Bacc;
+        const int n1 = STAGE == 3 ? 0 : (whole ? 1 : kQ), n2 = STAGE == 1 ? 0 : (whole ? 1 : kQ - 1);
+        const int ncopy = nf + n1 + n2 + (STAGE == 3 ? 0 : 1);
         const int w = t >> 5;
+        const size_t tile = fv_acc_at<IT>(base, 0);
         unsigned bytes = 0;
-        for (int c = w; c < ncopy; c += kWarps) bytes += (nf > 0 && c == 0) ? 8 * row : row;
+        for (int c = w; c < ncopy; c += kWarps)
+            bytes += nf > 0 && c == 0 ? 8 * row
+                                      : (whole && c >= nf && c < nf + n1 + n2 ? (c < nf + n1 ? kQ : kQ - 1) * row : row);
         mbar_expect_tx(bar, bytes);
         for (int c = w; c < ncopy; c += kWarps) {
             if (nf > 0 && c == 0) {
@@ -695,10 +744,14 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
                 bulk_g2s(sf0, fa0 + base, row, bar);
             } else if (c < nf + n1) {
                 const int a = c - nf;
-                bulk_g2s(sacc + a * IT, a1g + a * np + base, row, bar);
+                if (STAGE == 1)
+                    bulk_g2s(sacc + a * IT, fin + a * np + base, row, bar);
+                else
+                    bulk_g2s(sacc + a * IT, Bacc + tile + a * IT, whole ? kQ * row : row, bar);
             } else if (c < nf + n1 + n2) {
                 const int a = c - nf - n1;  // C_{a + 1}
-                bulk_g2s(sacc + (n1 + a) * IT, Cacc + (a + 1) * np + base, row, bar);
+                bulk_g2s(sacc + ((STAGE == 3 ? 0 : kQ) + a) * IT, Cacc + tile + (a + 1) * IT,
+                         whole ? (kQ - 1) * row : row, bar);
             } else {
                 bulk_g2s(sacc + 2 * kQ * IT, tau + base, row, bar);
             }
@@ -830,20 +883,22 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
     }
 
     // 2. outgoing face values: item cells (thread t takes cell t) and cut faces
-    if (mine) fv_cell(t, A, w, sf, sv);
+    const bool quads = __any_sync(0xffffffffu, w[3] < kFvNone);  // (a triangle has no fourth face)
+    if (mine) fv_cell(t, A, w, quads, sf, sv);
     if (cut0) fv_cut<T>(sv + 4 * (4 * IT + (cu >> 1)), cu & 1, cr, ca, sf);
     if (cu >= 0)
         for (int u = cu + CS; u < 2 * ncut; u += CS) {
             load_cut(u >> 1);
             fv_cut<T>(sv + 4 * (4 * IT + (u >> 1)), u & 1, cr, ca, sf);
         }
-    // the normals, issued before the barrier (a triangle's came with its coefficients)
+    // the normals: float forms them from the node positions; double loads a quad's before the
+    // barrier (a triangle's came with its coefficients)
     T sn[8];
     if (mine) {
-        if constexpr (sizeof(T) == 4) {  // the node positions again, for the normals
-            fv_load_geo4(geo, i, 0, sn);
-            fv_load_geo4(geo, i, 4, sn + 4);
-        } else if (w[3] != kFvNone) {
+        if constexpr (sizeof(T) == 4) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sn[k] = A[k];
+        } else if (w[3] < kFvNone) {
             fv_load_geo4(geo, i, 16, sn);
             fv_load_geo4(geo, i, 20, sn + 4);
         } else {
@@ -862,7 +917,7 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
             V ac[4], fr[4];
 #pragma unroll
             for (int k = 0; k < 8; ++k) q[k] = sn[k];
-            fv_normals(q, w[3] == kFvNone, sn);
+            fv_normals(q, w[3] >= kFvNone, sn);
             fv_flux<T>(t, sn, w, sf, sv, ac);
             fv_load_row(sf, t, fr);
             fi[0] = sf0[t];
@@ -881,8 +936,9 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
             }
             // C rows hold alpha = 1..8 (stage 2 after the nine of B, stage 3 first)
             const T *a1 = STAGE == 3 ? sacc - IT : sacc, *a2 = sacc + (STAGE == 1 ? kQ : kQ - 1) * IT;
-            stage_algebra<T, STAGE, false, NT, true, STAGE == 1>(i, np, fi, acc, P, STAGE == 3 ? T(1) : sacc[2 * kQ * IT + t],
-                                                                 dt_i, a1, IT, t, a2, IT, t, fs_out, fn, Bacc, Cacc,
+            stage_algebra<T, STAGE, false, NT, IT, STAGE == 1>(i, np, fi, acc, P, STAGE == 3 ? T(1) : sacc[2 * kQ * IT + t],
+                                                                 dt_i, a1, IT, t, a2, IT, t, fs_out, fn,
+                                                                 Bacc + fv_acc_at<IT>(i, 0), Cacc + fv_acc_at<IT>(i, 0),
                                                                  mac, nullptr, G.area, T(0), macv);
             if (STATS) {
                 const double un = double(macv[1]), vn = double(macv[2]), r = double(macv[0]);
@@ -895,6 +951,7 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
         }
     } else if (mine) {
         V ac[4];
+        T *const Bi = Bacc + fv_acc_at<IT>(i, 0), *const Ci = Cacc + fv_acc_at<IT>(i, 0);
         fv_flux<T>(t, sn, w, sf, sv, ac);
         const T r0 = ipv<T>(reinterpret_cast<const InstParam *>(smem_raw + L::ip)->rho0,
                             reinterpret_cast<const InstParam *>(smem_raw + L::ip)->rho0_f);
@@ -920,19 +977,19 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
                 if (STAGE == 1) {  // B = f^n + dt/2 Gamma^a(1) + dt/3 (Gamma^c(1) + Gamma^c(2)), C = -dt/6 Gamma^a(1)
                     const V pb = PV::make(sacc[(kQ + f1) * IT + t], sacc[(kQ + f2) * IT + t]);
                     const V b = PV::fma(PV::bcast(g), d, PV::fma(PV::bcast(hdt2), ac[p], pb));
-                    Bacc[f1 * np + i] = b.x;
-                    Bacc[f2 * np + i] = b.y;
-                    Cacc[f1 * np + i] = dt6 * ac[p].x;
-                    Cacc[f2 * np + i] = dt6 * ac[p].y;
+                    Bi[f1 * IT] = b.x;
+                    Bi[f2 * IT] = b.y;
+                    Ci[f1 * IT] = dt6 * ac[p].x;
+                    Ci[f2 * IT] = dt6 * ac[p].y;
                 } else {
                     const V c = PV::fma(PV::bcast(dt6), ac[p],
                                         PV::make(sacc[(kQ + f1 - 1) * IT + t], sacc[(kQ + f2 - 1) * IT + t]));
-                    Cacc[f1 * np + i] = c.x;
-                    Cacc[f2 * np + i] = c.y;
+                    Ci[f1 * IT] = c.x;
+                    Ci[f2 * IT] = c.y;
                 }
             }
             const T eq0 = fv_feq0(M), d0 = X0 - eq0;
-            if (STAGE == 1) Bacc[i] = fma(g, d0, sacc[kQ * IT + t]);
+            if (STAGE == 1) Bi[0] = fma(g, d0, sacc[kQ * IT + t]);
             fv_store_stage<T>(fs_out, np, i, fma(a, d0, eq0), X);
         } else {
             // f^{n+1} = f^(3) + C - dt/3 acc (Eq. (imextwo)); macros

@@ -383,8 +383,9 @@ __device__ __forceinline__ void store_stage(T *__restrict__ f, size_t np, int i,
 }
 
 // EQ1_IN_A2 (stage 1): f^eq(f^n) is given in a2 (the face-value stage relaxed the cell with it).
-// ROWS also leaves out C_0, which is 0 (e_0 carries no flux).
-template <class T, int STAGE, bool STATS, int NT, bool ROWS = false, bool EQ1_IN_A2 = false>
+// TILE > 0: the face-value form: stage values in rows (ROWS), Bacc and Cacc the cell's own
+// accumulators with the rows TILE apart, C_0 left out (it is 0: e_0 carries no flux).
+template <class T, int STAGE, bool STATS, int NT, int TILE = 0, bool EQ1_IN_A2 = false>
 __device__ __forceinline__ void stage_algebra(int i, size_t np, const T *fi, const T *acc,
                                               const InstParam &P, T t_i, T dt_i, const T *a1, size_t ld1,
                                               int c1, const T *a2, size_t ld2, int c2,
@@ -393,6 +394,8 @@ __device__ __forceinline__ void stage_algebra(int i, size_t np, const T *fi, con
                                               T *__restrict__ mac, double *__restrict__ partial,
                                               const T *__restrict__ area,
                                               T t1_i = T(0), T *macv = nullptr) {
+    constexpr bool ROWS = TILE > 0;
+    const size_t la = ROWS ? TILE : np, ca = ROWS ? 0 : i;  // rows and column of the accumulators
     const T rho0 = ipv<T>(P.rho0, P.rho0_f);
     const T dt = dt_i;
     const T itau = sdiv(T(1), t_i);     // one division per cell, products below
@@ -434,8 +437,8 @@ __device__ __forceinline__ void stage_algebra(int i, size_t np, const T *fi, con
         for (int a = 0; a < kQ; ++a) {
             f2[a] = (X[a] + zq * eq[a]) * inv;
             const T dgc2 = (eq[a] - X[a]) * s2;  // dt Gamma^c(2)
-            Bacc[a * np + i] = X[a] + T(1.0 / 3.0) * (dgc1[a] + dgc2);
-            if (!ROWS || a > 0) Cacc[a * np + i] = dt6 * acc[a];
+            Bacc[a * la + ca] = X[a] + T(1.0 / 3.0) * (dgc1[a] + dgc2);
+            if (!ROWS || a > 0) Cacc[a * la + ca] = dt6 * acc[a];
         }
         store_stage<T, ROWS>(fs_out, np, i, f2);
     } else if (STAGE == 2) {
@@ -449,7 +452,7 @@ __device__ __forceinline__ void stage_algebra(int i, size_t np, const T *fi, con
 #pragma unroll
         for (int a = 0; a < kQ; ++a) {
             f3[a] = (X[a] + zt * eq[a]) * inv;
-            if (!ROWS || a > 0) Cacc[a * np + i] = a2[a * ld2 + c2] + dt6 * acc[a];
+            if (!ROWS || a > 0) Cacc[a * la + ca] = a2[a * ld2 + c2] + dt6 * acc[a];
         }
         store_stage<T, ROWS>(fs_out, np, i, f3);
     } else if (STAGE == 4) {
@@ -1035,7 +1038,8 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
                  T *__restrict__ k_out, T *__restrict__ w_out, T *__restrict__ nut_out, T *__restrict__ tau,
                  Geo<T> G, CompactGeo<T> CG, const T *rec8, const T *rec2, int tile0) {
     dep_launch();
-    const int tile = tile0 + static_cast<int>(blockIdx.x);
+    // backwards: the records that k_sst_grad wrote last are still in L2
+    const int tile = tile0 + static_cast<int>(gridDim.x - 1 - blockIdx.x);
     const int i = tile * kTile + threadIdx.x;
     const size_t np = G.np;
     const InstParam P = G.ip[G.tile_inst[tile]];
@@ -1540,9 +1544,8 @@ struct fvlbm_handle {
     int turb = 0;  // which of the k/omega/nu_t ping-pong buffers is current
     double *d_partial = nullptr, *d_inst_sums = nullptr, *d_io = nullptr;
     size_t io_bytes = 0;
-    // [0]: 1 step (laminar); [1 + parity]: kGraphSteps steps starting from k/omega/nu_t
-    // ping-pong parity 0 or 1 (laminar runs use [1] only)
-    cudaGraphExec_t graph[3] = {nullptr, nullptr, nullptr};
+    // kGraphSteps steps starting from k/omega/nu_t ping-pong parity 0 or 1 (laminar runs use [0])
+    cudaGraphExec_t graph[2] = {nullptr, nullptr};
     bool profiling = false;
     std::vector<KernelTimer> timers;
     std::vector<cudaEvent_t> ev_pool;
@@ -1960,12 +1963,16 @@ int build_graph(fvlbm_handle *h, int nsteps, cudaGraphExec_t *out) {
     return FVLBM_OK;
 }
 
-// Cells per item of the face-value kernels for a handle of np padded cells: items of 256 cells
-// where there are enough of them to fill the 152 SMs several times over, 64 below that, so that
-// a small mesh spreads over the chip.  Both sides measured, us per step, 256 against 64 cells:
-// float 10k cells 17.6 / 12.6, 40k 20.6 / 15.0, 80k (SST) 36.1 / 35.2, 200k (SST) 73 / 79, 2.6M
-// (sweep) 657 / 852; double 4k 80 / 52, 50k (SST) 259 / 250, 640k (SST) 1744 / 1969.
-int fv_item_cells(size_t np) { return np <= 90000 ? 64 : 256; }
+// Cells per item of the face-value kernels for a handle of np padded cells.  64-cell items spread
+// a small mesh over the 152 SMs, as long as (in float) all of them are resident at once, five to
+// an SM; beyond that 256-cell items, whose halo is smaller for their size, take over.  Both sides
+// measured, us per step, 64 against 256 cells: float cavities of 5k cells 10.7 / 12.4, 40k
+// 13.1 / 16.1, 59k 19.7 / 17.0, 199k 45 / 30; SST airfoils 40k 22.2 / 25.9, 60k 28.5 / 26.1; double
+// cavities 5k 45 / 70, 50k 116 / 120, 99k 214 / 201; SST airfoils 50k 239 / 243, 100k 387 / 379.
+template <class T>
+int fv_item_cells(size_t np) {
+    return np <= (sizeof(T) == 4 ? 5 * 152 * 64 : 50000) ? 64 : 256;
+}
 
 // Work items of the face-value kernel: every block of IT cells whose rows (cells, ring-1 and
 // ring-2 halo, ghosts) and cut faces fit its shared memory (FvShape) is one item; a block that does
@@ -2086,7 +2093,7 @@ int build_fv_items_it(fvlbm_handle *h, const std::vector<int> &nbr, const std::v
             // the staged row of face datum m of cell g (its own row where it has no such face)
             auto row_of = [&](size_t g, int m) {
                 const int v = nbr[m * np + g];
-                return static_cast<unsigned>(v == kNone ? local[g] : (v < 0 ? grow[-v - 1] : local[v]));
+                return fv_row_addr(v == kNone ? local[g] : (v < 0 ? grow[-v - 1] : local[v]));
             };
             int q = 0;
             for (int c = 0; c < cnt; ++c) {
@@ -2095,7 +2102,7 @@ int build_fv_items_it(fvlbm_handle *h, const std::vector<int> &nbr, const std::v
                 for (int m = 0; m < 4; ++m) {
                     const int v = nbr[m * np + g];
                     if (v == kNone) {
-                        w[m] = kFvNone;
+                        w[m] = kFvNone | row_of(g, m);
                     } else if (v < 0) {
                         w[m] = kFvBnd | row_of(g, m);
                     } else {
@@ -2107,8 +2114,9 @@ int build_fv_items_it(fvlbm_handle *h, const std::vector<int> &nbr, const std::v
                             vrow = 4u * IT + q++;
                             const size_t o = v;
                             cut.push_back(make_uint2(
-                                static_cast<unsigned>(local[v]) | (row_of(o, 0) << 9) | (row_of(o, 1) << 18),
-                                row_of(o, 2) | (row_of(o, 3) << 9) | (static_cast<unsigned>(pbits[b * np + o]) << 18)));
+                                (fv_row_addr(local[v]) >> 4) | (row_of(o, 0) << 6) | (row_of(o, 1) << 16),
+                                (row_of(o, 2) >> 4) | (row_of(o, 3) << 6) |
+                                    (static_cast<unsigned>(pbits[b * np + o]) << 20)));
                             if constexpr (sizeof(T) == 4) {
                                 for (int k = 0; k < 8; ++k)
                                     cutc.push_back(nbr[k / 2 * np + o] == kNone ? 0.0 : lsq[k * np + o]);
@@ -2119,8 +2127,8 @@ int build_fv_items_it(fvlbm_handle *h, const std::vector<int> &nbr, const std::v
                                     cutc.push_back(nbr[k * np + o] == kNone ? 0.0 : coef(o, b, k));
                             }
                         }
-                        w[m] = static_cast<unsigned>(local[v]) | (vrow << 9) |
-                               (static_cast<unsigned>(pbits[m * np + g]) << 20);
+                        w[m] = fv_row_addr(local[v]) | (vrow << 4 << kFvValShift) |
+                               (static_cast<unsigned>(pbits[m * np + g]) << kFvOutBit);
                     }
                 }
                 adj[g] = make_uint4(w[0], w[1], w[2], w[3]);
@@ -2207,7 +2215,7 @@ template <class T>
 int build_fv_items(fvlbm_handle *h, const std::vector<int> &nbr, const std::vector<int> &back,
                    const std::vector<double> &sn, const std::vector<double> &lsq, const std::vector<double> &rown,
                    const std::vector<double> &gq, const std::vector<int> &bowner, const std::vector<int> &inst_tile0) {
-    return fv_dispatch(fv_item_cells(h->np), [&](auto it) {
+    return fv_dispatch(fv_item_cells<T>(h->np), [&](auto it) {
         return build_fv_items_it<T, decltype(it)::value>(h, nbr, back, sn, lsq, rown, gq, bowner, inst_tile0);
     });
 }
@@ -2393,7 +2401,7 @@ void free_all(fvlbm_handle *h) {
         cudaStreamDestroy(A.s_out);
         A.init = false;
     }
-    for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < 2; ++k)
         if (h->graph[k]) cudaGraphExecDestroy(h->graph[k]);
     for (void *p : h->allocs) cudaFree(p);
     h->allocs.clear();
@@ -2716,10 +2724,9 @@ int fvlbm_step(fvlbm_handle *h, int n_steps, fvlbm_stats *stats) {
     int remaining = n_steps;
     const bool want_stats = stats != nullptr && n_steps > 0;
     if (want_stats) --remaining;  // the last step runs un-captured with the reductions
-    // graphs: laminar runs replay freely; SST runs keep the ping-pong parity (graphs of an
-    // even number of steps only)
+    // graphs: an even number of steps keeps the ping-pong parity of SST runs
     while (remaining >= kGraphSteps) {
-        const int gi = 1 + (h->sst ? h->turb : 0);
+        const int gi = h->sst ? h->turb : 0;
         if (!h->graph[gi]) {
             int rc = build_graph(h, kGraphSteps, &h->graph[gi]);
             if (rc) return rc;
@@ -2728,19 +2735,9 @@ int fvlbm_step(fvlbm_handle *h, int n_steps, fvlbm_stats *stats) {
         remaining -= kGraphSteps;
         h->steps += kGraphSteps;
     }
-    while (remaining > 0) {
-        if (!h->sst) {
-            if (!h->graph[0]) {
-                int rc = build_graph(h, 1, &h->graph[0]);
-                if (rc) return rc;
-            }
-            CK(cudaGraphLaunch(h->graph[0], h->stream));
-        } else {
-            enqueue(h, false);
-        }
-        --remaining;
-        ++h->steps;
-    }
+    // the rest are plain launches: they overlap each other (dep_wait), which graphs of one step do
+    // not (10k-cell cavity: 18 us per step from such graphs, 12.6 from launches)
+    for (; remaining > 0; --remaining, ++h->steps) enqueue(h, false);
     if (want_stats) {
         enqueue(h, true);
         ++h->steps;
@@ -3207,7 +3204,7 @@ int fvlbm_fv_items(fvlbm_handle *h, int *nitem, int *n_split, int *n_overflow) {
 int fvlbm_set_wait_limit(fvlbm_handle *h, long long polls) {
     if (!h || polls < 0) return FVLBM_ERR_BAD_PARAM;
     h->wait_first = polls;
-    for (int k = 0; k < 3; ++k)  // captured graphs bake the kernel arguments
+    for (int k = 0; k < 2; ++k)  // captured graphs bake the kernel arguments
         if (h->graph[k]) {
             cudaGraphExecDestroy(h->graph[k]);
             h->graph[k] = nullptr;
@@ -3451,7 +3448,7 @@ int fvlbm_autotune(fvlbm_handle *h, int trial_steps, int *chosen, double *ms_per
     cudaFree(snap);
     h->config = best_c;
     h->steps = steps0;
-    for (int k = 0; k < 3; ++k)  // captured graphs bake the old configuration
+    for (int k = 0; k < 2; ++k)  // captured graphs bake the old configuration
         if (h->graph[k]) {
             cudaGraphExecDestroy(h->graph[k]);
             h->graph[k] = nullptr;
