@@ -698,6 +698,16 @@ __global__ void k_adj_gather(const double *__restrict__ L, const int *__restrict
 
 namespace {
 
+// The geometry adjoints of instance cells off + k (SoA, `runs` runs of stride np) in input order:
+// out[perm[k] * runs + c].
+__global__ void k_adj_gather_geo(const double *__restrict__ a, const int *__restrict__ perm, int off, int nc, int runs,
+                                 size_t np, double *__restrict__ out) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= nc) return;
+    double *o = out + static_cast<size_t>(perm[k]) * runs;
+    for (int c = 0; c < runs; ++c) o[c] = a[c * np + off + k];
+}
+
 // Device buffers of one adjoint call: one allocation, carved in 256-byte aligned pieces, freed
 // when the call returns.  The carving runs twice: once to measure, once on the allocation.
 struct AdjScratch {
@@ -953,6 +963,7 @@ int adjoint_impl(fvlbm_handle *h, int instance, int n_steps, const double *w, do
     std::vector<AdjState> snap(nsnap), st(K);
     std::vector<AdjStep> slot(K);
     AdjVars A{};
+    double *gsrc = nullptr;  // geometry adjoints of the instance, in input order
     const size_t nbt = std::max(h->nbt, 1);
     auto state = [&](AdjState &x) {
         x.f = M.get(nq);
@@ -1047,6 +1058,7 @@ int adjoint_impl(fvlbm_handle *h, int instance, int n_steps, const double *w, do
                 A.a_wd = M.get(np);
             }
             if (h->limit_f) A.a_area = M.get(np);
+            gsrc = M.get(38 * static_cast<size_t>(I.nc));
         }
     };
     carve();
@@ -1177,29 +1189,30 @@ int adjoint_impl(fvlbm_handle *h, int instance, int n_steps, const double *w, do
     // shape adjoint: the instance's slices of the geometry adjoints, in input order, then the
     // reverse of the host preprocessing
     GeometryAdjoint GA;
-    std::vector<int> perm(std::max(I.nc, 1));
-    std::vector<double> runs;
-    if (dJ_dxy) {
+    std::vector<double> btab(3 * static_cast<size_t>(std::max(I.nb, 1)));
+    if (dJ_dxy && I.nc > 0) {
         const size_t nc = I.nc;
-        CK(cudaMemcpyAsync(perm.data(), h->d_perm + perm_offset(h, instance), sizeof(int) * nc,
-                           cudaMemcpyDeviceToHost, s));
-        runs.resize(4 * 8 * nc + 6 * nc + 3 * static_cast<size_t>(std::max(I.nb, 1)));
-        const double *src[4] = {A.a_sn, A.a_lsq, A.a_rown, A.a_rnbr};
-        for (int q = 0; q < 4; ++q)
-            for (int c = 0; c < 8; ++c)
-                CK(cudaMemcpyAsync(runs.data() + (8 * q + c) * nc, src[q] + c * np + I.cell_off, sizeof(double) * nc,
-                                   cudaMemcpyDeviceToHost, s));
-        if (sst) {  // 1 / |d| [4 runs] and the wall distance
-            for (int c = 0; c < 4; ++c)
-                CK(cudaMemcpyAsync(runs.data() + (32 + c) * nc, A.a_dinv + c * np + I.cell_off, sizeof(double) * nc,
-                                   cudaMemcpyDeviceToHost, s));
-            CK(cudaMemcpyAsync(runs.data() + 36 * nc, A.a_wd + I.cell_off, sizeof(double) * nc,
-                               cudaMemcpyDeviceToHost, s));
+        double *d = gsrc;
+        auto fetch = [&](const double *a, int runs, std::vector<double> *to) -> int {
+            k_adj_gather_geo<<<(I.nc + 255) / 256, 256, 0, s>>>(a, h->d_perm + perm_offset(h, instance), I.cell_off,
+                                                               I.nc, runs, np, d);
+            CK(cudaGetLastError());
+            to->resize(runs * nc);
+            CK(cudaMemcpyAsync(to->data(), d, sizeof(double) * runs * nc, cudaMemcpyDeviceToHost, s));
+            d += runs * nc;
+            return FVLBM_OK;
+        };
+        int rc = fetch(A.a_sn, 8, &GA.sn);
+        rc = rc ? rc : fetch(A.a_lsq, 8, &GA.lsq);
+        rc = rc ? rc : fetch(A.a_rown, 8, &GA.rown);
+        rc = rc ? rc : fetch(A.a_rnbr, 8, &GA.rnbr);
+        if (sst) {  // 1 / |d| and the wall distance
+            rc = rc ? rc : fetch(A.a_dinv, 4, &GA.dinv);
+            rc = rc ? rc : fetch(A.a_wd, 1, &GA.wdist);
         }
-        if (A.a_area)  // the limiter's cell areas
-            CK(cudaMemcpyAsync(runs.data() + 37 * nc, A.a_area + I.cell_off, sizeof(double) * nc,
-                               cudaMemcpyDeviceToHost, s));
-        double *bt = runs.data() + 38 * nc;
+        if (A.a_area) rc = rc ? rc : fetch(A.a_area, 1, &GA.area);  // the limiter's cell areas
+        if (rc) return rc;
+        double *bt = btab.data();
         if (I.nb > 0) {
             CK(cudaMemcpyAsync(bt, A.a_bnrm + I.bface_off, sizeof(double) * I.nb, cudaMemcpyDeviceToHost, s));
             CK(cudaMemcpyAsync(bt + I.nb, A.a_bnrm + h->nbt + I.bface_off, sizeof(double) * I.nb,
@@ -1211,31 +1224,11 @@ int adjoint_impl(fvlbm_handle *h, int instance, int n_steps, const double *w, do
     CK(cudaStreamSynchronize(s));
     CK(cudaGetLastError());
     if (dJ_dxy) {
-        const size_t nc = I.nc;
         const MeshCopy &mc = *I.mesh;
-        std::vector<double> *dst[4] = {&GA.sn, &GA.lsq, &GA.rown, &GA.rnbr};
-        for (int q = 0; q < 4; ++q) {
-            dst[q]->assign(8 * nc, 0.0);
-            for (size_t k = 0; k < nc; ++k)
-                for (int c = 0; c < 8; ++c)  // component c = 2 l + (x, y) of slot l
-                    (*dst[q])[8 * static_cast<size_t>(perm[k]) + c] = runs[(8 * q + c) * nc + k];
-        }
-        if (sst) {
-            GA.dinv.assign(4 * nc, 0.0);
-            GA.wdist.assign(nc, 0.0);
-            for (size_t k = 0; k < nc; ++k) {
-                for (int l = 0; l < 4; ++l) GA.dinv[4 * static_cast<size_t>(perm[k]) + l] = runs[(32 + l) * nc + k];
-                GA.wdist[perm[k]] = runs[36 * nc + k];
-            }
-        }
-        if (A.a_area) {
-            GA.area.assign(nc, 0.0);
-            for (size_t k = 0; k < nc; ++k) GA.area[perm[k]] = runs[37 * nc + k];
-        }
         const size_t nbe = mc.btype.size();
         GA.bnrm.assign(2 * nbe, 0.0);
         GA.blen.assign(nbe, 0.0);
-        const double *bt = runs.data() + 38 * nc;
+        const double *bt = btab.data();
         for (int f = 0; f < I.nb; ++f) {
             const int e = I.bedge_of[f];
             GA.bnrm[2 * e] = bt[f];

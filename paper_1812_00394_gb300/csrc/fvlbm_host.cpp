@@ -517,29 +517,38 @@ int geometry_adjoint(const fvlbm_mesh &m, const fvlbm_bc &bc, const GeometryAdjo
         return FVLBM_ERR_NOT_SUPPORTED;
     }
     // face neighbours (input ids) and boundary edges of every face slot
+    // (an open-addressing table of edges: a node-based map took a tenth of the call)
     std::vector<int> nbr(4 * static_cast<size_t>(nc), kNone);
-    std::unordered_map<uint64_t, Side> open;
-    open.reserve(static_cast<size_t>(nc) * 3);
+    size_t cap = 16;
+    while (cap < 2 * static_cast<size_t>(m.cell_ptr[nc])) cap *= 2;
+    std::vector<uint64_t> key(cap, ~0ull);
+    std::vector<int> side(cap);  // 4 cell + face
+    auto slot_of = [&](uint64_t id) {
+        size_t h = static_cast<size_t>((id * 0x9E3779B97F4A7C15ull) >> 20) & (cap - 1);
+        while (key[h] != ~0ull && key[h] != id) h = (h + 1) & (cap - 1);
+        return h;
+    };
     for (int i = 0; i < nc; ++i) {
         const int p0 = m.cell_ptr[i], nv = m.cell_ptr[i + 1] - p0;
         for (int l = 0; l < nv; ++l) {
             const uint64_t id = edge_id(m.cell_nodes[p0 + l], m.cell_nodes[p0 + (l + 1) % nv]);
-            auto it = open.find(id);
-            if (it == open.end()) {
-                open.emplace(id, Side{i, l});
+            const size_t h = slot_of(id);
+            if (key[h] == ~0ull) {
+                key[h] = id;
+                side[h] = 4 * i + l;
             } else {
-                nbr[4 * static_cast<size_t>(i) + l] = it->second.cell;
-                nbr[4 * static_cast<size_t>(it->second.cell) + it->second.local] = i;
+                nbr[4 * static_cast<size_t>(i) + l] = side[h] / 4;
+                nbr[side[h]] = i;
             }
         }
     }
     for (int b = 0; b < bc.n_bedges; ++b) {
-        auto it = open.find(edge_id(bc.bedge_nodes[2 * b], bc.bedge_nodes[2 * b + 1]));
-        if (it == open.end()) {
+        const size_t h = slot_of(edge_id(bc.bedge_nodes[2 * b], bc.bedge_nodes[2 * b + 1]));
+        if (key[h] == ~0ull) {
             *why = "boundary edge not on the mesh";
             return FVLBM_ERR_BAD_BC;
         }
-        nbr[4 * static_cast<size_t>(it->second.cell) + it->second.local] = -(b + 1);
+        nbr[side[h]] = -(b + 1);
     }
     std::vector<double> cxv(nc), cyv(nc), dc(2 * static_cast<size_t>(nc), 0.0);
     for (int i = 0; i < nc; ++i) {
@@ -547,8 +556,14 @@ int geometry_adjoint(const fvlbm_mesh &m, const fvlbm_bc &bc, const GeometryAdjo
         cell_area_centroid(m, i, m.xy, &ar, &cxv[i], &cyv[i]);
     }
     std::fill(dxy, dxy + 2 * static_cast<size_t>(nn), 0.0);
+    // Each cell's contributions are formed by all cores (every core seeds its own copy of the node
+    // positions), then added up in cell order, so that the sums do not depend on the cores.
+    std::vector<double> gown(8 * static_cast<size_t>(nc)), gnbr(8 * static_cast<size_t>(nc));
+#pragma omp parallel
+    {
     std::vector<Dual> xyd(2 * static_cast<size_t>(nn));
     for (size_t k = 0; k < xyd.size(); ++k) xyd[k] = Dual(m.xy[k], 0.0);
+#pragma omp for schedule(static)
     for (int i = 0; i < nc; ++i) {
         const int p0 = m.cell_ptr[i], nv = m.cell_ptr[i + 1] - p0;
         const int *nb = nbr.data() + 4 * static_cast<size_t>(i);
@@ -583,7 +598,7 @@ int geometry_adjoint(const fvlbm_mesh &m, const fvlbm_bc &bc, const GeometryAdjo
                 xyd[2 * a + c].d = 1.0;
                 cell_geometry<Dual>(m, i, xyd.data(), nb, nbx, nby, &G);
                 xyd[2 * a + c].d = 0.0;
-                dxy[2 * a + c] += contract(G);
+                gown[8 * static_cast<size_t>(i) + 2 * l + c] = contract(G);
             }
         }
         for (int l = 0; l < nv; ++l) {  // neighbour centroids
@@ -592,9 +607,20 @@ int geometry_adjoint(const fvlbm_mesh &m, const fvlbm_bc &bc, const GeometryAdjo
                 (c == 0 ? nbx[l] : nby[l]).d = 1.0;
                 cell_geometry<Dual>(m, i, xyd.data(), nb, nbx, nby, &G);
                 (c == 0 ? nbx[l] : nby[l]).d = 0.0;
-                dc[2 * static_cast<size_t>(nb[l]) + c] += contract(G);
+                gnbr[8 * static_cast<size_t>(i) + 2 * l + c] = contract(G);
             }
         }
+    }
+    }
+    for (int i = 0; i < nc; ++i) {
+        const int p0 = m.cell_ptr[i], nv = m.cell_ptr[i + 1] - p0;
+        const int *nb = nbr.data() + 4 * static_cast<size_t>(i);
+        for (int l = 0; l < nv; ++l)
+            for (int c = 0; c < 2; ++c) {
+                const size_t o = 8 * static_cast<size_t>(i) + 2 * l + c;
+                dxy[2 * m.cell_nodes[p0 + l] + c] += gown[o];
+                if (nb[l] >= 0) dc[2 * static_cast<size_t>(nb[l]) + c] += gnbr[o];
+            }
     }
     // wall distance: the nearest wall face (first of equals, in input order, as the forward
     // search keeps it) and the point-segment distance's local Jacobian
@@ -617,6 +643,7 @@ int geometry_adjoint(const fvlbm_mesh &m, const fvlbm_bc &bc, const GeometryAdjo
                 }
             }
         }
+#pragma omp parallel for schedule(static)
         for (int i = 0; i < static_cast<int>(nearest.size()); ++i) {
             const double lw = A.wdist[i];
             if (lw == 0.0 || nearest[i] < 0) continue;
@@ -626,7 +653,14 @@ int geometry_adjoint(const fvlbm_mesh &m, const fvlbm_bc &bc, const GeometryAdjo
                 Dual in[6] = {Dual(cxv[i]), Dual(cyv[i]), Dual(m.xy[2 * a0]), Dual(m.xy[2 * a0 + 1]),
                               Dual(m.xy[2 * a1]), Dual(m.xy[2 * a1 + 1])};
                 in[k].d = 1.0;
-                const double g = lw * point_segment(in[0], in[1], in[2], in[3], in[4], in[5]).d;
+                gown[8 * static_cast<size_t>(i) + k] = lw * point_segment(in[0], in[1], in[2], in[3], in[4], in[5]).d;
+            }
+        }
+        for (int i = 0; i < static_cast<int>(nearest.size()); ++i) {
+            if (A.wdist[i] == 0.0 || nearest[i] < 0) continue;
+            const int a0 = bc.bedge_nodes[2 * nearest[i]], a1 = bc.bedge_nodes[2 * nearest[i] + 1];
+            for (int k = 0; k < 6; ++k) {
+                const double g = gown[8 * static_cast<size_t>(i) + k];
                 if (k < 2)
                     dc[2 * static_cast<size_t>(i) + k] += g;
                 else
@@ -635,18 +669,31 @@ int geometry_adjoint(const fvlbm_mesh &m, const fvlbm_bc &bc, const GeometryAdjo
         }
     }
     // centroid adjoints to the nodes of their cells
-    for (int j = 0; j < nc; ++j) {
-        const int p0 = m.cell_ptr[j], nv = m.cell_ptr[j + 1] - p0;
-        for (int l = 0; l < nv; ++l) {
-            const int a = m.cell_nodes[p0 + l];
-            for (int c = 0; c < 2; ++c) {
-                xyd[2 * a + c].d = 1.0;
-                Dual ar, cx, cy;
-                cell_area_centroid<Dual>(m, j, xyd.data(), &ar, &cx, &cy);
-                xyd[2 * a + c].d = 0.0;
-                dxy[2 * a + c] += dc[2 * static_cast<size_t>(j)] * cx.d + dc[2 * static_cast<size_t>(j) + 1] * cy.d;
+#pragma omp parallel
+    {
+        std::vector<Dual> xyd(2 * static_cast<size_t>(nn));
+        for (size_t k = 0; k < xyd.size(); ++k) xyd[k] = Dual(m.xy[k], 0.0);
+#pragma omp for schedule(static)
+        for (int j = 0; j < nc; ++j) {
+            const int p0 = m.cell_ptr[j], nv = m.cell_ptr[j + 1] - p0;
+            for (int l = 0; l < nv; ++l) {
+                const int a = m.cell_nodes[p0 + l];
+                for (int c = 0; c < 2; ++c) {
+                    xyd[2 * a + c].d = 1.0;
+                    Dual ar, cx, cy;
+                    cell_area_centroid<Dual>(m, j, xyd.data(), &ar, &cx, &cy);
+                    xyd[2 * a + c].d = 0.0;
+                    gown[8 * static_cast<size_t>(j) + 2 * l + c] =
+                        dc[2 * static_cast<size_t>(j)] * cx.d + dc[2 * static_cast<size_t>(j) + 1] * cy.d;
+                }
             }
         }
+    }
+    for (int j = 0; j < nc; ++j) {
+        const int p0 = m.cell_ptr[j], nv = m.cell_ptr[j + 1] - p0;
+        for (int l = 0; l < nv; ++l)
+            for (int c = 0; c < 2; ++c)
+                dxy[2 * m.cell_nodes[p0 + l] + c] += gown[8 * static_cast<size_t>(j) + 2 * l + c];
     }
     return FVLBM_OK;
 }
