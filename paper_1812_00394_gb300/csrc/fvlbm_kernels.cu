@@ -1136,6 +1136,8 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
     tau[i] = tnew;
 }
 
+#include "fvlbm_sst64.cuh"
+
 // ------------------------------------------------------------------ state I/O kernels
 template <class T>
 __global__ void k_init_state(T *__restrict__ fn, T *__restrict__ mac, const double *__restrict__ r0,
@@ -1540,6 +1542,7 @@ struct fvlbm_handle {
     void *dtc = nullptr;    // local time stepping: dt of each cell (NULL: every instance global)
     void *kk[2] = {nullptr, nullptr}, *ww[2] = {nullptr, nullptr}, *nut[2] = {nullptr, nullptr};
     void *sgrad = nullptr, *f1 = nullptr;
+    double *ddl = nullptr;  // FP64 face-value handles with SST: |n dl / A| / |d| per face slot [4 np]
     void *sst_rec8 = nullptr, *sst_rec2 = nullptr;  // fused path: packed SST records [np][8], [np][2]
     int turb = 0;  // which of the k/omega/nu_t ping-pong buffers is current
     double *d_partial = nullptr, *d_inst_sums = nullptr, *d_io = nullptr;
@@ -1820,22 +1823,40 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
         if constexpr (kHasFused<T>) {
             if (h->config != 2) {  // compact geometry, packed records
                 T *r8 = static_cast<T *>(h->sst_rec8), *r2 = static_cast<T *>(h->sst_rec2);
-                launch(h, K_SST_GRAD, "sst_grad", [&] {
-                    for_sst_runs(h, [&](dim3 sg_grid, int t0) {
-                        launch_dep(k_sst_grad<T, true>, sg_grid, block, 0, s, mac, kc, wc, sg, f1, G, CG, nc, r8, r2,
-                                                                      !h->nonorth, t0);
+                if constexpr (std::is_same<T, double>::value) {
+                    if (!h->nonorth) {
+                        launch(h, K_SST_GRAD, "sst_grad", [&] {
+                            for_sst_runs(h, [&](dim3 g, int t0) {
+                                launch_dep(k_sst_grad64, dim3(g.x * (kTile / kSst64Block)), kSst64Block, 0, s, mac, kc, wc,
+                                           nc, sg, f1, r8, r2, G, t0 * kTile);
+                            });
+                        });
+                        launch(h, K_SST_UPDATE, "sst_update", [&] {
+                            for_sst_runs(h, [&](dim3 g, int t0) {
+                                launch_dep(k_sst_update64, dim3(g.x * (kTile / kSst64Block)), kSst64Block, 0, s, nc, sg, f1,
+                                           r8, r2, kn, wn, nn, tau, G, static_cast<const double *>(h->ddl), t0 * kTile);
+                            });
+                        });
+                    }
+                }
+                if (!std::is_same<T, double>::value || h->nonorth) {
+                    launch(h, K_SST_GRAD, "sst_grad", [&] {
+                        for_sst_runs(h, [&](dim3 sg_grid, int t0) {
+                            launch_dep(k_sst_grad<T, true>, sg_grid, block, 0, s, mac, kc, wc, sg, f1, G, CG, nc, r8, r2,
+                                                                          !h->nonorth, t0);
+                        });
                     });
-                });
-                launch(h, K_SST_UPDATE, "sst_update", [&] {
-                    for_sst_runs(h, [&](dim3 sg_grid, int t0) {
-                        if (h->nonorth)
-                            launch_dep(
-                                k_sst_update<T, true, true>, sg_grid, block, 0, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
-                        else
-                            launch_dep(
-                                k_sst_update<T, true, false>, sg_grid, block, 0, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
+                    launch(h, K_SST_UPDATE, "sst_update", [&] {
+                        for_sst_runs(h, [&](dim3 sg_grid, int t0) {
+                            if (h->nonorth)
+                                launch_dep(
+                                    k_sst_update<T, true, true>, sg_grid, block, 0, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
+                            else
+                                launch_dep(
+                                    k_sst_update<T, true, false>, sg_grid, block, 0, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
+                        });
                     });
-                });
+                }
             }
         }
         if (h->config == 2) {
@@ -2356,6 +2377,13 @@ int allocate_state(fvlbm_handle *h, const std::vector<const Prepared *> &P,
         if (h->fused) {
             if ((rc = build_fv_items<T>(h, nbr, back, sn, lsq, rown, gq, bowner, inst_tile0))) return rc;
             if (h->fv.ok) h->config = 3;
+            if (std::is_same<T, double>::value && h->fv.ok && h->sst) {
+                std::vector<double> ddl(4 * np);
+                for (int m = 0; m < 4; ++m)
+                    for (size_t k = 0; k < np; ++k)
+                        ddl[m * np + k] = std::hypot(sn[(2 * m) * np + k], sn[(2 * m + 1) * np + k]) * dinv[m * np + k];
+                if ((rc = upload_raw(h, &h->ddl, ddl))) return rc;
+            }
             if (h->config == 2) h->fused = false;
         }
     }
