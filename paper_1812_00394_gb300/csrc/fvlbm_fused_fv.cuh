@@ -652,7 +652,8 @@ __host__ __device__ constexpr size_t fv_acc_at(size_t i, int alpha) {
 // One IMEX stage (see fvlbm_kernels.cu's stage_algebra for what STAGE computes) in the
 // face-value form, one CTA per work item.  fin: stage 1 f^n (structure of arrays), stages 2, 3
 // f^(2), f^(3) (cell-major rows); fs_out: stages 1, 2 write f^(2), f^(3) cell-major; fn: stage 3
-// writes f^{n+1}; geo: the geometry rows, cutc: the cut faces' coefficients.
+// writes f^{n+1}; geo: the geometry rows, cutc: the cut faces' coefficients.  STAGE 4 is the explicit
+// Euler step: fin f^n, fs_out f^{n+1} (structure of arrays, another buffer: neighbours read f^n).
 template <class T, int STAGE, bool STATS, int IT>
 __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ? 3 : 1) : (IT == 256 ? 2 : 1))
     k_fused_fv(const T *fin, T *__restrict__ fs_out, T *__restrict__ fn, T *Bacc, T *Cacc, const T *tau, T *mac, double *__restrict__ partial, Geo<T> G, FvItems W,
@@ -662,6 +663,7 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
     using S = FvShape<IT>;
     using L = FvSmem<T, IT>;
     constexpr int NT = S::nt, HS = S::hs;
+    constexpr bool SOA = STAGE == 1 || STAGE == 4;  // reads f^n
     extern __shared__ __align__(128) unsigned char smem_raw[];
     T *sf = reinterpret_cast<T *>(smem_raw + L::sf);
     T *sf0 = reinterpret_cast<T *>(smem_raw + L::sf0);
@@ -726,9 +728,9 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
         // copies: (stages 2, 3) the item's f rows and f_0, then the accumulator rows (stage 1:
         // f^n; stage 2: B, then C of alpha = 1..8; stage 3: C of alpha = 1..8), then tau; the rows of
         // a whole tile are one copy
-        const bool whole = STAGE != 1 && cnt == IT;
-        constexpr int nf = STAGE == 1 ? 0 : 2;
-        const int n1 = STAGE == 3 ? 0 : (whole ? 1 : kQ), n2 = STAGE == 1 ? 0 : (whole ? 1 : kQ - 1);
+        const bool whole = !SOA && cnt == IT;
+        constexpr int nf = SOA ? 0 : 2;
+        const int n1 = STAGE == 3 ? 0 : (whole ? 1 : kQ), n2 = SOA ? 0 : (whole ? 1 : kQ - 1);
         const int ncopy = nf + n1 + n2 + (STAGE == 3 ? 0 : 1);
         const int w = t >> 5;
         const size_t tile = fv_acc_at<IT>(base, 0);
@@ -744,7 +746,7 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
                 bulk_g2s(sf0, fa0 + base, row, bar);
             } else if (c < nf + n1) {
                 const int a = c - nf;
-                if (STAGE == 1)
+                if (SOA)
                     bulk_g2s(sacc + a * IT, fin + a * np + base, row, bar);
                 else
                     bulk_g2s(sacc + a * IT, Bacc + tile + a * IT, whole ? kQ * row : row, bar);
@@ -765,12 +767,14 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
         const int gid = k == 0 ? gid0 : gid1;
         if (gid < 0) continue;
         const int e = cnt + t + k * HS;
-        if (STAGE == 1) {  // f^n is structure of arrays: one element per direction
+        if (SOA) {  // f^n is structure of arrays: one element per direction
 #pragma unroll
             for (int a = 1; a < kQ; ++a) cp_async<sizeof(T)>(sf + fv_alpha_off(e, a), fin + a * np + gid);
             cp_async<sizeof(T)>(sf0 + e, fin + gid);
-            htau[k] = tau[gid];
-            hdt[k] = G.dtc != nullptr ? G.dtc[gid] : dtg;
+            if (STAGE == 1) {
+                htau[k] = tau[gid];
+                hdt[k] = G.dtc != nullptr ? G.dtc[gid] : dtg;
+            }
         } else {  // one cell-major row: half h sits at half fv_half(gid, h) there, fv_half(e, h) here
             const T *src = fin + 8 * static_cast<size_t>(gid);
 #pragma unroll
@@ -870,6 +874,17 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
         }
         __syncthreads();
     }
+    if (STAGE == 4) {  // the item's staged rows from its f^n rows
+        if (mine) {
+            V f[4];
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+                f[p] = PV::make(sacc[fv_first(p) * IT + t], sacc[fv_second(p) * IT + t]);
+            sf0[t] = sacc[t];
+            fv_store_row(sf, t, f);
+        }
+        __syncthreads();
+    }
     // ghost rows of the boundary faces (few items have any; the count is the block's)
     if (hx.y > 0) {
         for (int q = t; q < hx.y; q += NT) {
@@ -955,7 +970,41 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
         fv_flux<T>(t, sn, w, sf, sv, ac);
         const T r0 = ipv<T>(reinterpret_cast<const InstParam *>(smem_raw + L::ip)->rho0,
                             reinterpret_cast<const InstParam *>(smem_raw + L::ip)->rho0_f);
-        if (STAGE == 1 || STAGE == 2) {
+        auto macros = [&](const V *f, T f0) {  // of the new f, and its statistics
+            const FvMoments<T> M = fv_moments<T>(f, f0, r0);
+            if (STATS) {
+                const double un = double(M.u), vn = double(M.v), r = double(M.r);
+                const double du = un - double(mac[np + i]), dv = vn - double(mac[2 * np + i]);
+                const bool bad = !(isfinite(un) && isfinite(vn) && isfinite(r));
+                st[0] = du * du + dv * dv;
+                st[1] = un * un + vn * vn;
+                st[2] = r * double(G.area[i]);
+                st[3] = bad ? 1.0 : 0.0;
+            }
+            mac[i] = M.r;
+            mac[np + i] = M.u;
+            mac[2 * np + i] = M.v;
+        };
+        if (STAGE == 4) {
+            // f^{n+1} = f^n + dt (Gamma^a + (f^eq - f^n) / tau)
+            const double itau = dt_i / sacc[2 * kQ * IT + t];
+            V f[4];
+            fv_load_row(sf, t, f);
+            const T f0 = sf0[t];
+            const FvMoments<T> M = fv_moments<T>(f, f0, r0);
+            T o[kQ];
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                const V eq = fv_feq<T>(M, p);
+                const V d = PV::make(eq.x - f[p].x, eq.y - f[p].y);
+                f[p] = PV::fma(PV::bcast(-dt_i), ac[p], PV::fma(PV::bcast(itau), d, f[p]));
+                o[fv_first(p)] = f[p].x;
+                o[fv_second(p)] = f[p].y;
+            }
+            o[0] = fma(itau, fv_feq0(M) - f0, f0);
+            store9(fs_out, np, i, o);
+            macros(f, o[0]);
+        } else if (STAGE == 1 || STAGE == 2) {
             // X = f^n - dt/2 acc (stage 1), B - dt/2 acc (stage 2); f^(J+1) = f^eq(X) + a (X - f^eq(X))
             T a, g;
             fv_factors(dt_i, sacc[2 * kQ * IT + t], STAGE == 1 ? T(0.25) : T(1.0 / 3.0), a, g);
@@ -1007,19 +1056,7 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
             }
             o[0] = sf0[t];
             store9(fn, np, i, o);
-            const FvMoments<T> M = fv_moments<T>(f, o[0], r0);
-            if (STATS) {
-                const double un = double(M.u), vn = double(M.v), r = double(M.r);
-                const double du = un - double(mac[np + i]), dv = vn - double(mac[2 * np + i]);
-                const bool bad = !(isfinite(un) && isfinite(vn) && isfinite(r));
-                st[0] = du * du + dv * dv;
-                st[1] = un * un + vn * vn;
-                st[2] = r * double(G.area[i]);
-                st[3] = bad ? 1.0 : 0.0;
-            }
-            mac[i] = M.r;
-            mac[np + i] = M.u;
-            mac[2 * np + i] = M.v;
+            macros(f, o[0]);
         }
     }
     if (STATS) block_sum<4, NT>(st, partial + 4 * it);

@@ -475,6 +475,11 @@ __device__ __forceinline__ void stage_algebra(int i, size_t np, const T *fi, con
         mac[0 * np + i] = r;
         mac[1 * np + i] = u;
         mac[2 * np + i] = v;
+        if (macv) {
+            macv[0] = r;
+            macv[1] = u;
+            macv[2] = v;
+        }
     } else {
         T fnew[kQ], dr, r, u, v;
 #pragma unroll
@@ -1509,7 +1514,7 @@ struct fvlbm_handle {
         int4 *d_ghost = nullptr;
         void *geo = nullptr, *cutc = nullptr;   // geometry of the cells, coefficients of the cuts
     } fv;
-    bool fused = false;     // fused kernels available (IMEX scheme, kernel_path 0 or 2)
+    bool fused = false;     // fused kernels wanted (kernel_path 0 or 2) and available
     int config = 2;         // 2: two-pass, 3: face-value fused (see fvlbm_autotune)
     int scheme = 0;         // 0: IMEX Runge-Kutta; 1: explicit Euler (comparison scheme)
     int kernel_path = 0;    // as requested at create (fvlbm_params.kernel_path)
@@ -1547,8 +1552,10 @@ struct fvlbm_handle {
     int turb = 0;  // which of the k/omega/nu_t ping-pong buffers is current
     double *d_partial = nullptr, *d_inst_sums = nullptr, *d_io = nullptr;
     size_t io_bytes = 0;
-    // kGraphSteps steps starting from k/omega/nu_t ping-pong parity 0 or 1 (laminar runs use [0])
-    cudaGraphExec_t graph[2] = {nullptr, nullptr};
+    // kGraphSteps steps starting from k/omega/nu_t ping-pong parity 0 or 1 (laminar runs use the
+    // first), and from either f^n buffer (+ 2; explicit Euler on the face-value kernel)
+    cudaGraphExec_t graph[4] = {nullptr, nullptr, nullptr, nullptr};
+    int fn_parity = 0;
     bool profiling = false;
     std::vector<KernelTimer> timers;
     std::vector<cudaEvent_t> ev_pool;
@@ -1754,10 +1761,33 @@ auto fv_dispatch(int it, F &&f) {
     return f(std::integral_constant<int, 64>());
 }
 
+// The explicit Euler step in the same form: f^n into the other buffer, which becomes f^n.
+template <class T, int IT>
+void fv_euler(fvlbm_handle *h, bool stats) {
+    Geo<T> G = geo_of<T>(h);
+    T *fn = static_cast<T *>(h->fn), *out = static_cast<T *>(h->s0);
+    const auto &F = h->fv;
+    const FvItems W{F.d_hdr, F.d_halo, F.d_ovf, F.d_adj, F.d_cut, F.d_ghost, h->d_err, h->wait_first};
+    launch(h, K_EULER, "euler", [&] {
+        launch_dep(stats ? k_fused_fv<T, 4, true, IT> : k_fused_fv<T, 4, false, IT>, dim3(static_cast<unsigned>(F.nitem)),
+                   dim3(FvShape<IT>::nt), FvSmem<T, IT>::bytes, h->stream, fn, out, fn, static_cast<T *>(h->bacc),
+                   static_cast<T *>(h->cacc), static_cast<T *>(h->tau), static_cast<T *>(h->mac),
+                   stats ? h->d_partial : nullptr, G, W, static_cast<const T *>(F.geo), static_cast<const T *>(F.cutc),
+                   static_cast<const T *>(h->bnrm));
+    });
+    std::swap(h->fn, h->s0);
+    h->fn_parity ^= 1;
+}
+
 template <class T>
 void enqueue_fused_fv(fvlbm_handle *h, bool stats) {
     cudaStream_t s = h->stream;
-    fv_dispatch(h->fv.it, [&](auto it) { fv_stages<T, decltype(it)::value>(h, stats); });
+    fv_dispatch(h->fv.it, [&](auto it) {
+        if (h->scheme == 1)
+            fv_euler<T, decltype(it)::value>(h, stats);
+        else
+            fv_stages<T, decltype(it)::value>(h, stats);
+    });
     if (stats)
         launch(h, K_REDUCE, "reduce", [&] {
             k_reduce_instances<<<h->ninst, kTile, 0, s>>>(h->d_partial, h->fv.d_inst_item0, h->d_inst_sums);
@@ -1851,7 +1881,7 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
                             if (h->nonorth)
                                 launch_dep(
                                     k_sst_update<T, true, true>, sg_grid, block, 0, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
-                            else
+                            else if constexpr (!std::is_same<T, double>::value)
                                 launch_dep(
                                     k_sst_update<T, true, false>, sg_grid, block, 0, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
                         });
@@ -1908,6 +1938,12 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
         }
         h->turb = n;
     }
+    if constexpr (kHasFused<T>) {
+        if (h->config == 3) {
+            enqueue_fused_fv<T>(h, stats);
+            return;
+        }
+    }
     if (h->scheme == 1) {  // explicit Euler: gradient, flux + collision into s0, copy back
         launch(h, K_GRAD, "grad_f", [&] { grad_f<T>(h, grid, block, s, fn, g, G); });
         if (stats) {
@@ -1924,12 +1960,6 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
         }
         cudaMemcpyAsync(fn, s0, sizeof(T) * kQ * static_cast<size_t>(h->np), cudaMemcpyDeviceToDevice, s);
         return;
-    }
-    if constexpr (kHasFused<T>) {
-        if (h->config == 3) {
-            enqueue_fused_fv<T>(h, stats);
-            return;
-        }
     }
     launch(h, K_STAGE1, "stage1", [&] { k_stage1<T><<<grid, block, 0, s>>>(fn, s0, tau, G); });
     launch(h, K_GRAD, "grad_f", [&] { grad_f<T>(h, grid, block, s, s0, g, G); });
@@ -1964,7 +1994,7 @@ void enqueue(fvlbm_handle *h, bool stats) {
 
 int launches_per_step(const fvlbm_handle *h) {
     if (h->sst && h->per_stage && h->scheme == 0) return 2 + 1 + 3 + 2 + 3 + 2 + 2;
-    return (h->sst ? 2 : 0) + (h->scheme == 1 ? 2 : (h->config != 2 ? 3 : 7));
+    return (h->sst ? 2 : 0) + (h->scheme == 1 ? (h->config == 3 ? 1 : 2) : (h->config != 2 ? 3 : 7));
 }
 
 // Capture `nsteps` plain steps into an executable graph.  A replay always starts from the
@@ -2224,6 +2254,8 @@ int build_fv_items_it(fvlbm_handle *h, const std::vector<int> &nbr, const std::v
     CK(cudaFuncSetAttribute(k_fused_fv<T, 2, false, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     CK(cudaFuncSetAttribute(k_fused_fv<T, 3, false, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     CK(cudaFuncSetAttribute(k_fused_fv<T, 3, true, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CK(cudaFuncSetAttribute(k_fused_fv<T, 4, false, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CK(cudaFuncSetAttribute(k_fused_fv<T, 4, true, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     h->fv.it = IT;
     h->fv.nitem = nitem;
     h->fv.n_split = n_split;
@@ -2429,7 +2461,7 @@ void free_all(fvlbm_handle *h) {
         cudaStreamDestroy(A.s_out);
         A.init = false;
     }
-    for (int k = 0; k < 2; ++k)
+    for (int k = 0; k < 4; ++k)
         if (h->graph[k]) cudaGraphExecDestroy(h->graph[k]);
     for (void *p : h->allocs) cudaFree(p);
     h->allocs.clear();
@@ -2485,7 +2517,7 @@ int create_impl(int n, const fvlbm_mesh *meshes, const fvlbm_bc *bcs, const fvlb
     for (int q = 0; q < n; ++q) periodic_inexact |= !(P[q]->periodic_gap <= 1e-12);
     h->kernel_path = params[0].kernel_path;
     if (h->kernel_path < 0 || h->kernel_path > 2) return FVLBM_ERR_BAD_PARAM;
-    h->fused = h->kernel_path != 1 && h->scheme == 0 && prec != FVLBM_FP64_TANGENT &&
+    h->fused = h->kernel_path != 1 && prec != FVLBM_FP64_TANGENT &&
                !h->limit_f && !h->per_stage && !periodic_inexact;
     h->ninst = n;
     int cell_off = 0, bface_off = 0;
@@ -2754,7 +2786,7 @@ int fvlbm_step(fvlbm_handle *h, int n_steps, fvlbm_stats *stats) {
     if (want_stats) --remaining;  // the last step runs un-captured with the reductions
     // graphs: an even number of steps keeps the ping-pong parity of SST runs
     while (remaining >= kGraphSteps) {
-        const int gi = h->sst ? h->turb : 0;
+        const int gi = (h->sst ? h->turb : 0) + 2 * h->fn_parity;
         if (!h->graph[gi]) {
             int rc = build_graph(h, kGraphSteps, &h->graph[gi]);
             if (rc) return rc;
@@ -3232,7 +3264,7 @@ int fvlbm_fv_items(fvlbm_handle *h, int *nitem, int *n_split, int *n_overflow) {
 int fvlbm_set_wait_limit(fvlbm_handle *h, long long polls) {
     if (!h || polls < 0) return FVLBM_ERR_BAD_PARAM;
     h->wait_first = polls;
-    for (int k = 0; k < 2; ++k)  // captured graphs bake the kernel arguments
+    for (int k = 0; k < 4; ++k)  // captured graphs bake the kernel arguments
         if (h->graph[k]) {
             cudaGraphExecDestroy(h->graph[k]);
             h->graph[k] = nullptr;
@@ -3476,7 +3508,7 @@ int fvlbm_autotune(fvlbm_handle *h, int trial_steps, int *chosen, double *ms_per
     cudaFree(snap);
     h->config = best_c;
     h->steps = steps0;
-    for (int k = 0; k < 2; ++k)  // captured graphs bake the old configuration
+    for (int k = 0; k < 4; ++k)  // captured graphs bake the old configuration
         if (h->graph[k]) {
             cudaGraphExecDestroy(h->graph[k]);
             h->graph[k] = nullptr;
