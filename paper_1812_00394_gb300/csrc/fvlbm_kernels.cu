@@ -1142,6 +1142,7 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
 }
 
 #include "fvlbm_sst64.cuh"
+#include "fvlbm_tangent.cuh"
 
 // ------------------------------------------------------------------ state I/O kernels
 template <class T>
@@ -1500,7 +1501,7 @@ struct fvlbm_handle {
     std::vector<int2> sst_runs;  // (first tile, tiles) of each contiguous run of SST instances
     int *d_all_map = nullptr;   // output position (all instances) -> internal cell
     int *d_all_inv = nullptr;   // internal cell -> output position (all instances), -1: padding
-    int *d_back = nullptr;      // FP64 handles: slot of each face at its neighbour [4 np] (adjoint)
+    int *d_back = nullptr;      // FP64 and tangent handles: slot of each face at its neighbour [4 np]
     size_t adj_budget = 0;      // device bytes the adjoint may keep stage values in (0: half the free)
     int total_nc = 0, total_nb = 0;
     struct FvSet {          // work items of the face-value fused kernel (config 3)
@@ -1547,6 +1548,12 @@ struct fvlbm_handle {
     void *dtc = nullptr;    // local time stepping: dt of each cell (NULL: every instance global)
     void *kk[2] = {nullptr, nullptr}, *ww[2] = {nullptr, nullptr}, *nut[2] = {nullptr, nullptr};
     void *sgrad = nullptr, *f1 = nullptr;
+    struct Tan {            // tangent handles on the face-value form (fvlbm_tangent.cuh)
+        Dual *A = nullptr;  // coefficients A_mk [16 np] at (4 m + k) np + i
+        Dual *brow = nullptr;  // boundary values [nbt][8]
+        Dual *fv2 = nullptr;    // the other members at ties [np][16] (NULL without ties)
+        int *d_bits = nullptr;  // outgoing bits and ties [np]
+    } tan;
     double *ddl = nullptr;  // FP64 face-value handles with SST: |n dl / A| / |d| per face slot [4 np]
     void *sst_rec8 = nullptr, *sst_rec2 = nullptr;  // fused path: packed SST records [np][8], [np][2]
     int turb = 0;  // which of the k/omega/nu_t ping-pong buffers is current
@@ -1834,6 +1841,43 @@ void sst_update_twopass(const fvlbm_handle *h, const T *mac, const T *kc, const 
     });
 }
 
+// The stages of a tangent handle on the face-value form.
+void enqueue_tangent(fvlbm_handle *h, bool stats) {
+    const Geo<Dual> G = geo_of<Dual>(h);
+    cudaStream_t s = h->stream;
+    Dual *fn = static_cast<Dual *>(h->fn), *s0 = static_cast<Dual *>(h->s0), *s1 = static_cast<Dual *>(h->s1);
+    Dual *B = static_cast<Dual *>(h->bacc), *C = static_cast<Dual *>(h->cacc), *fv = static_cast<Dual *>(h->grad);
+    Dual *tau = static_cast<Dual *>(h->tau), *mac = static_cast<Dual *>(h->mac), *br = h->tan.brow;
+    const Dual *bn = static_cast<const Dual *>(h->bnrm);
+    Dual *f2 = h->tan.fv2;
+    const int *bk = h->d_back, *bits = h->tan.d_bits;
+    const int g1 = h->np / kTanBlock, gf = 4 * h->np / (2 * kTanBlock);
+    auto face = [&](const Dual *rows) {
+        launch(h, K_GRAD, "grad_f", [&] { k_tan_face<<<gf, 2 * kTanBlock, 0, s>>>(rows, br, G, h->tan.A, bits, fv, f2); });
+    };
+    launch(h, K_STAGE1, "stage1", [&] { k_tan_relax<<<g1, kTanBlock, 0, s>>>(fn, tau, s0, br, G, bn); });
+    face(s0);
+    launch(h, K_FLUX1, "flux_stage1", [&] {
+        k_tan_flux<1, false><<<g1, kTanBlock, 0, s>>>(s0, s1, br, fv, f2, fn, B, C, tau, mac, nullptr, G, bk, bits, bn);
+    });
+    face(s1);
+    launch(h, K_FLUX2, "flux_stage2", [&] {
+        k_tan_flux<2, false><<<g1, kTanBlock, 0, s>>>(s1, s0, br, fv, f2, fn, B, C, tau, mac, nullptr, G, bk, bits, bn);
+    });
+    face(s0);
+    launch(h, K_FLUX3, "flux_stage3", [&] {
+        if (stats)
+            k_tan_flux<3, true><<<h->ntiles, kTile, 0, s>>>(s0, s1, br, fv, f2, fn, B, C, tau, mac, h->d_partial, G, bk,
+                                                            bits, bn);
+        else
+            k_tan_flux<3, false><<<g1, kTanBlock, 0, s>>>(s0, s1, br, fv, f2, fn, B, C, tau, mac, nullptr, G, bk, bits, bn);
+    });
+    if (stats)
+        launch(h, K_REDUCE, "reduce", [&] {
+            k_reduce_instances<<<h->ninst, kTile, 0, s>>>(h->d_partial, h->d_inst_tile0, h->d_inst_sums);
+        });
+}
+
 template <class T>
 void enqueue_step(fvlbm_handle *h, bool stats) {
     Geo<T> G = geo_of<T>(h);
@@ -1961,6 +2005,12 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
         cudaMemcpyAsync(fn, s0, sizeof(T) * kQ * static_cast<size_t>(h->np), cudaMemcpyDeviceToDevice, s);
         return;
     }
+    if constexpr (std::is_same<T, Dual>::value) {
+        if (h->tan.A) {
+            enqueue_tangent(h, stats);
+            return;
+        }
+    }
     launch(h, K_STAGE1, "stage1", [&] { k_stage1<T><<<grid, block, 0, s>>>(fn, s0, tau, G); });
     launch(h, K_GRAD, "grad_f", [&] { grad_f<T>(h, grid, block, s, s0, g, G); });
     launch(h, K_FLUX1, "flux_stage1", [&] {
@@ -2014,35 +2064,11 @@ int build_graph(fvlbm_handle *h, int nsteps, cudaGraphExec_t *out) {
     return FVLBM_OK;
 }
 
-// Cells per item of the face-value kernels for a handle of np padded cells.  64-cell items spread
-// a small mesh over the 152 SMs, as long as (in float) all of them are resident at once, five to
-// an SM; beyond that 256-cell items, whose halo is smaller for their size, take over.  Both sides
-// measured, us per step, 64 against 256 cells: float cavities of 5k cells 10.7 / 12.4, 40k
-// 13.1 / 16.1, 59k 19.7 / 17.0, 199k 45 / 30; SST airfoils 40k 22.2 / 25.9, 60k 28.5 / 26.1; double
-// cavities 5k 45 / 70, 50k 116 / 120, 99k 214 / 201; SST airfoils 50k 239 / 243, 100k 387 / 379.
-template <class T>
-int fv_item_cells(size_t np) {
-    return np <= (sizeof(T) == 4 ? 5 * 152 * 64 : 50000) ? 64 : 256;
-}
-
-// Work items of the face-value kernel: every block of IT cells whose rows (cells, ring-1 and
-// ring-2 halo, ghosts) and cut faces fit its shared memory (FvShape) is one item; a block that does
-// not fit is split into halves, and so on down to eighths.  Per item: the ring lists, the
-// adjacency words of its cells, the cut faces (interior faces between an item cell and a
-// ring cell: the ring cell's row, the rows of its face data, its coefficients and outgoing
-// bits) and the ghosts (boundary faces of item and ring-1 cells).  Which member of each
-// direction pair leaves the cell through a face is decided once per face from the FP64 normal
-// of one side (e_alpha . n >= 0, the upwind rule of Eq. (advection)) and complemented on the
-// other side, so that both sides always agree.  The ring lists sit at a fixed stride per item
-// (FvItems).  The set is left unusable (ok = false) if an eighth of a block still does not fit.
-template <class T, int IT>
-int build_fv_items_it(fvlbm_handle *h, const std::vector<int> &nbr, const std::vector<int> &back,
-                      const std::vector<double> &sn, const std::vector<double> &lsq,
-                      const std::vector<double> &rown, const std::vector<double> &gq, const std::vector<int> &bowner,
-                      const std::vector<int> &inst_tile0) {
-    using S = FvShape<IT>;
-    const size_t np = h->np;
-    // outgoing bits of every (cell, face slot)
+// Outgoing bits of every (cell, face slot) at [m * np + cell]: bit p set when the first member of
+// direction pair p leaves the cell through the face, decided once per face from the FP64 normal of
+// one side (e_alpha . n >= 0, the upwind rule of Eq. (advection)) and complemented on the other.
+std::vector<unsigned char> outgoing_bits(size_t np, const std::vector<int> &nbr, const std::vector<int> &back,
+                                         const std::vector<double> &sn) {
     std::vector<unsigned char> pbits(4 * np, 0);
     for (size_t g = 0; g < np; ++g)
         for (int m = 0; m < 4; ++m) {
@@ -2060,6 +2086,35 @@ int build_fv_items_it(fvlbm_handle *h, const std::vector<int> &nbr, const std::v
             }
             pbits[m * np + g] = static_cast<unsigned char>(owner ? bits : (~bits & 15u));
         }
+    return pbits;
+}
+
+// Cells per item of the face-value kernels for a handle of np padded cells.  64-cell items spread
+// a small mesh over the 152 SMs, as long as (in float) all of them are resident at once, five to
+// an SM; beyond that 256-cell items, whose halo is smaller for their size, take over.  Both sides
+// measured, us per step, 64 against 256 cells: float cavities of 5k cells 10.7 / 12.4, 40k
+// 13.1 / 16.1, 59k 19.7 / 17.0, 199k 45 / 30; SST airfoils 40k 22.2 / 25.9, 60k 28.5 / 26.1; double
+// cavities 5k 45 / 70, 50k 116 / 120, 99k 214 / 201; SST airfoils 50k 239 / 243, 100k 387 / 379.
+template <class T>
+int fv_item_cells(size_t np) {
+    return np <= (sizeof(T) == 4 ? 5 * 152 * 64 : 50000) ? 64 : 256;
+}
+
+// Work items of the face-value kernel: every block of IT cells whose rows (cells, ring-1 and
+// ring-2 halo, ghosts) and cut faces fit its shared memory (FvShape) is one item; a block that does
+// not fit is split into halves, and so on down to eighths.  Per item: the ring lists, the
+// adjacency words of its cells, the cut faces (interior faces between an item cell and a
+// ring cell: the ring cell's row, the rows of its face data, its coefficients and outgoing
+// bits) and the ghosts (boundary faces of item and ring-1 cells).  The ring lists sit at a fixed
+// stride per item (FvItems).  The set is left unusable (ok = false) if an eighth of a block still does not fit.
+template <class T, int IT>
+int build_fv_items_it(fvlbm_handle *h, const std::vector<int> &nbr, const std::vector<int> &back,
+                      const std::vector<double> &sn, const std::vector<double> &lsq,
+                      const std::vector<double> &rown, const std::vector<double> &gq, const std::vector<int> &bowner,
+                      const std::vector<int> &inst_tile0) {
+    using S = FvShape<IT>;
+    const size_t np = h->np;
+    const std::vector<unsigned char> pbits = outgoing_bits(np, nbr, back, sn);
     // A_mk = W_k . r_m of cell g
     auto coef = [&](size_t g, int m, int k) {
         return lsq[(2 * k) * np + g] * rown[(2 * m) * np + g] + lsq[(2 * k + 1) * np + g] * rown[(2 * m + 1) * np + g];
@@ -2387,8 +2442,40 @@ int allocate_state(fvlbm_handle *h, const std::vector<const Prepared *> &P,
     if ((rc = upload_as<T>(h, &h->bval, bval))) return rc;
     if ((rc = upload_as<T>(h, &h->bnrm, bnrm))) return rc;
     if ((rc = upload_as<T>(h, &h->blen, blen))) return rc;
-    if (std::is_same<T, double>::value)
+    if (!std::is_same<T, float>::value)
         if ((rc = upload_raw(h, &h->d_back, back))) return rc;
+    if constexpr (std::is_same<T, Dual>::value) {
+        if (h->scheme == 0 && !h->limit_f && !h->per_stage) {
+            const std::vector<unsigned char> pb = outgoing_bits(np, nbr, back, sn);
+            bool ties = false;
+            std::vector<int> bits(np);
+            std::vector<double> A(16 * np, 0.0);
+            for (size_t k = 0; k < np; ++k)
+                for (int m = 0; m < 4; ++m) {
+                    bits[k] |= pb[m * np + k] << (4 * m);
+                    const int v = nbr[m * np + k];
+                    for (int p = 0; p < 4 && v >= 0; ++p) {  // e . n exactly 0 as seen from either side
+                        auto en = [&](size_t g, int f) {
+                            const double x = sn[(2 * f) * np + g], y = sn[(2 * f + 1) * np + g];
+                            return p == 0 ? x : (p == 1 ? y : (p == 2 ? x + y : y - x));
+                        };
+                        if (en(k, m) == 0.0 || en(v, back[m * np + k]) == 0.0) {
+                            bits[k] |= 1 << (16 + 4 * m + p);
+                            ties = true;
+                        }
+                    }
+                    for (int c = 0; c < 4; ++c)
+                        if (nbr[m * np + k] != kNone && nbr[c * np + k] != kNone)
+                            A[(4 * m + c) * np + k] = lsq[(2 * c) * np + k] * rown[(2 * m) * np + k] +
+                                                      lsq[(2 * c + 1) * np + k] * rown[(2 * m + 1) * np + k];
+                }
+            if (ties && (rc = dalloc(h, reinterpret_cast<void **>(&h->tan.fv2), 16 * np * sizeof(Dual)))) return rc;
+            if ((rc = upload_raw(h, &h->tan.d_bits, bits))) return rc;
+            if ((rc = upload_as<Dual>(h, reinterpret_cast<void **>(&h->tan.A), A))) return rc;
+            if ((rc = dalloc(h, reinterpret_cast<void **>(&h->tan.brow), 8 * sizeof(Dual) * std::max(h->nbt, 1))))
+                return rc;
+        }
+    }
     bool any_local = false;
     for (const Prepared *p : P) any_local |= !p->dt_cell.empty();
     if (any_local) {  // local time stepping: every cell's step (global instances: their dt)
@@ -3363,6 +3450,13 @@ int fvlbm_tangent_seed_nodes(fvlbm_handle *h, int instance, const double *dxy) {
     e = e ? e : put(h->wdist, 1, np, co, pn, [&](int, size_t k) { return D.wdist[k]; });
     e = e ? e : put(h->bnrm, 2, nbt, bo, nb, [&](int c, size_t f) { return D.bnrm[2 * f + c]; });
     e = e ? e : put(h->blen, 1, nbt, bo, nb, [&](int, size_t f) { return D.blen[f]; });
+    if (h->tan.A)  // A_mk = W_k . r_m
+        e = e ? e : put(h->tan.A, 16, np, co, pn, [&](int c, size_t k) {
+            const int m = c / 4, q = c % 4;
+            if (D.nbr[m * pn + k] == kNone || D.nbr[q * pn + k] == kNone) return Dual();
+            return D.lsq[(2 * q) * pn + k] * D.rown[(2 * m) * pn + k] +
+                   D.lsq[(2 * q + 1) * pn + k] * D.rown[(2 * m + 1) * pn + k];
+        });
     return e;
 }
 
