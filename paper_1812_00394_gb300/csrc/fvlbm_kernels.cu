@@ -1554,7 +1554,7 @@ struct fvlbm_handle {
         Dual *fv2 = nullptr;    // the other members at ties [np][16] (NULL without ties)
         int *d_bits = nullptr;  // outgoing bits and ties [np]
     } tan;
-    double *ddl = nullptr;  // FP64 face-value handles with SST: |n dl / A| / |d| per face slot [4 np]
+    void *ddl = nullptr;  // FP64 face-value and tangent handles with SST: |n dl / A| / |d| per face slot [4 np]
     void *sst_rec8 = nullptr, *sst_rec2 = nullptr;  // fused path: packed SST records [np][8], [np][2]
     int turb = 0;  // which of the k/omega/nu_t ping-pong buffers is current
     double *d_partial = nullptr, *d_inst_sums = nullptr, *d_io = nullptr;
@@ -1841,6 +1841,26 @@ void sst_update_twopass(const fvlbm_handle *h, const T *mac, const T *kc, const 
     });
 }
 
+// The SST step in double or for tangents (fvlbm_sst64.cuh).
+template <class S>
+void sst64(fvlbm_handle *h, const Geo<S> &G, cudaStream_t s, const S *mac, const S *kc, const S *wc, const S *nc, S *sg,
+           S *f1, S *kn, S *wn, S *nn, S *tau) {
+    S *r8 = static_cast<S *>(h->sst_rec8), *r2 = static_cast<S *>(h->sst_rec2);
+    const S *ddl = static_cast<const S *>(h->ddl);
+    launch(h, K_SST_GRAD, "sst_grad", [&] {
+        for_sst_runs(h, [&](dim3 g, int t0) {
+            launch_dep(k_sst_grad64<S>, dim3(g.x * (kTile / kSst64Block)), kSst64Block, 0, s, mac, kc, wc, nc, sg, f1, r8,
+                       r2, G, t0 * kTile);
+        });
+    });
+    launch(h, K_SST_UPDATE, "sst_update", [&] {
+        for_sst_runs(h, [&](dim3 g, int t0) {
+            launch_dep(k_sst_update64<S>, dim3(g.x * (kTile / kSst64Block)), kSst64Block, 0, s, nc, sg, f1, r8, r2, kn,
+                       wn, nn, tau, G, ddl, t0 * kTile);
+        });
+    });
+}
+
 // The stages of a tangent handle on the face-value form.
 void enqueue_tangent(fvlbm_handle *h, bool stats) {
     const Geo<Dual> G = geo_of<Dual>(h);
@@ -1898,20 +1918,7 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
             if (h->config != 2) {  // compact geometry, packed records
                 T *r8 = static_cast<T *>(h->sst_rec8), *r2 = static_cast<T *>(h->sst_rec2);
                 if constexpr (std::is_same<T, double>::value) {
-                    if (!h->nonorth) {
-                        launch(h, K_SST_GRAD, "sst_grad", [&] {
-                            for_sst_runs(h, [&](dim3 g, int t0) {
-                                launch_dep(k_sst_grad64, dim3(g.x * (kTile / kSst64Block)), kSst64Block, 0, s, mac, kc, wc,
-                                           nc, sg, f1, r8, r2, G, t0 * kTile);
-                            });
-                        });
-                        launch(h, K_SST_UPDATE, "sst_update", [&] {
-                            for_sst_runs(h, [&](dim3 g, int t0) {
-                                launch_dep(k_sst_update64, dim3(g.x * (kTile / kSst64Block)), kSst64Block, 0, s, nc, sg, f1,
-                                           r8, r2, kn, wn, nn, tau, G, static_cast<const double *>(h->ddl), t0 * kTile);
-                            });
-                        });
-                    }
+                    if (!h->nonorth) sst64(h, G, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau);
                 }
                 if (!std::is_same<T, double>::value || h->nonorth) {
                     launch(h, K_SST_GRAD, "sst_grad", [&] {
@@ -1933,7 +1940,14 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
                 }
             }
         }
-        if (h->config == 2) {
+        bool lean = false;  // tangents on the face-value form
+        if constexpr (std::is_same<T, Dual>::value) {
+            if (h->tan.A && !h->nonorth) {
+                sst64(h, G, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau);
+                lean = true;
+            }
+        }
+        if (h->config == 2 && !lean) {
             launch(h, K_SST_GRAD, "sst_grad", [&] { sst_grad_twopass<T>(h, mac, kc, wc, sg, f1, G, CG); });
             launch(h, K_SST_UPDATE, "sst_update", [&] {
                 sst_update_twopass<T>(h, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG);
@@ -2444,6 +2458,13 @@ int allocate_state(fvlbm_handle *h, const std::vector<const Prepared *> &P,
     if ((rc = upload_as<T>(h, &h->blen, blen))) return rc;
     if (!std::is_same<T, float>::value)
         if ((rc = upload_raw(h, &h->d_back, back))) return rc;
+    if (!std::is_same<T, float>::value && h->sst) {
+        std::vector<double> ddl(4 * np);
+        for (int m = 0; m < 4; ++m)
+            for (size_t k = 0; k < np; ++k)
+                ddl[m * np + k] = std::hypot(sn[(2 * m) * np + k], sn[(2 * m + 1) * np + k]) * dinv[m * np + k];
+        if ((rc = upload_as<T>(h, &h->ddl, ddl))) return rc;
+    }
     if constexpr (std::is_same<T, Dual>::value) {
         if (h->scheme == 0 && !h->limit_f && !h->per_stage) {
             const std::vector<unsigned char> pb = outgoing_bits(np, nbr, back, sn);
@@ -2496,13 +2517,6 @@ int allocate_state(fvlbm_handle *h, const std::vector<const Prepared *> &P,
         if (h->fused) {
             if ((rc = build_fv_items<T>(h, nbr, back, sn, lsq, rown, gq, bowner, inst_tile0))) return rc;
             if (h->fv.ok) h->config = 3;
-            if (std::is_same<T, double>::value && h->fv.ok && h->sst) {
-                std::vector<double> ddl(4 * np);
-                for (int m = 0; m < 4; ++m)
-                    for (size_t k = 0; k < np; ++k)
-                        ddl[m * np + k] = std::hypot(sn[(2 * m) * np + k], sn[(2 * m + 1) * np + k]) * dinv[m * np + k];
-                if ((rc = upload_raw(h, &h->ddl, ddl))) return rc;
-            }
             if (h->config == 2) h->fused = false;
         }
     }
@@ -3450,6 +3464,11 @@ int fvlbm_tangent_seed_nodes(fvlbm_handle *h, int instance, const double *dxy) {
     e = e ? e : put(h->wdist, 1, np, co, pn, [&](int, size_t k) { return D.wdist[k]; });
     e = e ? e : put(h->bnrm, 2, nbt, bo, nb, [&](int c, size_t f) { return D.bnrm[2 * f + c]; });
     e = e ? e : put(h->blen, 1, nbt, bo, nb, [&](int, size_t f) { return D.blen[f]; });
+    if (h->ddl)
+        e = e ? e : put(h->ddl, 4, np, co, pn, [&](int c, size_t k) {
+            const Dual x = D.sn[(2 * c) * pn + k], y = D.sn[(2 * c + 1) * pn + k];
+            return sqrt(x * x + y * y) * D.dinv[c * pn + k];
+        });
     if (h->tan.A)  // A_mk = W_k . r_m
         e = e ? e : put(h->tan.A, 16, np, co, pn, [&](int c, size_t k) {
             const int m = c / 4, q = c % 4;
