@@ -7,7 +7,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <unordered_map>
 
 #include "fvlbm_internal.h"
 
@@ -22,6 +21,37 @@ inline uint64_t edge_id(int a, int b) {
     uint32_t lo = static_cast<uint32_t>(std::min(a, b)), hi = static_cast<uint32_t>(std::max(a, b));
     return (static_cast<uint64_t>(lo) << 32) | hi;
 }
+
+// Sides of mesh edges by edge id, open addressing: one array access an edge where a node-based map
+// took a third of the preprocessing.
+class EdgeTable {
+public:
+    explicit EdgeTable(size_t sides) {
+        size_t cap = 16;
+        while (cap < 2 * sides) cap *= 2;
+        key_.assign(cap, kFree);
+        side_.resize(cap);
+    }
+    Side *find(uint64_t id) {
+        const size_t h = slot(id);
+        return key_[h] == kFree ? nullptr : &side_[h];
+    }
+    void insert(uint64_t id, Side s) {
+        const size_t h = slot(id);
+        key_[h] = id;
+        side_[h] = s;
+    }
+
+private:
+    static constexpr uint64_t kFree = ~0ull;
+    size_t slot(uint64_t id) const {
+        size_t h = static_cast<size_t>((id * 0x9E3779B97F4A7C15ull) >> 20) & (key_.size() - 1);
+        while (key_[h] != kFree && key_[h] != id) h = (h + 1) & (key_.size() - 1);
+        return h;
+    }
+    std::vector<uint64_t> key_;
+    std::vector<Side> side_;
+};
 
 // Position of (x, y) along a Hilbert curve over a 2^32 x 2^32 grid (iterative quadrant
 // descent with the curve's reflections).  Consecutive keys are face neighbours on the grid, so
@@ -86,8 +116,7 @@ int prepare_instance_t(const fvlbm_mesh &m, const fvlbm_bc &bc, const fvlbm_para
     }
     std::vector<S> cx(nc), cy(nc), area(nc);
     std::vector<FaceGeo<S>> face(static_cast<size_t>(nc) * 4);
-    std::unordered_map<uint64_t, Side> open;
-    open.reserve(static_cast<size_t>(nc) * 3);
+    EdgeTable open(4 * static_cast<size_t>(nc));
     for (int i = 0; i < nc; ++i) {
         const int p0 = m.cell_ptr[i], nv = m.cell_ptr[i + 1] - p0;
         if (nv < 3 || nv > 4) {
@@ -131,20 +160,20 @@ int prepare_instance_t(const fvlbm_mesh &m, const fvlbm_bc &bc, const fvlbm_para
             F.xm = S(0.5) * (xy[2 * a] + xy[2 * b]);
             F.ym = S(0.5) * (xy[2 * a + 1] + xy[2 * b + 1]);
             const uint64_t id = edge_id(a, b);
-            auto it = open.find(id);
-            if (it == open.end()) {
-                open.emplace(id, Side{i, l});
+            Side *it = open.find(id);
+            if (it == nullptr) {
+                open.insert(id, Side{i, l});
             } else {
-                if (it->second.cell < 0) {
+                if (it->cell < 0) {
                     *why = "edge shared by more than two cells";
                     return FVLBM_ERR_BAD_MESH;
                 }
-                FaceGeo<S> &G = face[4 * static_cast<size_t>(it->second.cell) + it->second.local];
-                F.nbr = it->second.cell;
-                F.back = it->second.local;
+                FaceGeo<S> &G = face[4 * static_cast<size_t>(it->cell) + it->local];
+                F.nbr = it->cell;
+                F.back = it->local;
                 G.nbr = i;
                 G.back = l;
-                it->second.cell = -1;  // closed
+                it->cell = -1;  // closed
             }
         }
     }
@@ -153,8 +182,8 @@ int prepare_instance_t(const fvlbm_mesh &m, const fvlbm_bc &bc, const fvlbm_para
     std::vector<Side> bside(nbe);
     for (int b = 0; b < nbe; ++b) {
         const int a0 = bc.bedge_nodes[2 * b], a1 = bc.bedge_nodes[2 * b + 1];
-        auto it = open.find(edge_id(a0, a1));
-        if (it == open.end() || it->second.cell < 0) {
+        Side *it = open.find(edge_id(a0, a1));
+        if (it == nullptr || it->cell < 0) {
             *why = "boundary edge " + std::to_string(b) + " is not a boundary edge of the mesh";
             return FVLBM_ERR_BAD_BC;
         }
@@ -163,8 +192,8 @@ int prepare_instance_t(const fvlbm_mesh &m, const fvlbm_bc &bc, const fvlbm_para
             *why = "unknown boundary type";
             return FVLBM_ERR_BAD_BC;
         }
-        bside[b] = it->second;
-        face[4 * static_cast<size_t>(it->second.cell) + it->second.local].nbr = -(b + 1);
+        bside[b] = *it;
+        face[4 * static_cast<size_t>(it->cell) + it->local].nbr = -(b + 1);
     }
     std::vector<char> glued(nbe, 0);
     double gap = 0.0;  // largest mismatch of a glued pair (side B's own edge against side A's)
@@ -517,38 +546,28 @@ int geometry_adjoint(const fvlbm_mesh &m, const fvlbm_bc &bc, const GeometryAdjo
         return FVLBM_ERR_NOT_SUPPORTED;
     }
     // face neighbours (input ids) and boundary edges of every face slot
-    // (an open-addressing table of edges: a node-based map took a tenth of the call)
     std::vector<int> nbr(4 * static_cast<size_t>(nc), kNone);
-    size_t cap = 16;
-    while (cap < 2 * static_cast<size_t>(m.cell_ptr[nc])) cap *= 2;
-    std::vector<uint64_t> key(cap, ~0ull);
-    std::vector<int> side(cap);  // 4 cell + face
-    auto slot_of = [&](uint64_t id) {
-        size_t h = static_cast<size_t>((id * 0x9E3779B97F4A7C15ull) >> 20) & (cap - 1);
-        while (key[h] != ~0ull && key[h] != id) h = (h + 1) & (cap - 1);
-        return h;
-    };
+    EdgeTable open(4 * static_cast<size_t>(nc));
     for (int i = 0; i < nc; ++i) {
         const int p0 = m.cell_ptr[i], nv = m.cell_ptr[i + 1] - p0;
         for (int l = 0; l < nv; ++l) {
             const uint64_t id = edge_id(m.cell_nodes[p0 + l], m.cell_nodes[p0 + (l + 1) % nv]);
-            const size_t h = slot_of(id);
-            if (key[h] == ~0ull) {
-                key[h] = id;
-                side[h] = 4 * i + l;
+            const Side *it = open.find(id);
+            if (it == nullptr) {
+                open.insert(id, Side{i, l});
             } else {
-                nbr[4 * static_cast<size_t>(i) + l] = side[h] / 4;
-                nbr[side[h]] = i;
+                nbr[4 * static_cast<size_t>(i) + l] = it->cell;
+                nbr[4 * static_cast<size_t>(it->cell) + it->local] = i;
             }
         }
     }
     for (int b = 0; b < bc.n_bedges; ++b) {
-        const size_t h = slot_of(edge_id(bc.bedge_nodes[2 * b], bc.bedge_nodes[2 * b + 1]));
-        if (key[h] == ~0ull) {
+        const Side *it = open.find(edge_id(bc.bedge_nodes[2 * b], bc.bedge_nodes[2 * b + 1]));
+        if (it == nullptr) {
             *why = "boundary edge not on the mesh";
             return FVLBM_ERR_BAD_BC;
         }
-        nbr[side[h]] = -(b + 1);
+        nbr[4 * static_cast<size_t>(it->cell) + it->local] = -(b + 1);
     }
     std::vector<double> cxv(nc), cyv(nc), dc(2 * static_cast<size_t>(nc), 0.0);
     for (int i = 0; i < nc; ++i) {
