@@ -19,7 +19,7 @@ LIB = os.path.join(BUILD, "libfvlbm.so")
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 SOURCES = ["fvlbm_host.cpp", "fvlbm_kernels.cu", "fvlbm_noalloc.cu", "fvlbm_peak.cu"]
 HEADERS = ["fvlbm_internal.h", "fvlbm_dual.h", "fvlbm_adjoint.cuh", "fvlbm_adjoint_sst.cuh",
-           "fvlbm_fused_fv.cuh", "fvlbm_sst64.cuh", "fvlbm_tangent.cuh"]
+           "fvlbm_fused_fv.cuh", "fvlbm_sst64.cuh", "fvlbm_lanes.cuh", "fvlbm_tangent.cuh"]
 
 
 def _nvcc() -> str:

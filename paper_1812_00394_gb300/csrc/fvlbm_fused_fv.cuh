@@ -406,11 +406,20 @@ __device__ __forceinline__ void fv_normals(const float *q, bool tri, float *sn) 
 // ---- double: the cell algebra on pairs.  With S = f + f-bar and D = f - f-bar of a pair the moments
 // are plain sums, and f^eq of a pair is w (s + a), w (s - a) with the parts even and odd in u:
 // about half the operations of the direction-by-direction form, which counts in double, where
-// every operation takes 64 times a float one on this GPU.
+// every operation takes 64 times a float one on this GPU.  Products that are added are written as
+// fused operations, so that every kernel that uses these functions rounds alike.
 template <class T>
 struct FvMoments {
     T dr, r, u, v, jx, jy, uu;  // uu = 1.5 (u^2 + v^2)
 };
+template <class T>
+__device__ __forceinline__ void fv_velocity(FvMoments<T> &M, T rho0) {
+    M.r = rho0 + M.dr;
+    const T ir = sdiv(T(1), M.r);
+    M.u = M.jx * ir;
+    M.v = M.jy * ir;
+    M.uu = T(1.5) * fma(M.u, M.u, M.v * M.v);
+}
 template <class T>
 __device__ __forceinline__ FvMoments<T> fv_moments(const typename FvPair<T>::V *f, T f0, T rho0) {
     FvMoments<T> M;
@@ -418,11 +427,7 @@ __device__ __forceinline__ FvMoments<T> fv_moments(const typename FvPair<T>::V *
     M.dr = f0 + (((f[0].x + f[0].y) + (f[1].x + f[1].y)) + ((f[2].x + f[2].y) + (f[3].x + f[3].y)));
     M.jx = (f[0].x - f[0].y) + (d2 - d3);
     M.jy = (f[1].x - f[1].y) + (d2 + d3);
-    M.r = rho0 + M.dr;
-    const T ir = sdiv(T(1), M.r);
-    M.u = M.jx * ir;
-    M.v = M.jy * ir;
-    M.uu = T(1.5) * (M.u * M.u + M.v * M.v);
+    fv_velocity(M, rho0);
     return M;
 }
 template <class T>
@@ -433,13 +438,13 @@ __device__ __forceinline__ T fv_w(int p) {
 template <class T>
 __device__ __forceinline__ typename FvPair<T>::V fv_feq(const FvMoments<T> &M, int p) {
     const T eu = fv_en<T>(p, M.u, M.v);
-    const T s = fv_w<T>(p) * (M.dr + M.r * (T(4.5) * eu * eu - M.uu));
-    const T a = (T(3) * fv_w<T>(p)) * fv_en<T>(p, M.jx, M.jy);
-    return FvPair<T>::make(s + a, s - a);
+    const T s = fv_w<T>(p) * fma(M.r, fma(T(4.5) * eu, eu, -M.uu), M.dr);
+    const T ej = fv_en<T>(p, M.jx, M.jy), w3 = p < 2 ? T(1.0 / 3.0) : T(1.0 / 12.0);
+    return FvPair<T>::make(fma(w3, ej, s), fma(-w3, ej, s));
 }
 template <class T>
 __device__ __forceinline__ T fv_feq0(const FvMoments<T> &M) {
-    return T(4.0 / 9.0) * (M.dr - M.r * M.uu);
+    return T(4.0 / 9.0) * fma(-M.r, M.uu, M.dr);
 }
 
 // Relaxation factors of an implicit collision with coefficient m: f = f^eq + a (X - f^eq) with
@@ -447,16 +452,49 @@ __device__ __forceinline__ T fv_feq0(const FvMoments<T> &M) {
 // division.  In this form rounding of a leaves the conserved moments alone.
 template <class T>
 __device__ __forceinline__ void fv_factors(T dt, T tau, T m, T &a, T &g) {
-    const T r = sdiv(T(1), tau + m * dt);
+    const T r = sdiv(T(1), fma(m, dt, tau));
     a = tau * r;
     g = dt * r;
 }
 
-// Boundary values f_{alpha,bc} (boundary_values, which states the readings) of a cell with
-// staged row fc, f0, as differences to the cell's own values: wall and inlet
+// Pair p of the boundary values f_{alpha,bc} (boundary_values, which states the readings) of a cell
+// with that pair f and moments M, as differences to the cell's own values: wall and inlet
 // f + f^eq(rho, u_b) - f^eq(rho, u), outlet f + f^eq(rho_b, u) - f^eq(rho, u), far field
-// f^eq(rho_b, u_b) where e . n < 0.  The face's type and values are read kept in L2, like the
-// item tables: a few hundred kB read once per launch by the items along the boundaries.
+// f^eq(rho_b, u_b) where e . n < 0.
+__device__ __forceinline__ double2 fv_ghost_pair(int type, double rb, double ub, double vb, double nx, double ny,
+                                                 const FvMoments<double> &M, double rho0, int p, double2 f) {
+    if (type == FVLBM_BC_FARFIELD) {
+        FvMoments<double> B;
+        B.dr = rb - rho0;
+        B.r = rb;
+        B.u = ub;
+        B.v = vb;
+        B.jx = rb * ub;
+        B.jy = rb * vb;
+        B.uu = 1.5 * ::fma(ub, ub, vb * vb);
+        const double en = fv_en<double>(p, nx, ny);
+        const double2 eq = fv_feq<double>(B, p);
+        return make_double2(en < 0.0 ? eq.x : f.x, en > 0.0 ? eq.y : f.y);
+    }
+    double s, a;
+    if (type == FVLBM_BC_OUTLET) {
+        const double q = (rb - rho0) - M.dr;  // rho_b - rho
+        const double eu = fv_en<double>(p, M.u, M.v);
+        s = ::fma(q, ::fma(4.5 * eu, eu, -M.uu), q);
+        a = 3.0 * q * eu;
+    } else {
+        const double du = ub - M.u, dv = vb - M.v, su = ub + M.u, sv = vb + M.v;
+        const double de = fv_en<double>(p, du, dv);
+        s = M.r * ::fma(4.5 * de, fv_en<double>(p, su, sv), -(1.5 * ::fma(du, su, dv * sv)));
+        a = 3.0 * M.r * de;
+    }
+    const double w = fv_w<double>(p);
+    return make_double2(::fma(w, s + a, f.x), ::fma(w, s - a, f.y));
+}
+
+// Boundary values of a cell with staged row fc, f0 at ghost gh.  The face's type and values are read
+// kept in L2, like the item tables: a few hundred kB read once per launch by the items along the
+// boundaries.
 template <class T>
 __device__ __forceinline__ void fv_ghost(const Geo<T> &G, const T *__restrict__ bnrm, const T *__restrict__ geo,
                                          const int4 &gh, T rho0, const typename FvPair<T>::V *fc, T f0,
@@ -487,44 +525,13 @@ __device__ __forceinline__ void fv_ghost(const Geo<T> &G, const T *__restrict__ 
         for (int p = 0; p < 4; ++p) out[p] = PV::make(fb[fv_first(p)], fb[fv_second(p)]);
         return;
     }
-    const T rb = ld_keep(G.bval + bf, keep), ub = ld_keep(G.bval + G.nbt + bf, keep),
-            vb = ld_keep(G.bval + 2 * static_cast<size_t>(G.nbt) + bf, keep);
-    if (type == FVLBM_BC_FARFIELD) {
+    if constexpr (sizeof(T) == 8) {
+        const T rb = ld_keep(G.bval + bf, keep), ub = ld_keep(G.bval + G.nbt + bf, keep),
+                vb = ld_keep(G.bval + 2 * static_cast<size_t>(G.nbt) + bf, keep);
         const T nx = ld_keep(bnrm + bf, keep), ny = ld_keep(bnrm + G.nbt + bf, keep);
-        FvMoments<T> B;
-        B.dr = rb - rho0;
-        B.r = rb;
-        B.u = ub;
-        B.v = vb;
-        B.jx = rb * ub;
-        B.jy = rb * vb;
-        B.uu = T(1.5) * (ub * ub + vb * vb);
+        const FvMoments<T> M = fv_moments<T>(fc, f0, rho0);
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            const T en = fv_en<T>(p, nx, ny);
-            const typename PV::V eq = fv_feq<T>(B, p);
-            out[p] = PV::make(en < T(0) ? eq.x : fc[p].x, en > T(0) ? eq.y : fc[p].y);
-        }
-        return;
-    }
-    const FvMoments<T> M = fv_moments<T>(fc, f0, rho0);
-    const bool outlet = type == FVLBM_BC_OUTLET;
-    const T q = (rb - rho0) - M.dr;                              // rho_b - rho
-    const T du = ub - M.u, dv = vb - M.v, su = ub + M.u, sv = vb + M.v;
-    const T duu = T(1.5) * (du * su + dv * sv);                  // change of uu
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        T s, a;
-        if (outlet) {
-            const T eu = fv_en<T>(p, M.u, M.v);
-            s = q * (T(1) + (T(4.5) * eu * eu - M.uu));
-            a = T(3) * q * eu;
-        } else {
-            const T de = fv_en<T>(p, du, dv);
-            s = M.r * (T(4.5) * de * fv_en<T>(p, su, sv) - duu);
-            a = T(3) * M.r * de;
-        }
-        out[p] = PV::make(fc[p].x + fv_w<T>(p) * (s + a), fc[p].y + fv_w<T>(p) * (s - a));
+        for (int p = 0; p < 4; ++p) out[p] = fv_ghost_pair(type, rb, ub, vb, nx, ny, M, rho0, p, fc[p]);
     }
 }
 
@@ -671,7 +678,6 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
     T *sacc = reinterpret_cast<T *>(smem_raw + L::sacc);
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem_raw + L::bar);
 
-    dep_launch();
     const int t = threadIdx.x;
     // Stage 2 walks the items backwards: what stage 1 wrote last (100 MB or so of a large batch) it
     // finds in L2, and stage 3 what stage 2 wrote last (sweep step 502 -> 494 us).
@@ -925,6 +931,8 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
 
     // 3. flux of item cell t (Eq. (advection)) from the published face values, then the stage
     //    algebra with the accumulator rows, tau and the parameters from shared memory
+    // (double: not released early, see dep_launch)
+    if (sizeof(T) == 4) dep_launch();
     double st[4] = {0.0, 0.0, 0.0, 0.0};
     if constexpr (sizeof(T) == 4) {
         if (mine) {

@@ -625,12 +625,16 @@ __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
-// Programmatic dependent launch of a step's kernels: a kernel lets its successor start as soon as
-// its own blocks have all started (dep_launch), and the successor reads nothing that a kernel
+// Programmatic dependent launch of a step's kernels: a float kernel lets its successor start when
+// its own blocks have their inputs (dep_launch), and the successor reads nothing that a kernel
 // writes before dep_wait, which returns when every earlier kernel has finished and its stores are
 // visible.  Until then it may read the tables and geometry fixed at create, so its launch, its
 // block start-up and those loads run beside the predecessor's last blocks.  (A kernel finishes
 // only after its own dep_wait, so a chain of early starts never overtakes a kernel two back.)
+// Released at entry instead, the successor's blocks take their places before the predecessor's
+// have left: 80k-cell SST step 25.6 us against 24.2.  In double that spread costs more than it
+// gives, since a scheduler with two warps takes twice as long (50k-cell airfoil 189 us against
+// 161, 64 x 64 cavity 61 against 34): the FP64 kernels only overlap the launch itself.
 // What a kernel writes is read through pointers that are not const __restrict__: such loads
 // may be taken for loop-invariant and moved above dep_wait.
 __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -955,7 +959,6 @@ __global__ void __launch_bounds__(kTile)
     k_sst_grad(const T *mac, const T *kk, const T *ww, T *__restrict__ grads, T *__restrict__ f1out, Geo<T> G,
                CompactGeo<T> CG, const T *nut, T *__restrict__ rec8, T *__restrict__ rec2, bool inv_only,
                int tile0) {
-    dep_launch();
     const int tile = tile0 + static_cast<int>(blockIdx.x);
     const int i = tile * kTile + threadIdx.x;
     const size_t np = G.np;
@@ -1010,6 +1013,7 @@ __global__ void __launch_bounds__(kTile)
                       q[m][3]);
         }
     }
+    dep_launch();
     T g[8], lg[4], f1;
     sst_cell_grad(own[2], own[3], di, nu, has, q, W, R, own, g, lg, f1);
     if (inv_only) {  // the update needs the invariants of the own gradient only
@@ -1042,7 +1046,6 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
     k_sst_update(const T *mac, const T *kk, const T *ww, const T *nut, const T *grads, const T *f1a,
                  T *__restrict__ k_out, T *__restrict__ w_out, T *__restrict__ nut_out, T *__restrict__ tau,
                  Geo<T> G, CompactGeo<T> CG, const T *rec8, const T *rec2, int tile0) {
-    dep_launch();
     // backwards: the records that k_sst_grad wrote last are still in L2
     const int tile = tile0 + static_cast<int>(gridDim.x - 1 - blockIdx.x);
     const int i = tile * kTile + threadIdx.x;
@@ -1131,6 +1134,7 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
             sst_bvals(G, -nb - 1, nu, ui, vi, ki, wi, di, f.u, f.v, f.k, f.w);
         }
     }
+    dep_launch();
     T kn, wn, ntn, tnew;
     const T dt_i = cell_dt(G, P, i);
     sst_cell_update<T, NONORTH>(P, dt_i, ui, vi, ki, wi, nti, di, g, SS, dv, kw, lgi, f1i, F, kn, wn, ntn,
@@ -1141,6 +1145,7 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
     tau[i] = tnew;
 }
 
+#include "fvlbm_lanes.cuh"
 #include "fvlbm_sst64.cuh"
 #include "fvlbm_tangent.cuh"
 
@@ -1554,6 +1559,11 @@ struct fvlbm_handle {
         Dual *fv2 = nullptr;    // the other members at ties [np][16] (NULL without ties)
         int *d_bits = nullptr;  // outgoing bits and ties [np]
     } tan;
+    struct Lanes {          // small FP64 handles: four threads per cell (fvlbm_lanes.cuh)
+        bool ok = false;
+        double *brow = nullptr;  // boundary values [nbt][8]
+        int *d_bits = nullptr;   // outgoing bits [np]
+    } lanes;
     void *ddl = nullptr;  // FP64 face-value and tangent handles with SST: |n dl / A| / |d| per face slot [4 np]
     void *sst_rec8 = nullptr, *sst_rec2 = nullptr;  // fused path: packed SST records [np][8], [np][2]
     int turb = 0;  // which of the k/omega/nu_t ping-pong buffers is current
@@ -1768,6 +1778,36 @@ auto fv_dispatch(int it, F &&f) {
     return f(std::integral_constant<int, 64>());
 }
 
+// The three stages with four threads per cell.
+void lane_stages(fvlbm_handle *h) {
+    const Geo<double> G = geo_of<double>(h);
+    cudaStream_t s = h->stream;
+    double *fn = static_cast<double *>(h->fn), *s0 = static_cast<double *>(h->s0), *s1 = static_cast<double *>(h->s1);
+    double *B = static_cast<double *>(h->bacc), *C = static_cast<double *>(h->cacc), *fv = static_cast<double *>(h->grad);
+    double *tau = static_cast<double *>(h->tau), *mac = static_cast<double *>(h->mac), *br = h->lanes.brow;
+    const double *geo = static_cast<const double *>(h->fv.geo), *bn = static_cast<const double *>(h->bnrm);
+    const int *bk = h->d_back, *bits = h->lanes.d_bits;
+    const dim3 g(4 * h->np / kLaneBlock), b(kLaneBlock);
+    auto face = [&](const double *rows) {
+        launch(h, K_GRAD, "lane_face", [&] { launch_dep(k_lane_face, g, b, 0, s, rows, br, fv, G, geo, bits, bn); });
+    };
+    launch(h, K_STAGE1, "lane_relax", [&] { launch_dep(k_lane_relax, g, b, 0, s, fn, tau, s0, B, G); });
+    face(s0);
+    launch(h, K_FLUX1, "lane_flux1", [&] {
+        launch_dep(k_lane_flux<1>, g, b, 0, s, s0, br, fv, s1, fn, B, C, tau, mac, G, geo, bk, bits);
+    });
+    face(s1);
+    launch(h, K_FLUX2, "lane_flux2", [&] {
+        launch_dep(k_lane_flux<2>, g, b, 0, s, s1, br, fv, s0, fn, B, C, tau, mac, G, geo, bk, bits);
+    });
+    face(s0);
+    launch(h, K_FLUX3, "lane_flux3", [&] {
+        launch_dep(k_lane_flux<3>, g, b, 0, s, s0, br, fv, s1, fn, B, C, tau, mac, G, geo, bk, bits);
+    });
+}
+// The lane kernels have no staging wait: a handle whose wait is limited runs the fused ones.
+bool use_lanes(const fvlbm_handle *h) { return h->lanes.ok && h->config == 3 && h->wait_first == kWaitLimit; }
+
 // The explicit Euler step in the same form: f^n into the other buffer, which becomes f^n.
 template <class T, int IT>
 void fv_euler(fvlbm_handle *h, bool stats) {
@@ -1790,7 +1830,9 @@ template <class T>
 void enqueue_fused_fv(fvlbm_handle *h, bool stats) {
     cudaStream_t s = h->stream;
     fv_dispatch(h->fv.it, [&](auto it) {
-        if (h->scheme == 1)
+        if (std::is_same<T, double>::value && h->scheme == 0 && !stats && use_lanes(h))
+            lane_stages(h);
+        else if (h->scheme == 1)
             fv_euler<T, decltype(it)::value>(h, stats);
         else
             fv_stages<T, decltype(it)::value>(h, stats);
@@ -2058,7 +2100,7 @@ void enqueue(fvlbm_handle *h, bool stats) {
 
 int launches_per_step(const fvlbm_handle *h) {
     if (h->sst && h->per_stage && h->scheme == 0) return 2 + 1 + 3 + 2 + 3 + 2 + 2;
-    return (h->sst ? 2 : 0) + (h->scheme == 1 ? (h->config == 3 ? 1 : 2) : (h->config != 2 ? 3 : 7));
+    return (h->sst ? 2 : 0) + (h->scheme == 0 && use_lanes(h) ? 7 : h->scheme == 1 ? (h->config == 3 ? 1 : 2) : (h->config != 2 ? 3 : 7));
 }
 
 // Capture `nsteps` plain steps into an executable graph.  A replay always starts from the
@@ -2109,6 +2151,8 @@ std::vector<unsigned char> outgoing_bits(size_t np, const std::vector<int> &nbr,
 // measured, us per step, 64 against 256 cells: float cavities of 5k cells 10.7 / 12.4, 40k
 // 13.1 / 16.1, 59k 19.7 / 17.0, 199k 45 / 30; SST airfoils 40k 22.2 / 25.9, 60k 28.5 / 26.1; double
 // cavities 5k 45 / 70, 50k 116 / 120, 99k 214 / 201; SST airfoils 50k 239 / 243, 100k 387 / 379.
+// Padded cells up to which FP64 handles take four threads per cell (fvlbm_lanes.cuh has both sides).
+constexpr size_t kLaneCells = 24576;
 template <class T>
 int fv_item_cells(size_t np) {
     return np <= (sizeof(T) == 4 ? 5 * 152 * 64 : 50000) ? 64 : 256;
@@ -2517,6 +2561,16 @@ int allocate_state(fvlbm_handle *h, const std::vector<const Prepared *> &P,
         if (h->fused) {
             if ((rc = build_fv_items<T>(h, nbr, back, sn, lsq, rown, gq, bowner, inst_tile0))) return rc;
             if (h->fv.ok) h->config = 3;
+            if (std::is_same<T, double>::value && h->fv.ok && h->scheme == 0 && np <= kLaneCells) {
+                const std::vector<unsigned char> pb = outgoing_bits(np, nbr, back, sn);
+                std::vector<int> bits(np);
+                for (size_t k = 0; k < np; ++k)
+                    for (int m = 0; m < 4; ++m) bits[k] |= pb[m * np + k] << (4 * m);
+                if ((rc = upload_raw(h, &h->lanes.d_bits, bits))) return rc;
+                if ((rc = dalloc(h, reinterpret_cast<void **>(&h->lanes.brow), 8 * sizeof(double) * std::max(h->nbt, 1))))
+                    return rc;
+                h->lanes.ok = true;
+            }
             if (h->config == 2) h->fused = false;
         }
     }

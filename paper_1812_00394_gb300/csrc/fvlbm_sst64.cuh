@@ -18,9 +18,9 @@
 //     read by its neighbours in place of (f1, nu_t).
 // Measured on 473k SST cells (with the generic kernels before): gradient 154 us (354),
 // update 164 us (397).
-// Both are bound by the FP64 pipe, one thread per cell, in blocks of 64 so that a mesh of 50k cells
+// Both are bound by the FP64 pipe, one thread per cell, one warp a block so that a mesh of 50k cells
 // still spreads evenly over 608 schedulers.
-constexpr int kSst64Block = 64;
+constexpr int kSst64Block = 32;
 
 // ---- arithmetic of doubles and Duals, the derivatives that are zero left out
 __device__ __forceinline__ Dual mad(const Dual &a, const Dual &b, const Dual &c) {
@@ -134,7 +134,6 @@ template <class S>
 __global__ void __launch_bounds__(kSst64Block)
     k_sst_grad64(const S *mac, const S *kk, const S *ww, const S *nut, S *__restrict__ grads, S *__restrict__ f1out,
                  S *__restrict__ rec8, S *__restrict__ rec2, Geo<S> G, int i0) {
-    dep_launch();
     const int i = i0 + static_cast<int>(blockIdx.x) * kSst64Block + threadIdx.x;
     const size_t np = G.np;
     const double nu = G.ip[G.tile_inst[i / kTile]].nu;
@@ -217,7 +216,6 @@ __global__ void __launch_bounds__(kSst64Block)
     k_sst_update64(const S *nut, const S *grads, const S *f1a, const S *rec8, const S *rec2, S *__restrict__ k_out,
                    S *__restrict__ w_out, S *__restrict__ nut_out, S *__restrict__ tau, Geo<S> G,
                    const S *__restrict__ ddl, int i0) {
-    dep_launch();
     // backwards: the records that k_sst_grad64 wrote last are still in L2
     const int i = i0 + static_cast<int>(gridDim.x - 1 - blockIdx.x) * kSst64Block + threadIdx.x;
     const size_t np = G.np;

@@ -16,7 +16,7 @@
 //   k_tan_flux<STAGE>  one thread per cell: flux, stage algebra, boundary values of the new stage
 // and k_tan_relax before them (f^(1) and its boundary values).  Measured on two 20k-cell SST
 // airfoils: the stages took 694 us a step in the generic kernels, 248 here.
-constexpr int kTanBlock = 64;
+constexpr int kTanBlock = 32;
 
 // e_first(p) . (x, y)
 __device__ __forceinline__ Dual tan_en(int p, const Dual &x, const Dual &y) {
