@@ -1150,6 +1150,19 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
 #include "fvlbm_tangent.cuh"
 
 // ------------------------------------------------------------------ state I/O kernels
+// Records of N values per cell pass between the caller's order and the kernels' arrays through
+// shared memory, kIoBlock records at a time, so that the records are read and written as whole
+// cache lines: a thread that walks its own record touches a line per value (a 36-byte record: nine
+// times the transactions).  Gathering 640k FP32 records took 31.5 us that way, 14.2 now; packing
+// 200k cells for an exchange 16.6 and 13.9.
+constexpr int kIoBlock = 128;
+template <class V, int N>
+__device__ __forceinline__ void io_put(const V *sm, V *__restrict__ out, int j0, int n) {
+    __syncthreads();
+    const int m = min(n - j0, kIoBlock) * N;
+    for (int e = threadIdx.x; e < m; e += kIoBlock) out[static_cast<size_t>(j0) * N + e] = sm[e];
+}
+
 template <class T>
 __global__ void k_init_state(T *__restrict__ fn, T *__restrict__ mac, const double *__restrict__ r0,
                              const double *__restrict__ u0, const double *__restrict__ v0,
@@ -1167,19 +1180,6 @@ __global__ void k_init_state(T *__restrict__ fn, T *__restrict__ mac, const doub
     mac[i] = rr;
     mac[np + i] = uu;
     mac[2 * np + i] = vv;
-}
-
-// out[perm[k] * 9 + a] = f[a][off + k] + w_a rho0   (k < nc)
-template <class T>
-__global__ void k_gather_f(const T *__restrict__ f, const int *__restrict__ perm, int off, int nc,
-                           double rho0, size_t np, double *__restrict__ out) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nc) return;
-    const int dst = perm[k];
-    for (int a = 0; a < kQ; ++a) {
-        const double wa = a == 0 ? 4.0 / 9.0 : (a < 5 ? 1.0 / 9.0 : 1.0 / 36.0);
-        out[static_cast<size_t>(dst) * kQ + a] = double(f[a * np + off + k]) + wa * rho0;
-    }
 }
 
 // Per wall face momentum flux and Cp (FP64): out[5][nb_inst] = fx, fy, cp, dfx/dp, dfy/dp (the
@@ -1220,20 +1220,23 @@ __global__ void k_wall_forces(const T *__restrict__ fn, const int *__restrict__ 
     out[2 * nbi + q] = (kCs2 * double(r) - kCs2 * rho0) / (0.5 * rho0 * uref * uref);
 }
 
-// All instances at once: output position j (instances concatenated in input order, cells in
-// input order within each) maps to internal cell map[j].
+// Absolute f of the cells map[0..total) (output position -> internal cell; one instance's part of
+// the map, or all of it), cell-major.
 template <class T>
-__global__ void k_gather_f_all(const T *__restrict__ f, const int *__restrict__ map, int total,
-                               size_t np, const int *__restrict__ tile_inst,
-                               const InstParam *__restrict__ ip, double *__restrict__ out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= total) return;
-    const int i = map[j];
-    const double rho0 = ip[tile_inst[i / kTile]].rho0;
-    for (int a = 0; a < kQ; ++a) {
-        const double wa = a == 0 ? 4.0 / 9.0 : (a < 5 ? 1.0 / 9.0 : 1.0 / 36.0);
-        out[static_cast<size_t>(j) * kQ + a] = double(f[a * np + i]) + wa * rho0;
+__global__ void __launch_bounds__(kIoBlock)
+    k_gather_f_all(const T *__restrict__ f, const int *__restrict__ map, int total, size_t np,
+                   const int *__restrict__ tile_inst, const InstParam *__restrict__ ip, double *__restrict__ out) {
+    __shared__ double sm[kIoBlock * kQ];
+    const int j0 = blockIdx.x * kIoBlock, j = j0 + threadIdx.x;
+    if (j < total) {
+        const int i = map[j];
+        const double rho0 = ip[tile_inst[i / kTile]].rho0;
+        for (int a = 0; a < kQ; ++a) {
+            const double wa = a == 0 ? 4.0 / 9.0 : (a < 5 ? 1.0 / 9.0 : 1.0 / 36.0);
+            sm[threadIdx.x * kQ + a] = double(f[a * np + i]) + wa * rho0;
+        }
     }
+    io_put<double, kQ>(sm, out, j0, total);
 }
 
 // State input: internal cells [i0, i0 + n), each reading its record at input position
@@ -1352,22 +1355,25 @@ __global__ void k_set_wdist(T *__restrict__ wdist, const int *__restrict__ map, 
 // Ghost exchange of a split mesh on device buffers: row j of vals (kXRow doubles) holds cell
 // map[j]'s f (absolute: deviation + w_alpha rho0), k, omega, nu_t (current buffers).
 template <class T>
-__global__ void k_pack_cells(const T *__restrict__ f, const T *__restrict__ kk, const T *__restrict__ ww,
-                             const T *__restrict__ nut, const int *__restrict__ map, int n, Geo<T> G,
-                             double *__restrict__ vals) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    const int i = map[j];
-    const size_t np = G.np;
-    const double rho0 = G.ip[G.tile_inst[i / kTile]].rho0;
-    double *v = vals + static_cast<size_t>(j) * kXRow;
-    for (int a = 0; a < kQ; ++a) {
-        const double wa = a == 0 ? 4.0 / 9.0 : (a < 5 ? 1.0 / 9.0 : 1.0 / 36.0);
-        v[a] = value_of(f[a * np + i]) + wa * rho0;
+__global__ void __launch_bounds__(kIoBlock)
+    k_pack_cells(const T *__restrict__ f, const T *__restrict__ kk, const T *__restrict__ ww,
+                 const T *__restrict__ nut, const int *__restrict__ map, int n, Geo<T> G, double *__restrict__ vals) {
+    __shared__ double sm[kIoBlock * kXRow];
+    const int j0 = blockIdx.x * kIoBlock, j = j0 + threadIdx.x;
+    if (j < n) {
+        const int i = map[j];
+        const size_t np = G.np;
+        const double rho0 = G.ip[G.tile_inst[i / kTile]].rho0;
+        double *v = sm + threadIdx.x * kXRow;
+        for (int a = 0; a < kQ; ++a) {
+            const double wa = a == 0 ? 4.0 / 9.0 : (a < 5 ? 1.0 / 9.0 : 1.0 / 36.0);
+            v[a] = value_of(f[a * np + i]) + wa * rho0;
+        }
+        v[9] = value_of(kk[i]);
+        v[10] = value_of(ww[i]);
+        v[11] = value_of(nut[i]);
     }
-    v[9] = value_of(kk[i]);
-    v[10] = value_of(ww[i]);
-    v[11] = value_of(nut[i]);
+    io_put<double, kXRow>(sm, vals, j0, n);
 }
 
 // The reverse: f^n (deviation) and the macros (as fvlbm_set_f writes them), k, omega and nu_t of
@@ -1417,12 +1423,15 @@ __global__ void k_gather_fields_map(const T *__restrict__ mac, const T *__restri
 }
 
 template <class T>
-__global__ void k_gather_fdev32(const T *__restrict__ f, const int *__restrict__ map, int n, size_t np,
-                                float *__restrict__ out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    const int i = map[j];
-    for (int a = 0; a < kQ; ++a) out[static_cast<size_t>(j) * kQ + a] = float(double(f[a * np + i]));
+__global__ void __launch_bounds__(kIoBlock)
+    k_gather_fdev32(const T *__restrict__ f, const int *__restrict__ map, int n, size_t np, float *__restrict__ out) {
+    __shared__ float sm[kIoBlock * kQ];
+    const int j0 = blockIdx.x * kIoBlock, j = j0 + threadIdx.x;
+    if (j < n) {
+        const int i = map[j];
+        for (int a = 0; a < kQ; ++a) sm[threadIdx.x * kQ + a] = float(double(f[a * np + i]));
+    }
+    io_put<float, kQ>(sm, out, j0, n);
 }
 
 // Tangent seed: df/dp of instance cells (off + k) from in[perm[k] * 9 + a]; the macros are
@@ -3015,33 +3024,17 @@ int fvlbm_step(fvlbm_handle *h, int n_steps, fvlbm_stats *stats) {
 int fvlbm_get_f(fvlbm_handle *h, int instance, double *f) {
     if (!h || instance < -1 || instance >= h->ninst || !f) return FVLBM_ERR_BAD_PARAM;
     CK(cudaSetDevice(h->device));
-    if (instance == -1) {
-        const int n = h->total_nc;
-        int rc = io_buffer(h, sizeof(double) * kQ * n);
-        if (rc) return rc;
-        const int nb = (n + 255) / 256;
-        dispatch(h->precision, [&](auto z_) {
-            using T = decltype(z_);
-            k_gather_f_all<T><<<nb, 256, 0, h->stream>>>(static_cast<T *>(h->fn), h->d_all_map, n,
-                                                              h->np, h->d_tile_inst, h->d_ip, h->d_io);
-        });
-        CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(f, h->d_io, sizeof(double) * kQ * n, cudaMemcpyDeviceToHost, h->stream));
-        CK(cudaStreamSynchronize(h->stream));
-        return FVLBM_OK;
-    }
-    const InstInfo &I = h->inst[instance];
-    int rc = io_buffer(h, sizeof(double) * kQ * I.nc);
+    const int n = static_cast<int>(io_cells(h, instance));
+    const int po = instance == -1 ? 0 : perm_offset(h, instance);
+    int rc = io_buffer(h, sizeof(double) * kQ * static_cast<size_t>(n));
     if (rc) return rc;
-    const int po = perm_offset(h, instance);
-    const int nb = (I.nc + 255) / 256;
     dispatch(h->precision, [&](auto z_) {
         using T = decltype(z_);
-        k_gather_f<T><<<nb, 256, 0, h->stream>>>(static_cast<T *>(h->fn), h->d_perm + po,
-                                                      I.cell_off, I.nc, I.rho0, h->np, h->d_io);
+        k_gather_f_all<T><<<(n + kIoBlock - 1) / kIoBlock, kIoBlock, 0, h->stream>>>(
+            static_cast<T *>(h->fn), h->d_all_map + po, n, h->np, h->d_tile_inst, h->d_ip, h->d_io);
     });
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(f, h->d_io, sizeof(double) * kQ * I.nc, cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(f, h->d_io, sizeof(double) * kQ * static_cast<size_t>(n), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     return FVLBM_OK;
 }
@@ -3221,7 +3214,7 @@ int fvlbm_pack_cells_dev(fvlbm_handle *h, int list_id, double *vals) {
     dispatch(h->precision, [&](auto z_) {
         using T = decltype(z_);
         const int c = h->turb;
-        k_pack_cells<T><<<(L.n + 255) / 256, 256, 0, h->stream>>>(
+        k_pack_cells<T><<<(L.n + kIoBlock - 1) / kIoBlock, kIoBlock, 0, h->stream>>>(
             static_cast<const T *>(h->fn), static_cast<const T *>(h->kk[c]), static_cast<const T *>(h->ww[c]),
             static_cast<const T *>(h->nut[c]), L.d_map, L.n, geo_of<T>(h), vals);
     });
@@ -3307,7 +3300,7 @@ int fvlbm_get_fdev_f32(fvlbm_handle *h, int instance, float *fdev) {
     float *buf = reinterpret_cast<float *>(h->d_io);
     dispatch(h->precision, [&](auto z_) {
         using T = decltype(z_);
-        k_gather_fdev32<T><<<(n + 255) / 256, 256, 0, h->stream>>>(static_cast<const T *>(h->fn),
+        k_gather_fdev32<T><<<(n + kIoBlock - 1) / kIoBlock, kIoBlock, 0, h->stream>>>(static_cast<const T *>(h->fn),
                                                                    h->d_all_map + po, n, h->np, buf);
     });
     CK(cudaGetLastError());
