@@ -20,6 +20,11 @@
 
 namespace fvlbm {
 
+// One warp a block: FP64 work is issued at one warp instruction per 64 cycles and scheduler, so what
+// counts is an even number of warps on each; single warps go to the emptiest scheduler (50k cells:
+// blocks of 128 left every sixth round of the chip unused).
+constexpr int kAdjBlock = 32;
+
 // ---- per-cell maps.  Each is affine in its inputs except through the equilibrium of a stage
 // value X, f^eq(X) = feq_dev(moments(X)), so its adjoint needs only the transposed Jacobian of
 // that map, formed in closed form:
@@ -126,7 +131,7 @@ __device__ __forceinline__ void adj_flux_acc(int i, const double *fs, const doub
             for (int a = 0; a < kQ; ++a) {
                 const double en = edot<double>(a, snx, sny);
                 double fv;
-                if (en >= 0.0)
+                if (nonneg(en))
                     fv = fi[a] + g[(2 * a) * np + i] * rox + g[(2 * a + 1) * np + i] * roy;
                 else
                     fv = fs[a * np + nb] + g[(2 * a) * np + nb] * rnx + g[(2 * a + 1) * np + nb] * rny;
@@ -148,11 +153,11 @@ __device__ __forceinline__ void adj_bv3(const Geo<double> &G, int b, double *bv3
 }
 
 // ---- transposed flux over interior faces: la (adjoint of acc) -> lf += (d acc / d f)^T la,
-// lg = (d acc / d g)^T la (boundary faces: k_adj_bndT)
+// lg = (d acc / d g)^T la (boundary faces: k_adj_gradT)
 __global__ void __launch_bounds__(kTile) k_adj_fluxT(const double *__restrict__ la, double *__restrict__ lf,
                                                      double *__restrict__ lg, Geo<double> G,
                                                      const int *__restrict__ back) {
-    const int j = blockIdx.x * kTile + threadIdx.x;
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
     double lfj[kQ], lgx[kQ], lgy[kQ], laj[kQ];
 #pragma unroll
@@ -172,13 +177,13 @@ __global__ void __launch_bounds__(kTile) k_adj_fluxT(const double *__restrict__ 
 #pragma unroll
         for (int a = 1; a < kQ; ++a) {
             const double en = edot<double>(a, snx, sny);
-            if (en >= 0.0) {  // this cell's own flux took its own reconstruction
+            if (nonneg(en)) {  // this cell's own flux took its own reconstruction
                 lfj[a] += en * laj[a];
                 lgx[a] += en * rox * laj[a];
                 lgy[a] += en * roy * laj[a];
             }
             const double eni = edot<double>(a, six, siy);
-            if (!(eni >= 0.0)) {  // the neighbour's flux through this face took this cell's
+            if (!nonneg(eni)) {  // the neighbour's flux through this face took this cell's
                 const double lai = la[a * np + nb];
                 lfj[a] += eni * lai;
                 lgx[a] += eni * rix * lai;
@@ -194,12 +199,18 @@ __global__ void __launch_bounds__(kTile) k_adj_fluxT(const double *__restrict__ 
     }
 }
 
-// ---- transposed gradient, linear part: lf += (d g / d f)^T lg with the boundary values held
-// fixed (g_j = sum_m W_m (f_m - f_j)); their dependence on f_j is added by k_adj_bndT
+// ---- transposed gradient: lf += (d g / d f)^T lg (g_j = sum_m W_m (f_m - f_j)), then the cell's
+// boundary faces.  The face value f_bc(f_j, bval) enters the flux (weight e.n) and the gradient
+// (weight W_m); one transposed local Jacobian per face serves both:
+//   c = (e.n) la_j + W_m^T lg_j,  lf_j += (d f_bc / d f_j)^T c,  lbval += (d f_bc / d bval)^T c
+// (as a kernel of its own the boundary part held the chip for 33 us for a few hundred cells).
 __global__ void __launch_bounds__(kTile) k_adj_gradT(const double *__restrict__ lg, double *__restrict__ lf,
                                                      Geo<double> G, const int *__restrict__ back,
-                                                     const double *__restrict__ lnb) {
-    const int j = blockIdx.x * kTile + threadIdx.x;
+                                                     const double *__restrict__ lnb,
+                                                     const double *__restrict__ fs,
+                                                     const double *__restrict__ la, double *__restrict__ lbval,
+                                                     const double *__restrict__ lbf) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
     double lfj[kQ], lgx[kQ], lgy[kQ];
 #pragma unroll
@@ -208,9 +219,11 @@ __global__ void __launch_bounds__(kTile) k_adj_gradT(const double *__restrict__ 
         lgx[a] = lg[(2 * a) * np + j];
         lgy[a] = lg[(2 * a + 1) * np + j];
     }
+    int nbnd = 0;
     for (int m = 0; m < 4; ++m) {
         const int nb = G.nbr[m * np + j];
         if (nb == kNone) continue;
+        nbnd += nb < 0 ? 1 : 0;
         const double wx = G.lsq[(2 * m) * np + j], wy = G.lsq[(2 * m + 1) * np + j];
 #pragma unroll
         for (int a = 0; a < kQ; ++a) lfj[a] -= wx * lgx[a] + wy * lgy[a];
@@ -224,6 +237,28 @@ __global__ void __launch_bounds__(kTile) k_adj_gradT(const double *__restrict__ 
                 for (int a = 1; a < kQ; ++a) lfj[a] += lnb[(a * 4 + b) * np + nb];
         }
     }
+    if (nbnd > 0) {
+        const double rho0 = G.ip[G.tile_inst[j / kTile]].rho0;
+        double fj[kQ];
+#pragma unroll
+        for (int a = 0; a < kQ; ++a) fj[a] = fs[a * np + j];
+        for (int m = 0; m < 4; ++m) {
+            const int nb = G.nbr[m * np + j];
+            if (nb >= 0 || nb == kNone) continue;
+            const int bf = -nb - 1;
+            const double snx = G.sn[(2 * m) * np + j], sny = G.sn[(2 * m + 1) * np + j];
+            const double wx = G.lsq[(2 * m) * np + j], wy = G.lsq[(2 * m + 1) * np + j];
+            double c[kQ], bv3[3], lb3[3] = {0, 0, 0};
+#pragma unroll
+            for (int a = 0; a < kQ; ++a)
+                c[a] = edot<double>(a, snx, sny) * la[a * np + j] + wx * lgx[a] + wy * lgy[a] +
+                       (lbf != nullptr ? lbf[(a * 4 + m) * np + j] : 0.0);
+            adj_bv3(G, bf, bv3);
+            adj_bvals_T(G.btype[bf], bv3, snx, sny, fj, rho0, c, lfj, lb3);
+            if (lbval != nullptr)
+                for (int q = 0; q < 3; ++q) lbval[q * G.nbt + bf] += lb3[q];
+        }
+    }
 #pragma unroll
     for (int a = 0; a < kQ; ++a) lf[a * np + j] = lfj[a];
 }
@@ -234,15 +269,15 @@ __global__ void __launch_bounds__(kTile) k_adj_gradT(const double *__restrict__ 
 // In: lg, the adjoint of the limited gradient.  Out: lg <- the adjoint of g_raw; lf_i gets the
 // adjoint of f_i through d1; the extreme's share goes to the per-face buffers, lnb[(a * 4 + m)
 // * np + i] for a neighbour (gathered by k_adj_gradT) and lbf for a boundary value (added by
-// k_adj_bndT).  Branches (extremes, the minimum over faces) follow the values, ties keeping the
+// its boundary part).  Branches (extremes, the minimum over faces) follow the values, ties keeping the
 // first argument, as the forward's fmin / fmax.
 __global__ void __launch_bounds__(kTile) k_adj_limT(const double *__restrict__ fs, double *__restrict__ lg,
                                                     double *__restrict__ lf, double *__restrict__ lnb,
                                                     double *__restrict__ lbf, Geo<double> G,
                                                     double *__restrict__ a_rown, double *__restrict__ a_area) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[blockIdx.x]];
+    const InstParam P = G.ip[G.tile_inst[i / kTile]];
     for (int c = 0; c < 4 * kQ; ++c) {
         lnb[c * np + i] = 0.0;
         lbf[c * np + i] = 0.0;
@@ -335,48 +370,6 @@ __global__ void __launch_bounds__(kTile) k_adj_limT(const double *__restrict__ f
     if (a_area != nullptr) a_area[i] += l_e2 * 1.5 * sqrt(ar);
 }
 
-// ---- boundary faces: the face value f_bc(f_j, bval) enters the flux (weight e.n) and the
-// gradient (weight W_m); one transposed local Jacobian per face serves both:
-//   c = (e.n) la_j + W_m^T lg_j,  lf_j += (d f_bc / d f_j)^T c,  lbval += (d f_bc / d bval)^T c
-__global__ void __launch_bounds__(kTile) k_adj_bndT(const double *__restrict__ fs, const double *__restrict__ la,
-                                                    const double *__restrict__ lg, double *__restrict__ lf,
-                                                    double *__restrict__ lbval, Geo<double> G,
-                                                    const double *__restrict__ lbf) {
-    const int j = blockIdx.x * kTile + threadIdx.x;
-    const size_t np = G.np;
-    int nbnd = 0;
-    for (int m = 0; m < 4; ++m) {
-        const int nb = G.nbr[m * np + j];
-        nbnd += (nb < 0 && nb != kNone) ? 1 : 0;
-    }
-    if (nbnd == 0) return;
-    const double rho0 = G.ip[G.tile_inst[blockIdx.x]].rho0;
-    double lfj[kQ], fj[kQ];
-#pragma unroll
-    for (int a = 0; a < kQ; ++a) {
-        lfj[a] = lf[a * np + j];
-        fj[a] = fs[a * np + j];
-    }
-    for (int m = 0; m < 4; ++m) {
-        const int nb = G.nbr[m * np + j];
-        if (nb >= 0 || nb == kNone) continue;
-        const int bf = -nb - 1;
-        const double snx = G.sn[(2 * m) * np + j], sny = G.sn[(2 * m + 1) * np + j];
-        const double wx = G.lsq[(2 * m) * np + j], wy = G.lsq[(2 * m + 1) * np + j];
-        double c[kQ], bv3[3], lb3[3] = {0, 0, 0};
-#pragma unroll
-        for (int a = 0; a < kQ; ++a)
-            c[a] = edot<double>(a, snx, sny) * la[a * np + j] + wx * lg[(2 * a) * np + j] +
-                   wy * lg[(2 * a + 1) * np + j] + (lbf != nullptr ? lbf[(a * 4 + m) * np + j] : 0.0);
-        adj_bv3(G, bf, bv3);
-        adj_bvals_T(G.btype[bf], bv3, snx, sny, fj, rho0, c, lfj, lb3);
-        if (lbval != nullptr)
-            for (int q = 0; q < 3; ++q) lbval[q * G.nbt + bf] += lb3[q];
-    }
-#pragma unroll
-    for (int a = 0; a < kQ; ++a) lf[a * np + j] = lfj[a];
-}
-
 // ---- adjoints of the geometry arrays read by one flux and gradient evaluation: with la the
 // adjoint of acc and lg that of g at this stage value, accumulate dJ/d(sn, rown, rnbr, lsq) of
 // every face slot of the cell (one thread per cell, its own slots only).
@@ -385,9 +378,9 @@ __global__ void __launch_bounds__(kTile) k_adj_geom(const double *__restrict__ f
                                                     Geo<double> G, double *__restrict__ a_sn,
                                                     double *__restrict__ a_lsq, double *__restrict__ a_rown,
                                                     double *__restrict__ a_rnbr) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const double rho0 = G.ip[G.tile_inst[blockIdx.x]].rho0;
+    const double rho0 = G.ip[G.tile_inst[i / kTile]].rho0;
     double fi[kQ];
     load9(fs, np, i, fi);
     for (int m = 0; m < 4; ++m) {
@@ -404,7 +397,7 @@ __global__ void __launch_bounds__(kTile) k_adj_geom(const double *__restrict__ f
                 const double l = la[a * np + i];
                 const double fm = fs[a * np + nb];
                 double fv;
-                if (en >= 0.0) {
+                if (nonneg(en)) {
                     const double gx = g[(2 * a) * np + i], gy = g[(2 * a + 1) * np + i];
                     fv = fi[a] + gx * rox + gy * roy;
                     s_rox += l * en * gx;
@@ -449,9 +442,9 @@ __global__ void __launch_bounds__(kTile) k_adj_geom(const double *__restrict__ f
 __global__ void __launch_bounds__(kTile) k_adj_stage3(const double *__restrict__ L, double *__restrict__ lf3,
                                                       double *__restrict__ lc, double *__restrict__ la,
                                                       Geo<double> G) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const double dt = cell_dt(G, G.ip[G.tile_inst[blockIdx.x]], i);
+    const double dt = cell_dt(G, G.ip[G.tile_inst[i / kTile]], i);
 #pragma unroll
     for (int a = 0; a < kQ; ++a) {
         const double l = L[a * np + i];
@@ -468,9 +461,9 @@ __global__ void __launch_bounds__(kTile) k_adj_stage2(const double *__restrict__
                                                       const double *__restrict__ lf3, const double *__restrict__ lc,
                                                       double *__restrict__ lB, double *__restrict__ la,
                                                       double *__restrict__ ltau, Geo<double> G) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[blockIdx.x]];
+    const InstParam P = G.ip[G.tile_inst[i / kTile]];
     const double dt = cell_dt(G, P, i);
     double acc[kQ], X[kQ], mu[kQ], lX[kQ];
     adj_flux_acc(i, f2, g2, G, P.rho0, acc);
@@ -511,9 +504,9 @@ __global__ void __launch_bounds__(kTile) k_adj_stage1(const double *__restrict__
                                                       double *__restrict__ la, double *__restrict__ ltau,
                                                       Geo<double> G, const double *__restrict__ tau1,
                                                       double *__restrict__ ltau1) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[blockIdx.x]];
+    const InstParam P = G.ip[G.tile_inst[i / kTile]];
     const double dt = cell_dt(G, P, i);
     double acc[kQ], x0[kQ], X[kQ], lX[kQ], mu[kQ], lb[kQ];
     adj_flux_acc(i, s1, g1, G, P.rho0, acc);
@@ -573,9 +566,9 @@ __global__ void __launch_bounds__(kTile) k_adj_stage1(const double *__restrict__
 __global__ void __launch_bounds__(kTile) k_adj_relax(const double *__restrict__ f0, const double *__restrict__ tau,
                                                      const double *__restrict__ ls1, double *__restrict__ lf0,
                                                      double *__restrict__ ltau, Geo<double> G) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[blockIdx.x]];
+    const InstParam P = G.ip[G.tile_inst[i / kTile]];
     const double zq = cell_dt(G, P, i) / tau[i] * 0.25;
     const double inv = 1.0 / (1.0 + zq);
     double x0[kQ], l0[kQ], mu[kQ];
@@ -606,9 +599,9 @@ __global__ void __launch_bounds__(kTile) k_adj_euler(const double *__restrict__ 
                                                      const double *__restrict__ L, double *__restrict__ lf0,
                                                      double *__restrict__ la, double *__restrict__ ltau,
                                                      Geo<double> G) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[blockIdx.x]];
+    const InstParam P = G.ip[G.tile_inst[i / kTile]];
     const double dt = cell_dt(G, P, i), c = dt / tau[i];
     double x0[kQ], l0[kQ], mu[kQ];
 #pragma unroll
@@ -639,16 +632,16 @@ __global__ void __launch_bounds__(kTile) k_adj_seed(const double *__restrict__ f
                                                     double *__restrict__ L, double *__restrict__ lbval,
                                                     double *__restrict__ a_bnrm, double *__restrict__ a_blen,
                                                     Geo<double> G) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const double rho0 = G.ip[G.tile_inst[blockIdx.x]].rho0;
+    const double rho0 = G.ip[G.tile_inst[i / kTile]].rho0;
     double lfi[kQ], fi[kQ];
 #pragma unroll
     for (int a = 0; a < kQ; ++a) {
         lfi[a] = 0.0;
         fi[a] = fn[a * np + i];
     }
-    if (G.tile_inst[blockIdx.x] == inst) {
+    if (G.tile_inst[i / kTile] == inst) {
         for (int m = 0; m < 4; ++m) {
             const int nb = G.nbr[m * np + i];
             if (nb == kNone || nb >= 0) continue;
@@ -752,7 +745,7 @@ struct AdjStep {
 // per-stage reading), with the stage values kept in S.
 void adj_forward_step(fvlbm_handle *h, const Geo<double> &G, const AdjState &in, const AdjState &out,
                       const AdjStep &S) {
-    const dim3 grid(h->ntiles), block(kTile);
+    const dim3 grid(h->np / kAdjBlock), block(kAdjBlock);
     cudaStream_t s = h->stream;
     const double *tau = static_cast<const double *>(h->tau);
     double *mac_out = S.mac;
@@ -832,7 +825,7 @@ struct AdjVars {
 // SST handles (lk, lw, lnt) <- adjoints of (k, omega, nu_t)^n.
 void adj_backward_step(fvlbm_handle *h, const Geo<double> &G, const AdjState &in, const AdjStep &S,
                        AdjVars &A) {
-    const dim3 grid(h->ntiles), block(kTile);
+    const dim3 grid(h->np / kAdjBlock), block(kAdjBlock);
     cudaStream_t s = h->stream;
     const size_t nq = static_cast<size_t>(kQ) * h->np;
     const double *tau = h->sst ? S.tau : static_cast<const double *>(h->tau);
@@ -847,8 +840,7 @@ void adj_backward_step(fvlbm_handle *h, const Geo<double> &G, const AdjState &in
         k_adj_fluxT<<<grid, block, 0, s>>>(A.la, lf, A.lg, G, back);
         if (A.lnb) k_adj_limT<<<grid, block, 0, s>>>(fs, A.lg, lf, A.lnb, A.lbf, G, A.a_rown, A.a_area);
         geom(fs, g);
-        k_adj_gradT<<<grid, block, 0, s>>>(A.lg, lf, G, back, A.lnb);
-        k_adj_bndT<<<grid, block, 0, s>>>(fs, A.la, A.lg, lf, A.lbval, G, A.lbf);
+        k_adj_gradT<<<grid, block, 0, s>>>(A.lg, lf, G, back, A.lnb, fs, A.la, A.lbval, A.lbf);
     };
     if (h->scheme == 1) {
         k_adj_euler<<<grid, block, 0, s>>>(f0, tau, A.L, A.lf0, A.la, A.ltau, G);
@@ -1142,7 +1134,7 @@ int adjoint_impl(fvlbm_handle *h, int instance, int n_steps, const double *w, do
         const double al = I.alpha_deg * M_PI / 180.0, ca = std::cos(al), sa = std::sin(al);
         const double cx = (w[0] * ca - w[1] * sa) / q, cy = (w[0] * sa + w[1] * ca) / q;
         CK(cudaMemsetAsync(A.lbval, 0, 5 * nbt * sizeof(double), s));
-        k_adj_seed<<<h->ntiles, kTile, 0, s>>>(fN, static_cast<const double *>(h->bnrm),
+        k_adj_seed<<<h->np / kAdjBlock, kAdjBlock, 0, s>>>(fN, static_cast<const double *>(h->bnrm),
                                                static_cast<const double *>(h->blen), instance, cx, cy, A.L,
                                                A.lbval, A.a_bnrm, A.a_blen, G);
         CK(cudaGetLastError());

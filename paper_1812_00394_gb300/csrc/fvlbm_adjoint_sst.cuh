@@ -123,9 +123,9 @@ __global__ void __launch_bounds__(kTile) k_adj_sst_update(
     const double *__restrict__ lk1, const double *__restrict__ lw1, const double *__restrict__ lnt1,
     const double *__restrict__ ltau, double *__restrict__ own, double *__restrict__ fbuf,
     double *__restrict__ lbval, Geo<double> G, AdjGeo AG) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[blockIdx.x]];
+    const InstParam P = G.ip[G.tile_inst[i / kTile]];
     if (!P.sst) return;
     const double nu = P.nu, dt = cell_dt(G, P, i);
     const double ui = mac[np + i], vi = mac[2 * np + i], ki = kk[i], wi = ww[i], nti = nut[i];
@@ -428,9 +428,9 @@ __global__ void __launch_bounds__(kTile) k_adj_sst_grad(
     const double *__restrict__ grads, const double *__restrict__ f1a, const double *__restrict__ fbu,
     double *__restrict__ own, double *__restrict__ fbg, double *__restrict__ lbval, Geo<double> G,
     const int *__restrict__ back, AdjGeo AG) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[blockIdx.x]];
+    const InstParam P = G.ip[G.tile_inst[i / kTile]];
     if (!P.sst) return;
     const double nu = P.nu;
     const double ow[4] = {mac[np + i], mac[2 * np + i], kk[i], ww[i]};
@@ -624,9 +624,9 @@ __global__ void __launch_bounds__(kTile) k_adj_sst_finish(
     const double *__restrict__ fn, const double *__restrict__ own, const double *__restrict__ fbu,
     const double *__restrict__ fbg, double *__restrict__ lf, double *__restrict__ lk,
     double *__restrict__ lw, double *__restrict__ lnt, Geo<double> G, const int *__restrict__ back, bool add) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[blockIdx.x]];
+    const InstParam P = G.ip[G.tile_inst[i / kTile]];
     if (!P.sst) return;
     double l[5];
 #pragma unroll

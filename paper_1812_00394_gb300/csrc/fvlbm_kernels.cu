@@ -115,6 +115,15 @@ __device__ __forceinline__ T cell_dt(const Geo<T> &G, const InstParam &P, int i)
     return G.dtc != nullptr ? G.dtc[i] : ipv<T>(P.dt, P.dt_f);
 }
 
+// x >= 0.  In double on the bit pattern (a compare would take a slot of the FP64 pipe, 64 cycles;
+// -0 counts, a NaN goes by its sign).
+__device__ __forceinline__ bool nonneg(float x) { return x >= 0.f; }
+__device__ __forceinline__ bool nonneg(double x) {
+    const long long b = __double_as_longlong(x);
+    return b >= 0 || (b << 1) == 0;
+}
+__device__ __forceinline__ bool nonneg(const Dual &x) { return nonneg(x.v); }
+
 // ------------------------------------------------------------------ cell algebra
 // Quotient a / b in the collision and stage algebra and in the SST gradients (limiter, f1).
 // In float it is the fast form (within 2 ulp instead of correctly rounded): the FP32 path
@@ -217,9 +226,9 @@ __device__ __forceinline__ void relax9(T *f, T rho0, T dt, T tau_i, T *eq_out = 
 template <class T>
 __global__ void __launch_bounds__(kTile) k_stage1(const T *__restrict__ fn, T *__restrict__ fs,
                                                   const T *__restrict__ tau, Geo<T> G) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[blockIdx.x]];
+    const InstParam P = G.ip[G.tile_inst[i / kTile]];
     T f[kQ];
     load9(fn, np, i, f);
     relax9(f, ipv<T>(P.rho0, P.rho0_f), cell_dt(G, P, i), tau[i]);
@@ -231,11 +240,11 @@ __global__ void __launch_bounds__(kTile) k_stage1(const T *__restrict__ fn, T *_
 template <class T>
 __global__ void __launch_bounds__(kTile) k_stage_macros(const T *__restrict__ fs, T *__restrict__ mac,
                                                         Geo<T> G) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
     T f[kQ], dr, r, u, v;
     load9(fs, np, i, f);
-    const InstParam &P = G.ip[G.tile_inst[blockIdx.x]];
+    const InstParam &P = G.ip[G.tile_inst[i / kTile]];
     moments(f, ipv<T>(P.rho0, P.rho0_f), dr, r, u, v);
     mac[i] = r;
     mac[np + i] = u;
@@ -248,9 +257,9 @@ __global__ void __launch_bounds__(kTile) k_stage_macros(const T *__restrict__ fs
 template <class T, bool LIMIT>
 __global__ void __launch_bounds__(kTile) k_grad(const T *__restrict__ f, T *__restrict__ g,
                                                 Geo<T> G) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[blockIdx.x]];
+    const InstParam P = G.ip[G.tile_inst[i / kTile]];
     const T rho0 = ipv<T>(P.rho0, P.rho0_f);
     T fi[kQ], gx[kQ], gy[kQ], lo[kQ], hi[kQ];
     load9(f, np, i, fi);
@@ -528,9 +537,9 @@ __global__ void __launch_bounds__(kTile)
                  T *__restrict__ fn, T *__restrict__ Bacc, T *__restrict__ Cacc,
                  const T *__restrict__ tau, T *__restrict__ mac, double *__restrict__ partial,
                  Geo<T> G, const T *__restrict__ tau1 = nullptr) {
-    const int i = blockIdx.x * kTile + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[blockIdx.x]];
+    const InstParam P = G.ip[G.tile_inst[i / kTile]];
     const T rho0 = ipv<T>(P.rho0, P.rho0_f);
     T fi[kQ], acc[kQ];
     load9(fs, np, i, fi);
@@ -548,7 +557,7 @@ __global__ void __launch_bounds__(kTile)
             for (int a = 0; a < kQ; ++a) {
                 const T en = edot<T>(a, snx, sny);
                 T fv;
-                if (en >= T(0))
+                if (nonneg(en))
                     fv = fi[a] + g[(2 * a) * np + i] * rox + g[(2 * a + 1) * np + i] * roy;
                 else
                     fv = fs[a * np + nb] + g[(2 * a) * np + nb] * rnx + g[(2 * a + 1) * np + nb] * rny;
@@ -959,8 +968,7 @@ __global__ void __launch_bounds__(kTile)
     k_sst_grad(const T *mac, const T *kk, const T *ww, T *__restrict__ grads, T *__restrict__ f1out, Geo<T> G,
                CompactGeo<T> CG, const T *nut, T *__restrict__ rec8, T *__restrict__ rec2, bool inv_only,
                int tile0) {
-    const int tile = tile0 + static_cast<int>(blockIdx.x);
-    const int i = tile * kTile + threadIdx.x;
+    const int i = tile0 * kTile + static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x), tile = i / kTile;
     const size_t np = G.np;
     const InstParam P = G.ip[G.tile_inst[tile]];
     const T nu = ipv<T>(P.nu, P.nu_f);
@@ -1047,8 +1055,8 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
                  T *__restrict__ k_out, T *__restrict__ w_out, T *__restrict__ nut_out, T *__restrict__ tau,
                  Geo<T> G, CompactGeo<T> CG, const T *rec8, const T *rec2, int tile0) {
     // backwards: the records that k_sst_grad wrote last are still in L2
-    const int tile = tile0 + static_cast<int>(gridDim.x - 1 - blockIdx.x);
-    const int i = tile * kTile + threadIdx.x;
+    const int i = tile0 * kTile + static_cast<int>((gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x);
+    const int tile = i / kTile;
     const size_t np = G.np;
     const InstParam P = G.ip[G.tile_inst[tile]];
     const T nu = ipv<T>(P.nu, P.nu_f);
@@ -1868,13 +1876,18 @@ void for_sst_runs(const fvlbm_handle *h, F &&f) {
     for (const int2 &r : h->sst_runs) f(dim3(static_cast<unsigned>(r.y)), r.x);
 }
 
+// Threads per block of the two-pass kernels without statistics: in double one warp, which goes to
+// the emptiest scheduler (an FP64 instruction holds one for 64 cycles).
+template <class T>
+constexpr int kTwoPassBlock = sizeof(T) == 8 ? 32 : kTile;
+
 // The two SST kernels of the two-pass path (unpacked gradients, geometry read as stored), on
 // stream h->stream: gradients and f1 of the macros mac, then k, omega, nu_t and tau_out.
 template <class T>
 void sst_grad_twopass(const fvlbm_handle *h, const T *mac, const T *kc, const T *wc, T *sg, T *f1,
                       const Geo<T> &G, const CompactGeo<T> &CG) {
     for_sst_runs(h, [&](dim3 g, int t0) {
-        k_sst_grad<T, false><<<g, kTile, 0, h->stream>>>(mac, kc, wc, sg, f1, G, CG, nullptr, nullptr,
+        k_sst_grad<T, false><<<g.x * (kTile / kTwoPassBlock<T>), kTwoPassBlock<T>, 0, h->stream>>>(mac, kc, wc, sg, f1, G, CG, nullptr, nullptr,
                                                          nullptr, false, t0);
     });
 }
@@ -1884,10 +1897,10 @@ void sst_update_twopass(const fvlbm_handle *h, const T *mac, const T *kc, const 
                         const CompactGeo<T> &CG) {
     for_sst_runs(h, [&](dim3 g, int t0) {
         if (h->nonorth)
-            k_sst_update<T, false, true><<<g, kTile, 0, h->stream>>>(mac, kc, wc, nc, sg, f1, kn, wn, nn, tau_out,
+            k_sst_update<T, false, true><<<g.x * (kTile / kTwoPassBlock<T>), kTwoPassBlock<T>, 0, h->stream>>>(mac, kc, wc, nc, sg, f1, kn, wn, nn, tau_out,
                                                                      G, CG, nullptr, nullptr, t0);
         else
-            k_sst_update<T, false, false><<<g, kTile, 0, h->stream>>>(mac, kc, wc, nc, sg, f1, kn, wn, nn, tau_out,
+            k_sst_update<T, false, false><<<g.x * (kTile / kTwoPassBlock<T>), kTwoPassBlock<T>, 0, h->stream>>>(mac, kc, wc, nc, sg, f1, kn, wn, nn, tau_out,
                                                                       G, CG, nullptr, nullptr, t0);
     });
 }
@@ -1952,7 +1965,7 @@ void enqueue_tangent(fvlbm_handle *h, bool stats) {
 template <class T>
 void enqueue_step(fvlbm_handle *h, bool stats) {
     Geo<T> G = geo_of<T>(h);
-    const dim3 grid(h->ntiles), block(kTile);
+    const dim3 grid(h->np / kTwoPassBlock<T>), block(kTwoPassBlock<T>), sgrid(h->ntiles), sblock(kTile);
     cudaStream_t s = h->stream;
     T *fn = static_cast<T *>(h->fn), *s0 = static_cast<T *>(h->s0), *s1 = static_cast<T *>(h->s1);
     T *B = static_cast<T *>(h->bacc), *C = static_cast<T *>(h->cacc);
@@ -1974,7 +1987,7 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
                 if (!std::is_same<T, double>::value || h->nonorth) {
                     launch(h, K_SST_GRAD, "sst_grad", [&] {
                         for_sst_runs(h, [&](dim3 sg_grid, int t0) {
-                            launch_dep(k_sst_grad<T, true>, sg_grid, block, 0, s, mac, kc, wc, sg, f1, G, CG, nc, r8, r2,
+                            launch_dep(k_sst_grad<T, true>, sg_grid, sblock, 0, s, mac, kc, wc, sg, f1, G, CG, nc, r8, r2,
                                                                           !h->nonorth, t0);
                         });
                     });
@@ -1982,10 +1995,10 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
                         for_sst_runs(h, [&](dim3 sg_grid, int t0) {
                             if (h->nonorth)
                                 launch_dep(
-                                    k_sst_update<T, true, true>, sg_grid, block, 0, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
+                                    k_sst_update<T, true, true>, sg_grid, sblock, 0, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
                             else if constexpr (!std::is_same<T, double>::value)
                                 launch_dep(
-                                    k_sst_update<T, true, false>, sg_grid, block, 0, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
+                                    k_sst_update<T, true, false>, sg_grid, sblock, 0, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG, r8, r2, t0);
                         });
                     });
                 }
@@ -2032,7 +2045,7 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
             launch(h, K_GRAD, "grad_f", [&] { grad_f<T>(h, grid, block, s, s0, g, G); });
             if (stats) {
                 launch(h, K_FLUX3, "flux_stage3", [&] {
-                    k_flux_stage<T, 3, true><<<grid, block, 0, s>>>(s0, g, s1, fn, B, C, tau, mac, h->d_partial, G);
+                    k_flux_stage<T, 3, true><<<sgrid, sblock, 0, s>>>(s0, g, s1, fn, B, C, tau, mac, h->d_partial, G);
                 });
                 launch(h, K_REDUCE, "reduce", [&] {
                     k_reduce_instances<<<h->ninst, kTile, 0, s>>>(h->d_partial, h->d_inst_tile0, h->d_inst_sums);
@@ -2057,7 +2070,7 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
         launch(h, K_GRAD, "grad_f", [&] { grad_f<T>(h, grid, block, s, fn, g, G); });
         if (stats) {
             launch(h, K_EULER, "euler", [&] {
-                k_flux_stage<T, 4, true><<<grid, block, 0, s>>>(fn, g, s0, fn, B, C, tau, mac, h->d_partial, G);
+                k_flux_stage<T, 4, true><<<sgrid, sblock, 0, s>>>(fn, g, s0, fn, B, C, tau, mac, h->d_partial, G);
             });
             launch(h, K_REDUCE, "reduce", [&] {
                 k_reduce_instances<<<h->ninst, kTile, 0, s>>>(h->d_partial, h->d_inst_tile0, h->d_inst_sums);
@@ -2088,7 +2101,7 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
     launch(h, K_GRAD, "grad_f", [&] { grad_f<T>(h, grid, block, s, s0, g, G); });
     if (stats) {
         launch(h, K_FLUX3, "flux_stage3", [&] {
-            k_flux_stage<T, 3, true><<<grid, block, 0, s>>>(s0, g, s1, fn, B, C, tau, mac, h->d_partial, G);
+            k_flux_stage<T, 3, true><<<sgrid, sblock, 0, s>>>(s0, g, s1, fn, B, C, tau, mac, h->d_partial, G);
         });
         launch(h, K_REDUCE, "reduce", [&] {
             k_reduce_instances<<<h->ninst, kTile, 0, s>>>(h->d_partial, h->d_inst_tile0, h->d_inst_sums);

@@ -54,13 +54,6 @@ template <class S>
 __device__ __forceinline__ S max64(const S &a, const S &b) {
     return ord64(b) > ord64(a) ? b : a;
 }
-// x >= 0, -0 included (a NaN of either sign counts by it)
-__device__ __forceinline__ bool nonneg64(double x) {
-    const long long b = __double_as_longlong(x);
-    return b >= 0 || (b << 1) == 0;
-}
-__device__ __forceinline__ bool nonneg64(const Dual &x) { return nonneg64(x.v); }
-
 // tanh of x >= 0
 __device__ __forceinline__ double tanh64(double x) {
     const long long b = __double_as_longlong(x);
@@ -264,7 +257,7 @@ __global__ void __launch_bounds__(kSst64Block)
             sw = scale(2.0, gwi);
         }
         const S un = mad(su, snx, sv * sny);  // 2 (u_f . n) dl / A
-        const bool out = nonneg64(un);        // upwind side
+        const bool out = nonneg(un);        // upwind side
         const S rx = out ? rox : rnx, ry = out ? roy : rny;
         const S kup = mad(out ? lkx : jkx, rx, mad(out ? lky : jky, ry, out ? ki : kj));
         const S wup = mad(out ? lwx : jwx, rx, mad(out ? lwy : jwy, ry, out ? wi : wj));
