@@ -82,6 +82,54 @@ S point_segment(S px, S py, S ax, S ay, S bx, S by) {
     return sqrt(dx * dx + dy * dy);
 }
 
+// Nearest wall face of points that come one after another: the first of equals in the walls' order,
+// as a plain search finds it.  A wall is passed over where the distance to its midpoint less half
+// its length already exceeds the distance to the wall nearest to the point before, or the best so far
+// (with a margin for rounding), which leaves a few of several hundred to measure.
+class NearestWall {
+public:
+    template <class S>
+    NearestWall(const fvlbm_bc &bc, const std::vector<int> &walls, const S *xy) : bc_(bc), walls_(walls) {
+        for (int b : walls) {
+            const int a0 = bc.bedge_nodes[2 * b], a1 = bc.bedge_nodes[2 * b + 1];
+            const double x0 = value_of(xy[2 * a0]), y0 = value_of(xy[2 * a0 + 1]);
+            const double x1 = value_of(xy[2 * a1]), y1 = value_of(xy[2 * a1 + 1]);
+            mx_.push_back(0.5 * (x0 + x1));
+            my_.push_back(0.5 * (y0 + y1));
+            half_.push_back(0.5 * std::sqrt((x1 - x0) * (x1 - x0) + (y1 - y0) * (y1 - y0)));
+        }
+    }
+    // (*last: index into the walls to start from, updated; returns the distance)
+    template <class S>
+    S find(const S &px, const S &py, const S *xy, int *last) const {
+        auto dist = [&](int q) {
+            const int b = walls_[q];
+            const int a0 = bc_.bedge_nodes[2 * b], a1 = bc_.bedge_nodes[2 * b + 1];
+            return point_segment(px, py, xy[2 * a0], xy[2 * a0 + 1], xy[2 * a1], xy[2 * a1 + 1]);
+        };
+        const double x = value_of(px), y = value_of(py);
+        double bound = value_of(dist(*last)) * (1.0 + 1e-9);
+        S best = 1e300;
+        const int n = static_cast<int>(walls_.size());
+        for (int q = 0; q < n; ++q) {
+            const double dx = x - mx_[q], dy = y - my_[q], r = bound + half_[q];
+            if (dx * dx + dy * dy > r * r * (1.0 + 1e-9)) continue;
+            const S d = dist(q);
+            if (d < best) {
+                best = d;
+                *last = q;
+                bound = std::min(bound, value_of(d) * (1.0 + 1e-9));
+            }
+        }
+        return best;
+    }
+
+private:
+    const fvlbm_bc &bc_;
+    const std::vector<int> &walls_;
+    std::vector<double> mx_, my_, half_;
+};
+
 template <class S>
 struct FaceGeo {
     int nbr = kNone;        // neighbour input cell id, or -(b+1) boundary edge, or kNone
@@ -400,21 +448,20 @@ int prepare_instance_t(const fvlbm_mesh &m, const fvlbm_bc &bc, const fvlbm_para
             P.lsq[(2 * l + 1) * np + k] = (mxx * dy[l] - mxy * dx[l]) / det;
         }
     }
-    // wall distance: centroid to nearest wall face (brute force over wall faces)
+    // wall distance: centroid to nearest wall face
     std::vector<int> walls;
     for (int b = 0; b < nbe; ++b)
         if (!glued[b] && bc.bedge_type[b] == FVLBM_BC_WALL) walls.push_back(b);
     if (!walls.empty()) {
-#pragma omp parallel for schedule(static)
-        for (int k = 0; k < nc; ++k) {
-            const int i = P.perm[k];
-            S best = 1e300;
-            for (int b : walls) {
-                const int a0 = bc.bedge_nodes[2 * b], a1 = bc.bedge_nodes[2 * b + 1];
-                best = smin(best, point_segment(cx[i], cy[i], xy[2 * a0], xy[2 * a0 + 1],
-                                                xy[2 * a1], xy[2 * a1 + 1]));
+        const NearestWall search(bc, walls, xy);
+#pragma omp parallel
+        {
+            int last = 0;
+#pragma omp for schedule(static)
+            for (int k = 0; k < nc; ++k) {
+                const int i = P.perm[k];
+                P.wdist[k] = search.find(cx[i], cy[i], xy, &last);
             }
-            P.wdist[k] = best;
         }
     }
     // time step: dt, or cfl over the largest upwind outflow rate max_i max_alpha
@@ -648,17 +695,16 @@ int geometry_adjoint(const fvlbm_mesh &m, const fvlbm_bc &bc, const GeometryAdjo
         for (int b = 0; b < bc.n_bedges; ++b)
             if (bc.bedge_type[b] == FVLBM_BC_WALL) walls.push_back(b);
         std::vector<int> nearest(walls.empty() ? 0 : nc, -1);
-#pragma omp parallel for schedule(static)
-        for (int i = 0; i < static_cast<int>(nearest.size()); ++i) {
-            if (A.wdist[i] == 0.0) continue;
-            double best = 1e300;
-            for (int b : walls) {
-                const int a0 = bc.bedge_nodes[2 * b], a1 = bc.bedge_nodes[2 * b + 1];
-                const double d = point_segment(cxv[i], cyv[i], m.xy[2 * a0], m.xy[2 * a0 + 1], m.xy[2 * a1],
-                                               m.xy[2 * a1 + 1]);
-                if (d < best) {
-                    best = d;
-                    nearest[i] = b;
+        if (!walls.empty()) {
+            const NearestWall search(bc, walls, m.xy);
+#pragma omp parallel
+            {
+                int last = 0;
+#pragma omp for schedule(static)
+                for (int i = 0; i < static_cast<int>(nearest.size()); ++i) {
+                    if (A.wdist[i] == 0.0) continue;
+                    search.find(cxv[i], cyv[i], m.xy, &last);
+                    nearest[i] = walls[last];
                 }
             }
         }
