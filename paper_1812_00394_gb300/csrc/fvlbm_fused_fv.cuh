@@ -661,6 +661,14 @@ __host__ __device__ constexpr size_t fv_acc_at(size_t i, int alpha) {
 // f^(2), f^(3) (cell-major rows); fs_out: stages 1, 2 write f^(2), f^(3) cell-major; fn: stage 3
 // writes f^{n+1}; geo: the geometry rows, cutc: the cut faces' coefficients.  STAGE 4 is the explicit
 // Euler step: fin f^n, fs_out f^{n+1} (structure of arrays, another buffer: neighbours read f^n).
+//
+// What bounds it.  Float: the chain inside a CTA (ids, rows, face values, barrier, flux, algebra)
+// at 24 warps an SM, neither memory nor issue alone.  A 2.57M-cell batch takes 145 + 119 + 109 us
+// for the stages (2.9, 4.3 and 3.3 TB/s of state words; 47 % of the issue slots in stage 1), 217 +
+// 174 + 156 before cut faces, ghost rows and byte addresses took the warp instructions of 640k cells
+// from 27.5 / 23.5 / 19.9 M to 21.6 / 16.2 / 13.4 M.  Double: the FP64 pipe, 84 to 87 % busy (one warp
+// instruction holds a scheduler for 64 cycles, compares and conversions too), so operations are
+// what is saved: 640k cells, 475 + 292 + 223 us.
 template <class T, int STAGE, bool STATS, int IT>
 __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ? 3 : 1) : (IT == 256 ? 2 : 1))
     k_fused_fv(const T *fin, T *__restrict__ fs_out, T *__restrict__ fn, T *Bacc, T *Cacc, const T *tau, T *mac, double *__restrict__ partial, Geo<T> G, FvItems W,

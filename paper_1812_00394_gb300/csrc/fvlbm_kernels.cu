@@ -9,7 +9,14 @@
 // deterministic.
 //
 // Step (Sec. 3.2, Steps 1-7) as launched per time step:
-//   [k_sst_grad, k_sst_update]      Step 1 (k-omega SST, Eq. (SSTequint), Eq. (turbtau))
+//   [k_sst_grad, k_sst_update]      Step 1 (k-omega SST, Eq. (SSTequint), Eq. (turbtau)); in double
+//                                   and for tangents the kernels of fvlbm_sst64.cuh
+//   k_fused_fv<T, J>, J = 1, 2, 3   one kernel a stage (fvlbm_fused_fv.cuh): Gamma^a(f^(J)) (Eq.
+//                                   (advection)) and the next stage's solve, Eq. (imextwo) and the
+//                                   macros in the third (Steps 2-7).  Explicit Euler is one launch
+//                                   of the same kernel.  Small FP64 handles run fvlbm_lanes.cuh,
+//                                   tangents fvlbm_tangent.cuh.
+// and with kernel_path 1, the reading variants 1 and 4, or items that do not fit, as two-pass kernels:
 //   k_stage1                        stage 1: f^(1) from f^n (Eq. (fnewstage), J = 1)
 //   k_grad, k_flux_stage<1>         Gamma^a(f^(1)) (Eq. (advection)); stage 2 solve
 //   k_grad, k_flux_stage<2>         Gamma^a(f^(2)); stage 3 solve
@@ -694,7 +701,7 @@ __global__ void k_reduce_instances(const double *__restrict__ partial,
 #include "fvlbm_fused_fv.cuh"
 
 // ------------------------------------------------------------------ SST (Step 1)
-// ---- per-cell SST arithmetic, shared by the two-pass and the fused kernels
+// ---- per-cell SST arithmetic, with geometry read as stored or derived on chip (COMPACT)
 // Boundary values of (u, v, k, omega) on boundary face b of a cell with values (ui, vi, ki, wi)
 // and wall distance di (Menter 1994 boundary conditions; wall omega = 60 nu / (beta1 d^2)).
 template <class T>
@@ -1044,8 +1051,8 @@ __global__ void __launch_bounds__(kTile)
     }
 }
 
-// The k / omega update and the new relaxation time.  In
-// float, 5 blocks of 128 per SM (96 registers, a few spilled) run faster than 4 (120).
+// The k / omega update and the new relaxation time.  In float, 5 blocks of 128 per SM (96 registers, a
+// few spilled): 80.1 us on the 2.57M-cell batch, against 93.6 with 4 and 90.8 to 94.2 with 6, 7 and 8.
 // NONORTH compiles the SST reading variants in (2: non-orthogonal diffusion correction, 8:
 // production limiter); without them the kernel keeps the register count (and occupancy) of
 // the default reading.
@@ -1612,7 +1619,7 @@ void dispatch(int precision, F &&f) {
         f(Dual());
 }
 
-// The fused stage kernels exist for double and float; the tangent type runs the two-pass kernels.
+// The face-value kernels exist for double and float; the tangent type has its own (fvlbm_tangent.cuh).
 template <class T>
 constexpr bool kHasFused = !std::is_same<T, Dual>::value;
 
