@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(kTile)
             for (int a = 0; a < kQ; ++a) {
                 const T en = edot<T>(a, snx, sny);
                 T fv;
-                if (nonneg(en))
+                if (en >= T(0))
                     fv = fi[a] + g[(2 * a) * np + i] * rox + g[(2 * a + 1) * np + i] * roy;
                 else
                     fv = fs[a * np + nb] + g[(2 * a) * np + nb] * rnx + g[(2 * a + 1) * np + nb] * rny;
