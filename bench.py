@@ -358,7 +358,7 @@ def run_ours(args):
     hbm, peak_kind = _peaks()
     lam_cells = total_cells - sst_cells
     face_value = results["f32"]["autotune"][0] == "facevalue"
-    kbytes = _kernel_bytes(kname, "f32", total_cells, sst_cells, face_value)
+    kbytes = _kernel_bytes(kname, "f32", total_cells, sst_cells)
     achieved = kbytes / (per_launch_ms * 1e-3) / 1e9
     step_bytes = lam_cells * STEP_BYTES[("f32", False)] + sst_cells * STEP_BYTES[("f32", True)]
     step_gbs = step_bytes / (ms32 / args.steps * 1e-3) / 1e9
@@ -419,7 +419,7 @@ def run_ours(args):
                                   "ms_per_step": results["f32"]["autotune"][1]},
                          "fp64": {"chosen": results["f64"]["autotune"][0],
                                   "ms_per_step": results["f64"]["autotune"][1]}},
-            "kernels": {k: _kernel_line(k, v, total_cells, sst_cells, face_value, hbm)
+            "kernels": {k: _kernel_line(k, v, total_cells, sst_cells, hbm)
                         for k, v in prof.items()},
             "cpu_baseline": cpu,
             "e2e": e2e,
@@ -448,14 +448,16 @@ def _workload_desc(name):
                            "step, 2 SST NACA0012 C-meshes"}[name]
 
 
-PROFILE_SUMMARY = {False: "k_fused_stage_fp32_sweep.md", True: "k_fused_fv_fp32_sweep.md"}
+PROFILE_SUMMARY = {False: "sweep_fp32_twopass_launches.md", True: "k_fused_fv_fp32_sweep.md"}
+FP64_COUNTS = {"twopass": "k_flux_stage_fp64_sweep.md", "facevalue": "k_fused_fv_fp64_sweep.md"}
 
 
 def kernel_source_sha256() -> str:
-    """SHA-256 over the sources of the stage kernels (fvlbm_kernels.cu, fvlbm_fused_fv.cuh)."""
+    """SHA-256 over the sources of a step's kernels (fvlbm_kernels.cu, fvlbm_fused_fv.cuh,
+    fvlbm_sst64.cuh)."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("fvlbm_kernels.cu", "fvlbm_fused_fv.cuh"):
+    for name in ("fvlbm_kernels.cu", "fvlbm_fused_fv.cuh", "fvlbm_sst64.cuh"):
         with open(os.path.join(ROOT, "paper_1812_00394_gb300", "csrc", name), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
@@ -487,7 +489,7 @@ def _ncu_traffic(kname, workload, world, face_value=False):
 
 def _fp64_roofline(fvlbm, dev, cells, sst_cells, ms_per_step, workload, config):
     """The FP64 path against the FP64 pipe: FP64 flops per step (from the committed ncu count of
-    the two-pass kernels' DADD, DMUL and DFMA instructions, per cell and per SST cell, valid
+    the DADD, DMUL and DFMA instructions of the kernels that ran, per cell and per SST cell, valid
     while the kernel sources hash to the recorded value) over the measured FMA peak."""
     import re
     try:
@@ -496,34 +498,35 @@ def _fp64_roofline(fvlbm, dev, cells, sst_cells, ms_per_step, workload, config):
         return {"bound": "alu", "pipe": "fp64", "peak": None, "error": str(e)}
     out = {"bound": "alu", "pipe": "fp64", "peak": peak, "unit": "TFLOP/s",
            "peak_kind": "measured FP64 FMA rate (fvlbm_fp64_peak)", "achieved": None, "frac": None}
-    if workload != "sweep" or config != "twopass":
-        out["source"] = "flop counts are for the two-pass kernels on the sweep only"
+    if workload != "sweep" or config not in FP64_COUNTS:
+        out["source"] = "flop counts are for the two-pass and the face-value kernels on the sweep only"
         return out
+    fname = FP64_COUNTS[config]
     try:
-        with open(os.path.join(ROOT, "profiles", "k_flux_stage_fp64_sweep.md")) as fh:
+        with open(os.path.join(ROOT, "profiles", fname)) as fh:
             txt = fh.read()
     except OSError:
-        out["source"] = "profiles/k_flux_stage_fp64_sweep.md not found"
+        out["source"] = f"profiles/{fname} not found"
         return out
     m = re.search(r"kernel_source_sha256=([0-9a-f]{64}) fp64_flops_per_cell=([0-9.e+]+) "
                   r"fp64_flops_per_sst_cell=([0-9.e+]+)", txt)
     if not m or m.group(1) != kernel_source_sha256():
-        out["source"] = "profiles/k_flux_stage_fp64_sweep.md was counted on other kernel sources"
+        out["source"] = f"profiles/{fname} was counted on other kernel sources"
         return out
     flops = cells * float(m.group(2)) + sst_cells * float(m.group(3))
     out.update(flops_per_step=flops, achieved=flops / (ms_per_step * 1e-3) / 1e12,
-               source="ncu instruction counts committed in profiles/k_flux_stage_fp64_sweep.md")
+               source=f"ncu instruction counts committed in profiles/{fname}")
     out["frac"] = out["achieved"] / peak
     return out
 
 
-def _kernel_line(kname, v, cells, sst_cells, face_value, hbm):
+def _kernel_line(kname, v, cells, sst_cells, hbm):
     """Average launch time of one kernel and, where its algorithmic bytes are defined, its
     achieved GB/s and fraction of the measured HBM peak."""
     ms = v["ms"] / v["launches"]
     out = {"avg_ms": ms, "launches": v["launches"]}
     try:
-        b = _kernel_bytes(kname, "f32", cells, sst_cells, face_value)
+        b = _kernel_bytes(kname, "f32", cells, sst_cells)
     except KeyError:
         return out
     gbs = b / (ms * 1e-3) / 1e9
@@ -531,15 +534,12 @@ def _kernel_line(kname, v, cells, sst_cells, face_value, hbm):
     return out
 
 
-def _kernel_bytes(kname, prec, cells, sst_cells, face_value=False):
+def _kernel_bytes(kname, prec, cells, sst_cells):
     """Algorithmic bytes of one launch of each kernel: its per-cell state reads and writes
     counted once (neighbour values assumed reused from cache), neighbour indices 4 B each
-    (3.5 per cell), geometry not counted (recomputable).  With the face-value stages the SST
-    update writes no f^(1) (stage 1 relaxes f^n itself)."""
+    (3.5 per cell), geometry not counted (recomputable)."""
     w = 4 if prec == "f32" else 8
     idx = 14.0
-    if face_value and kname == "sst_update":
-        return sst_cells * ((3 + 3 + 12 + 1 + 4) * w + idx)
     words = {
         "stage1": 9 + 1 + 9,                       # f^n, tau -> f^(1)
         "grad_f": 9 + 18,                          # f^(J) -> gradient
@@ -547,7 +547,7 @@ def _kernel_bytes(kname, prec, cells, sst_cells, face_value=False):
         "flux_stage2": 9 + 18 + 18 + 1 + 18,       # f2, g, B, C, tau -> f3, C
         "flux_stage3": 9 + 18 + 9 + 1 + 9 + 3,     # f3, g, C, tau -> f^{n+1}, macros
         "sst_grad": 3 + 2 + 1 + 12 + 1,
-        "sst_update": 3 + 3 + 12 + 1 + 4 + 9 + 9,  # + f^n -> f^(1) (fused path)
+        "sst_update": 3 + 3 + 12 + 1 + 4,
         "fused_stage1": 9 + 1 + 27,                # f^n, tau -> f2, B, C (gradient in smem)
         "fused_stage2": 9 + 18 + 1 + 18,           # f2, B, C, tau -> f3, C
         "fused_stage3": 9 + 9 + 1 + 12,            # f3, C, tau -> f^{n+1}, macros

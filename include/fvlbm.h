@@ -96,17 +96,17 @@ typedef struct {
     const double *v_init;      /* [n_cells] or NULL (0) */
     const double *k_init;      /* [n_cells] or NULL (0) */
     const double *omega_init;  /* [n_cells] or NULL (1) */
-    int kernel_path;           /* 0: fused stage kernels with shared-memory halo staging
-                                  (default); 1: two-pass kernels (gradient array in HBM);
-                                  2: fused stage kernels in the face-value form (each cell
-                                  publishes its upwind face values once per face; the
-                                  autotuner may still pick any fused form).
-                                  FVLBM_FP32_DEV handles run the face-value form for 0 and 2
-                                  (two-pass where its items do not fit): the 256- and
-                                  128-cell forms derive the least-squares weights on chip,
-                                  which in FP32 leaves wall cells of high aspect ratio with
-                                  few correct digits; the face-value and two-pass kernels
-                                  read weights formed in FP64 on the host.
+    int kernel_path;           /* 0 and 2: the stages in the face-value form (default), one fused
+                                  kernel a stage with its halo staged in shared memory; each
+                                  cell publishes its upwind face values once per face.  Small
+                                  FVLBM_FP64 handles run the same stages with four threads per
+                                  cell, FVLBM_FP64_TANGENT handles as face-value kernels of
+                                  their own, scheme 1 as one kernel a step.
+                                  1: two-pass kernels (gradient array in device memory), which
+                                  also run where the items of the face-value form do not fit and
+                                  for the variants 1 and 4.  Both forms read weights formed in
+                                  FP64 on the host: forming them in FP32 would leave wall cells
+                                  of high aspect ratio with few correct digits.
                                   A handle with a periodic pair whose edges are translates only
                                   to the gluing tolerance (not to 1e-12 of the edge length)
                                   runs the two-pass kernels: they give both sides of the glued
@@ -206,18 +206,19 @@ int fvlbm_check_mesh(const fvlbm_mesh *mesh, const fvlbm_bc *bc, const fvlbm_par
 int fvlbm_step(fvlbm_handle *h, int n_steps, fvlbm_stats *stats);
 
 /* Diagnostic for the error path above (not in the paper): the number of polls the first
- * staging wait of the fused stage kernels (both fused forms: kernel_path 0 with 256- and
- * 128-cell blocks, and the face-value form of kernel_path 2) makes before giving up; default
- * 2^26, 0 gives up at once, without polling.  Only that wait changes: before a block returns it
+ * staging wait of the fused stage kernels makes before giving up; default 2^26, 0 gives up at
+ * once, without polling.  With another limit than the default, small FVLBM_FP64 handles run the
+ * fused kernels too (their own have no such wait).  Only that wait changes: before a block returns it
  * still waits, with the full bound, for its own copies in flight, so that no copy lands in
  * shared memory after the block has left.  Drops the captured step graphs.
  * Errors: BAD_PARAM. */
 int fvlbm_set_wait_limit(fvlbm_handle *h, long long polls);
 
-/* Diagnostic (not in the paper): the work items of the face-value stages (kernel_path 2).
- * *nitem: items (256-cell blocks, or their halves / quarters); *n_split: 256-cell blocks split
- * because their ring-1 + ring-2 halo did not fit the shared memory; *n_overflow: items whose
- * halo has more than 192 cells (its ids continue in a second table).  All 0 when the handle
+/* Diagnostic (not in the paper): the work items of the face-value stages.
+ * *nitem: items (blocks of 256 cells, of 64 on small handles, or their halves, quarters and
+ * eighths); *n_split: blocks split because their ring-1 + ring-2 halo or their cut faces did not
+ * fit the shared memory; *n_overflow: items whose halo has more than the 192 cells (128 in 64-cell
+ * items) of its first table (its ids continue in a second table).  All 0 when the handle
  * has no face-value items.  Lets a test check that a mesh exercises those paths.
  * Errors: BAD_PARAM (null pointer). */
 int fvlbm_fv_items(fvlbm_handle *h, int *nitem, int *n_split, int *n_overflow);
@@ -341,13 +342,13 @@ int fvlbm_profile_kernels(fvlbm_handle *h, int n_steps, int max_kernels, char *n
                           double *ms, int *launches);
 
 /* Kernel autotuner (not in the paper).  Times trial_steps steps of each kernel configuration the
- * handle supports -- 0: fused stages with 256-cell blocks, 1: fused stages with 128-cell blocks,
- * 2: two-pass kernels, 3: fused stages in the face-value form -- on a snapshot of the current
- * state, restores the state exactly, and keeps the fastest for all later steps.  *chosen (may
- * be NULL) receives the configuration and ms_per_step[4] (may be NULL) the measured
- * milliseconds per step, -1 for configurations not
- * available (a block's halo too large for shared memory, kernel_path 1, the explicit
- * scheme, or configurations 0 and 1 on FVLBM_FP32_DEV handles, see kernel_path).  Allocates a temporary snapshot of the state (about 28 words per cell) and
+ * handle supports -- 2: two-pass kernels, 3: stages in the face-value form -- on a snapshot of the
+ * current state, restores the state exactly, and keeps the fastest for all later steps.  *chosen
+ * (may be NULL) receives the configuration and ms_per_step[4] (may be NULL) the measured
+ * milliseconds per step, -1 for configurations not available: 0 and 1 always (numbers of forms
+ * that no longer exist), 2 and 3 where there is nothing to choose (kernel_path 1, the explicit
+ * scheme, tangents, variants 1 and 4, items that do not fit); *chosen is then what the handle runs.
+ * Allocates a temporary snapshot of the state (about 28 words per cell) and
  * synchronises the stream.  Errors: BAD_PARAM, OOM, CUDA. */
 int fvlbm_autotune(fvlbm_handle *h, int trial_steps, int *chosen, double *ms_per_step);
 
@@ -362,8 +363,7 @@ int fvlbm_autotune(fvlbm_handle *h, int trial_steps, int *chosen, double *ms_per
  * closed-form implicit collision, the SST update and tau = (nu + nu_t) / c_s^2).  Where the step
  * is not differentiable (upwind switch on e.n = 0, limiter and clip branches, the nu_t limiter's
  * min), the derivative of the branch the value takes is carried.  The values equal those of an
- * FVLBM_FP64 handle with kernel_path 1 up to rounding (the compiler may fuse multiply-adds
- * differently).
+ * FVLBM_FP64 handle up to rounding (the order of operations differs).
  *
  * fvlbm_tangent_seed sets dp of the inputs p acts on, for `instance` (FVLBM_ALL_INSTANCES is not
  * accepted):
