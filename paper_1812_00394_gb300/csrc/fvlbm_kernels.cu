@@ -2981,6 +2981,14 @@ int fvlbm_step(fvlbm_handle *h, int n_steps, fvlbm_stats *stats) {
     }
     // the rest are plain launches: they overlap each other (dep_wait), which graphs of one step do
     // not (10k-cell cavity: 18 us per step from such graphs, 12.6 from launches)
+    // On a stream that is being captured, a laminar handle's steps are refused: an Euler step swaps two
+    // buffers on the host, which a replay would not.  (SST handles may be captured, in even numbers of
+    // steps: their ping-pong is then back where it was.)
+    if (remaining > 0 && !h->sst) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CK(cudaStreamIsCapturing(h->stream, &cap));
+        if (cap != cudaStreamCaptureStatusNone) return FVLBM_ERR_CUDA;
+    }
     for (; remaining > 0; --remaining, ++h->steps) enqueue(h, false);
     if (want_stats) {
         enqueue(h, true);
