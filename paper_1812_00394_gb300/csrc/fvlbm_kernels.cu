@@ -2149,6 +2149,14 @@ int build_graph(fvlbm_handle *h, int nsteps, cudaGraphExec_t *out) {
     return FVLBM_OK;
 }
 
+// FVLBM_ERR_CUDA on a stream that is being captured.  For calls that advance the handle's buffers on
+// the host and then wait for the stream: the wait would fail with nothing run and the buffers advanced.
+int refuse_capture(const fvlbm_handle *h) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(h->stream, &cap));
+    return cap == cudaStreamCaptureStatusNone ? FVLBM_OK : FVLBM_ERR_CUDA;
+}
+
 // Outgoing bits of every (cell, face slot) at [m * np + cell]: bit p set when the first member of
 // direction pair p leaves the cell through the face, decided once per face from the FP64 normal of
 // one side (e_alpha . n >= 0, the upwind rule of Eq. (advection)) and complemented on the other.
@@ -2967,6 +2975,14 @@ int fvlbm_step(fvlbm_handle *h, int n_steps, fvlbm_stats *stats) {
     CK(cudaSetDevice(h->device));
     int remaining = n_steps;
     const bool want_stats = stats != nullptr && n_steps > 0;
+    // On a stream that is being captured, a laminar handle's steps are refused: an Euler step swaps two
+    // buffers on the host, which a replay would not.  (SST handles may be captured, in even numbers of
+    // steps: their ping-pong is then back where it was.)  So are statistics, which wait for the stream,
+    // and runs that replay a graph of their own: all before anything of the handle has changed.
+    if (n_steps > 0 && (want_stats || !h->sst || n_steps >= kGraphSteps)) {
+        const int rc = refuse_capture(h);
+        if (rc) return rc;
+    }
     if (want_stats) --remaining;  // the last step runs un-captured with the reductions
     // graphs: an even number of steps keeps the ping-pong parity of SST runs
     while (remaining >= kGraphSteps) {
@@ -2981,14 +2997,6 @@ int fvlbm_step(fvlbm_handle *h, int n_steps, fvlbm_stats *stats) {
     }
     // the rest are plain launches: they overlap each other (dep_wait), which graphs of one step do
     // not (10k-cell cavity: 18 us per step from such graphs, 12.6 from launches)
-    // On a stream that is being captured, a laminar handle's steps are refused: an Euler step swaps two
-    // buffers on the host, which a replay would not.  (SST handles may be captured, in even numbers of
-    // steps: their ping-pong is then back where it was.)
-    if (remaining > 0 && !h->sst) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        CK(cudaStreamIsCapturing(h->stream, &cap));
-        if (cap != cudaStreamCaptureStatusNone) return FVLBM_ERR_CUDA;
-    }
     for (; remaining > 0; --remaining, ++h->steps) enqueue(h, false);
     if (want_stats) {
         enqueue(h, true);
@@ -3606,6 +3614,8 @@ int fvlbm_profile_kernels(fvlbm_handle *h, int n_steps, int max_kernels, char *n
                           int *launches) {
     if (!h || n_steps <= 0) return FVLBM_ERR_BAD_PARAM;
     CK(cudaSetDevice(h->device));
+    const int rc = refuse_capture(h);
+    if (rc) return rc;
     h->profiling = true;
     h->timers.clear();
     for (int k = 0; k < n_steps; ++k) enqueue(h, false);
@@ -3647,6 +3657,8 @@ int fvlbm_autotune(fvlbm_handle *h, int trial_steps, int *chosen, double *ms_per
         if (chosen) *chosen = h->config;
         return FVLBM_OK;
     }
+    const int refused = refuse_capture(h);
+    if (refused) return refused;
     // snapshot of the state a step reads (the rest is scratch)
     const std::vector<std::pair<void *, size_t>> st = state_regions(h);
     size_t total = 0;
