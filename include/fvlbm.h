@@ -200,8 +200,11 @@ int fvlbm_check_mesh(const fvlbm_mesh *mesh, const fvlbm_bc *bc, const fvlbm_par
 /* Advance n_steps time steps (Steps 1-7 of Sec. 3.2 each), asynchronously on the handle's
  * stream.  Runs of 16 steps are replayed from a captured CUDA graph, the rest are launches.  On a
  * stream that the caller captures, laminar handles, runs of 16 steps and statistics return
- * FVLBM_ERR_CUDA and change nothing (so do fvlbm_profile_kernels and fvlbm_autotune); an even number
- * of SST steps below that may be captured.  When `stats` is non-NULL the
+ * FVLBM_ERR_CUDA and change nothing (so do fvlbm_profile_kernels and fvlbm_autotune).  Fewer steps
+ * of an SST handle may be captured and replayed any number of times (an odd number copies k, omega
+ * and nu_t, and f of scheme 1, once more).  k, omega and nu_t alternate between two buffers from one
+ * step to the next, and captured calls keep to those of the capture: between capture and replay the
+ * handle takes an even number of other steps.  When `stats` is non-NULL the
  * call synchronises and fills it (FP64 residual of the last step, mass, NaN watchdog) and
  * returns FVLBM_ERR_DIVERGED if the state is not finite.  It also reads the device flag that
  * the fused stage kernels set when a staging wait gave up: FVLBM_ERR_TIMEOUT then (the flag is

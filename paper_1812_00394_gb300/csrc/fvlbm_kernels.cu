@@ -2157,6 +2157,29 @@ int refuse_capture(const fvlbm_handle *h) {
     return cap == cudaStreamCaptureStatusNone ? FVLBM_OK : FVLBM_ERR_CUDA;
 }
 
+// On a capturing stream: the state that an odd number of steps left in the other k / omega / nu_t (and,
+// explicit Euler with SST, f) buffers goes back to where the steps found it, so that the captured steps
+// replay any number of times.  Not on a capturing stream: nothing to do.
+int keep_buffers(fvlbm_handle *h, int turb0, int parity0) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(h->stream, &cap));
+    if (cap == cudaStreamCaptureStatusNone) return FVLBM_OK;
+    size_t ts = 0;
+    dispatch(h->precision, [&](auto z_) { ts = sizeof(z_); });
+    const size_t bytes = ts * static_cast<size_t>(h->np);
+    if (h->turb != turb0) {
+        for (void **b : {h->kk, h->ww, h->nut})
+            CK(cudaMemcpyAsync(b[turb0], b[h->turb], bytes, cudaMemcpyDeviceToDevice, h->stream));
+        h->turb = turb0;
+    }
+    if (h->fn_parity != parity0) {
+        CK(cudaMemcpyAsync(h->s0, h->fn, kQ * bytes, cudaMemcpyDeviceToDevice, h->stream));
+        std::swap(h->fn, h->s0);
+        h->fn_parity = parity0;
+    }
+    return FVLBM_OK;
+}
+
 // Outgoing bits of every (cell, face slot) at [m * np + cell]: bit p set when the first member of
 // direction pair p leaves the cell through the face, decided once per face from the FP64 normal of
 // one side (e_alpha . n >= 0, the upwind rule of Eq. (advection)) and complemented on the other.
@@ -2976,9 +2999,9 @@ int fvlbm_step(fvlbm_handle *h, int n_steps, fvlbm_stats *stats) {
     int remaining = n_steps;
     const bool want_stats = stats != nullptr && n_steps > 0;
     // On a stream that is being captured, a laminar handle's steps are refused: an Euler step swaps two
-    // buffers on the host, which a replay would not.  (SST handles may be captured, in even numbers of
-    // steps: their ping-pong is then back where it was.)  So are statistics, which wait for the stream,
-    // and runs that replay a graph of their own: all before anything of the handle has changed.
+    // buffers on the host, which a replay would not.  (SST handles may be captured: see keep_buffers.)
+    // So are statistics, which wait for the stream, and runs that replay a graph of their own: all before
+    // anything of the handle has changed.
     if (n_steps > 0 && (want_stats || !h->sst || n_steps >= kGraphSteps)) {
         const int rc = refuse_capture(h);
         if (rc) return rc;
@@ -2997,7 +3020,12 @@ int fvlbm_step(fvlbm_handle *h, int n_steps, fvlbm_stats *stats) {
     }
     // the rest are plain launches: they overlap each other (dep_wait), which graphs of one step do
     // not (10k-cell cavity: 18 us per step from such graphs, 12.6 from launches)
+    const int turb0 = h->turb, parity0 = h->fn_parity;
     for (; remaining > 0; --remaining, ++h->steps) enqueue(h, false);
+    if (!want_stats && (h->turb != turb0 || h->fn_parity != parity0)) {  // an odd number of steps
+        const int rc = keep_buffers(h, turb0, parity0);
+        if (rc) return rc;
+    }
     if (want_stats) {
         enqueue(h, true);
         ++h->steps;

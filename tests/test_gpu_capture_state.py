@@ -1,5 +1,6 @@
-"""What a stream capture leaves behind: calls that are refused change nothing.  Every comparison is bit
-for bit with a handle that was never captured."""
+"""What a stream capture leaves behind: calls that are refused change nothing, and a captured number of
+SST steps replays in any number.  Every comparison is bit for bit with a handle that was never
+captured: a replay launches the same kernels on the same values."""
 import numpy as np
 import pytest
 
@@ -52,5 +53,61 @@ def test_refused_calls_leave_the_state(make, scheme, prec):
         a, b = s.step(2, stats=True), ref.step(done + 2, stats=True)
         assert a == b
         _same(s, ref)
+        s.close()
+        ref.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3])
+@pytest.mark.parametrize("scheme,path", [(IMEX, 0), (IMEX, 1), (EULER, 0), (EULER, 1)],
+                         ids=["imex", "imex-twopass", "euler", "euler-twopass"])
+@pytest.mark.parametrize("prec", [FP64, FP32], ids=["fp64", "fp32"])
+def test_captured_sst_steps_replay_in_any_number(prec, scheme, path, n):
+    import torch
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        s = fvlbm.Solver(_sst(), precision=prec, device=0, stream=st.cuda_stream, scheme=scheme, kernel_path=path)
+        ref = fvlbm.Solver(_sst(), precision=prec, device=0, scheme=scheme, kernel_path=path)
+        s.step(1)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            s.step(n)
+        ref.step(1)
+        _same(s, ref)           # capturing runs nothing
+        for _ in range(3):
+            g.replay()
+        torch.cuda.synchronize()
+        ref.step(3 * n)
+        _same(s, ref)
+        s.step(1)
+        ref.step(1)
+        _same(s, ref)
+        s.close()
+        ref.close()
+
+
+def test_a_captured_step_and_exchange_of_an_sst_handle():
+    """One capture of two rounds of a step and a pack: every call of it stands for itself."""
+    import torch
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        s = fvlbm.Solver(_sst(), precision=FP32, device=0, stream=st.cuda_stream)
+        ref = fvlbm.Solver(_sst(), precision=FP32, device=0, stream=st.cuda_stream)
+        n = s.cells[0]
+        ls, lr = s.set_exchange_list(np.arange(n)), ref.set_exchange_list(np.arange(n))
+        rows, want = (torch.zeros((2, n, 12), dtype=torch.float64, device="cuda") for _ in range(2))
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            for q in range(2):
+                s.step(1)
+                s.pack_cells_dev(ls, rows[q].data_ptr())
+        for _ in range(2):
+            g.replay()
+            for q in range(2):
+                ref.step(1)
+                ref.pack_cells_dev(lr, want[q].data_ptr())
+            torch.cuda.synchronize()
+            assert torch.equal(rows, want)
         s.close()
         ref.close()
