@@ -295,7 +295,8 @@ int fvlbm_forces_edges(fvlbm_handle *h, int instance, double *fxy);
  * fvlbm_unpack_cells_dev: the reverse, as fvlbm_set_cells with all four fields (the macros
  * follow f).  Both are enqueued on the handle's stream and do not synchronise: vals must stay
  * valid until that work has run, and a caller that moves vals on another stream orders it
- * against the handle's stream.  Errors: BAD_PARAM (unknown list, NULL vals), CUDA. */
+ * against the handle's stream.  Both may be captured; a replay works on the f of that time (k, omega
+ * and nu_t: see fvlbm_step).  Errors: BAD_PARAM (unknown list, NULL vals), CUDA. */
 /* FP64 arithmetic peak of `device` (the current device when < 0), measured (no counterpart in
  * the paper): the rate of double-precision fused multiply-adds of a kernel that runs
  * independent FMA chains on every SM and reads no memory, in TFLOP/s (2 flops per FMA), the

@@ -128,6 +128,8 @@ struct FvItems {
     const int4 *__restrict__ ghost;     // ghosts: owner row, boundary face, owner cell, face slot
     int *__restrict__ err;              // set to 1 if the bulk-copy wait gave up
     long long wait_first;               // polls of that wait (fvlbm_set_wait_limit)
+    int *__restrict__ cur;              // explicit Euler: takes next, the number of the buffer that
+    int next;                           // f^{n+1} goes to (see k_pack_cells)
 };
 
 // Pair p: first members alpha = 1, 2, 5, 6 and their opposites 3, 4, 7, 8.
@@ -737,6 +739,7 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
     };
     if (cut0) load_cut(cu >> 1);
     dep_wait();  // f, the accumulators and tau of the kernels before
+    if (STAGE == 4 && blockIdx.x == 0 && t == 0) *W.cur = W.next;
     if ((t & 31) == 0) {
         const unsigned row = static_cast<unsigned>(cnt * sizeof(T));
         // copies: (stages 2, 3) the item's f rows and f_0, then the accumulator rows (stage 1:

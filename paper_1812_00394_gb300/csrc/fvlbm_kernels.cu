@@ -1369,11 +1369,15 @@ __global__ void k_set_wdist(T *__restrict__ wdist, const int *__restrict__ map, 
 
 // Ghost exchange of a split mesh on device buffers: row j of vals (kXRow doubles) holds cell
 // map[j]'s f (absolute: deviation + w_alpha rho0), k, omega, nu_t (current buffers).
+// Where f^n alternates between two buffers (explicit Euler in one kernel), *cur says on the device
+// which it is, f or f1, so that a captured exchange replays after any number of steps; else cur is null.
 template <class T>
 __global__ void __launch_bounds__(kIoBlock)
-    k_pack_cells(const T *__restrict__ f, const T *__restrict__ kk, const T *__restrict__ ww,
+    k_pack_cells(const T *__restrict__ f, const T *__restrict__ f1, const int *__restrict__ cur,
+                 const T *__restrict__ kk, const T *__restrict__ ww,
                  const T *__restrict__ nut, const int *__restrict__ map, int n, Geo<T> G, double *__restrict__ vals) {
     __shared__ double sm[kIoBlock * kXRow];
+    if (cur != nullptr && *cur != 0) f = f1;
     const int j0 = blockIdx.x * kIoBlock, j = j0 + threadIdx.x;
     if (j < n) {
         const int i = map[j];
@@ -1394,11 +1398,13 @@ __global__ void __launch_bounds__(kIoBlock)
 // The reverse: f^n (deviation) and the macros (as fvlbm_set_f writes them), k, omega and nu_t of
 // cell map[j] from row j of vals.
 template <class T>
-__global__ void k_unpack_cells(T *__restrict__ f, T *__restrict__ mac, T *__restrict__ kk, T *__restrict__ ww,
+__global__ void k_unpack_cells(T *__restrict__ f, T *__restrict__ f1, const int *__restrict__ cur,
+                               T *__restrict__ mac, T *__restrict__ kk, T *__restrict__ ww,
                                T *__restrict__ nut, const int *__restrict__ map, int n, Geo<T> G,
                                const double *__restrict__ vals) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
+    if (cur != nullptr && *cur != 0) f = f1;
     const int i = map[j];
     const size_t np = G.np;
     const InstParam P = G.ip[G.tile_inst[i / kTile]];
@@ -1597,6 +1603,7 @@ struct fvlbm_handle {
     // first), and from either f^n buffer (+ 2; explicit Euler on the face-value kernel)
     cudaGraphExec_t graph[4] = {nullptr, nullptr, nullptr, nullptr};
     int fn_parity = 0;
+    int *d_cur = nullptr;   // explicit Euler on the face-value kernel: fn_parity, kept on the device
     bool profiling = false;
     std::vector<KernelTimer> timers;
     std::vector<cudaEvent_t> ev_pool;
@@ -1776,7 +1783,7 @@ void fv_stages(fvlbm_handle *h, bool stats) {
     T *B = static_cast<T *>(h->bacc), *C = static_cast<T *>(h->cacc);
     T *tau = static_cast<T *>(h->tau), *mac = static_cast<T *>(h->mac);
     const auto &F = h->fv;
-    const FvItems W{F.d_hdr, F.d_halo, F.d_ovf, F.d_adj, F.d_cut, F.d_ghost, h->d_err, h->wait_first};
+    const FvItems W{F.d_hdr, F.d_halo, F.d_ovf, F.d_adj, F.d_cut, F.d_ghost, h->d_err, h->wait_first, nullptr, 0};
     const T *geo = static_cast<const T *>(F.geo), *cc = static_cast<const T *>(F.cutc);
     const T *bn = static_cast<const T *>(h->bnrm);
     const dim3 fg(static_cast<unsigned>(F.nitem)), fb(FvShape<IT>::nt);
@@ -1838,7 +1845,7 @@ void fv_euler(fvlbm_handle *h, bool stats) {
     Geo<T> G = geo_of<T>(h);
     T *fn = static_cast<T *>(h->fn), *out = static_cast<T *>(h->s0);
     const auto &F = h->fv;
-    const FvItems W{F.d_hdr, F.d_halo, F.d_ovf, F.d_adj, F.d_cut, F.d_ghost, h->d_err, h->wait_first};
+    const FvItems W{F.d_hdr, F.d_halo, F.d_ovf, F.d_adj, F.d_cut, F.d_ghost, h->d_err, h->wait_first, h->d_cur, 1 - h->fn_parity};
     launch(h, K_EULER, "euler", [&] {
         launch_dep(stats ? k_fused_fv<T, 4, true, IT> : k_fused_fv<T, 4, false, IT>, dim3(static_cast<unsigned>(F.nitem)),
                    dim3(FvShape<IT>::nt), FvSmem<T, IT>::bytes, h->stream, fn, out, fn, static_cast<T *>(h->bacc),
@@ -2149,6 +2156,10 @@ int build_graph(fvlbm_handle *h, int nsteps, cudaGraphExec_t *out) {
     return FVLBM_OK;
 }
 
+// Buffer q of f^n: the one that is current where the handle's fn_parity is q, which is what the device
+// word d_cur selects; handles whose f^n stays where it is have the one.
+void *f_buffer(const fvlbm_handle *h, int q) { return h->d_cur && q != h->fn_parity ? h->s0 : h->fn; }
+
 // FVLBM_ERR_CUDA on a stream that is being captured.  For calls that advance the handle's buffers on
 // the host and then wait for the stream: the wait would fail with nothing run and the buffers advanced.
 int refuse_capture(const fvlbm_handle *h) {
@@ -2176,6 +2187,7 @@ int keep_buffers(fvlbm_handle *h, int turb0, int parity0) {
         CK(cudaMemcpyAsync(h->s0, h->fn, kQ * bytes, cudaMemcpyDeviceToDevice, h->stream));
         std::swap(h->fn, h->s0);
         h->fn_parity = parity0;
+        CK(cudaMemsetAsync(h->d_cur, parity0, sizeof(int), h->stream));  // (0, or not 0)
     }
     return FVLBM_OK;
 }
@@ -2621,6 +2633,7 @@ int allocate_state(fvlbm_handle *h, const std::vector<const Prepared *> &P,
         if (h->fused) {
             if ((rc = build_fv_items<T>(h, nbr, back, sn, lsq, rown, gq, bowner, inst_tile0))) return rc;
             if (h->fv.ok) h->config = 3;
+            if (h->fv.ok && h->scheme == 1 && (rc = upload_raw(h, &h->d_cur, std::vector<int>(1, 0)))) return rc;
             if (std::is_same<T, double>::value && h->fv.ok && h->scheme == 0 && np <= kLaneCells) {
                 const std::vector<unsigned char> pb = outgoing_bits(np, nbr, back, sn);
                 std::vector<int> bits(np);
@@ -3279,8 +3292,9 @@ int fvlbm_pack_cells_dev(fvlbm_handle *h, int list_id, double *vals) {
         using T = decltype(z_);
         const int c = h->turb;
         k_pack_cells<T><<<(L.n + kIoBlock - 1) / kIoBlock, kIoBlock, 0, h->stream>>>(
-            static_cast<const T *>(h->fn), static_cast<const T *>(h->kk[c]), static_cast<const T *>(h->ww[c]),
-            static_cast<const T *>(h->nut[c]), L.d_map, L.n, geo_of<T>(h), vals);
+            static_cast<const T *>(f_buffer(h, 0)), static_cast<const T *>(f_buffer(h, 1)), h->d_cur,
+            static_cast<const T *>(h->kk[c]), static_cast<const T *>(h->ww[c]), static_cast<const T *>(h->nut[c]),
+            L.d_map, L.n, geo_of<T>(h), vals);
     });
     CK(cudaGetLastError());
     return FVLBM_OK;
@@ -3296,8 +3310,9 @@ int fvlbm_unpack_cells_dev(fvlbm_handle *h, int list_id, const double *vals) {
         using T = decltype(z_);
         const int c = h->turb;
         k_unpack_cells<T><<<(L.n + 255) / 256, 256, 0, h->stream>>>(
-            static_cast<T *>(h->fn), static_cast<T *>(h->mac), static_cast<T *>(h->kk[c]), static_cast<T *>(h->ww[c]),
-            static_cast<T *>(h->nut[c]), L.d_map, L.n, geo_of<T>(h), vals);
+            static_cast<T *>(f_buffer(h, 0)), static_cast<T *>(f_buffer(h, 1)), h->d_cur, static_cast<T *>(h->mac),
+            static_cast<T *>(h->kk[c]), static_cast<T *>(h->ww[c]), static_cast<T *>(h->nut[c]), L.d_map, L.n,
+            geo_of<T>(h), vals);
     });
     CK(cudaGetLastError());
     return FVLBM_OK;

@@ -1,13 +1,14 @@
-"""What a stream capture leaves behind: calls that are refused change nothing, and a captured number of
-SST steps replays in any number.  Every comparison is bit for bit with a handle that was never
-captured: a replay launches the same kernels on the same values."""
+"""What a stream capture leaves behind: calls that are refused change nothing, a captured number of SST
+steps replays in any number, and a captured exchange follows f^n between the two buffers of an
+explicit Euler handle.  Every comparison is bit for bit with a handle that was never captured: a
+replay launches the same kernels on the same values."""
 import numpy as np
 import pytest
 
 from paper_1812_00394_gb300 import fvlbm, meshgen as mg
 
 pytestmark = pytest.mark.gpu
-FP64, FP32 = fvlbm.FVLBM_FP64, fvlbm.FVLBM_FP32_DEV
+FP64, FP32, TAN = fvlbm.FVLBM_FP64, fvlbm.FVLBM_FP32_DEV, fvlbm.FVLBM_FP64_TANGENT
 IMEX, EULER = fvlbm.SCHEME_IMEX, fvlbm.SCHEME_EULER
 
 
@@ -109,5 +110,50 @@ def test_a_captured_step_and_exchange_of_an_sst_handle():
                 ref.pack_cells_dev(lr, want[q].data_ptr())
             torch.cuda.synchronize()
             assert torch.equal(rows, want)
+        s.close()
+        ref.close()
+
+
+@pytest.mark.parametrize("prec,path", [(FP64, 0), (FP32, 0), (FP32, 1), (TAN, 0)],
+                         ids=["fp64", "fp32", "fp32-twopass", "tangent"])
+def test_captured_exchange_follows_euler_steps(prec, path):
+    """Pack and unpack captured once on a laminar Euler handle, replayed after odd and even numbers of
+    steps, across a saved state and across a run from the 16-step graph."""
+    import torch
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        s, ref = (fvlbm.Solver(_laminar(), precision=prec, device=0, stream=st.cuda_stream, scheme=EULER,
+                               kernel_path=path) for _ in range(2))
+        n = s.cells[0]
+        some = np.arange(0, n, 3)
+        pack, unpack = s.set_exchange_list(np.arange(n)), s.set_exchange_list(some)
+        rpack, runpack = ref.set_exchange_list(np.arange(n)), ref.set_exchange_list(some)
+        out, want = (torch.zeros((n, 12), dtype=torch.float64, device="cuda") for _ in range(2))
+        back = torch.zeros((len(some), 12), dtype=torch.float64, device="cuda")
+        idx = torch.as_tensor(some, device="cuda")
+        torch.cuda.synchronize()
+        gp, gu = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+        with torch.cuda.graph(gp, stream=st):
+            s.pack_cells_dev(pack, out.data_ptr())
+        with torch.cuda.graph(gu, stream=st):
+            s.unpack_cells_dev(unpack, back.data_ptr())
+        blob = None
+        for steps in (1, 1, 2, 19, 1, 0, 3):
+            s.step(steps)
+            ref.step(steps)
+            if steps == 0:      # a state saved from the other buffer
+                s.load_state(blob)
+                ref.load_state(blob)
+            gp.replay()
+            ref.pack_cells_dev(rpack, want.data_ptr())
+            torch.cuda.synchronize()
+            assert torch.equal(out, want), steps
+            if blob is None:
+                blob = s.save_state()
+            back.copy_(1.001 * out[idx])
+            gu.replay()
+            ref.unpack_cells_dev(runpack, back.data_ptr())
+            torch.cuda.synchronize()
+            _same(s, ref)
         s.close()
         ref.close()
