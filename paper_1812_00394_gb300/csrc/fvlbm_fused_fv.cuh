@@ -96,7 +96,8 @@ __host__ __device__ constexpr unsigned fv_row_addr(int j) {  // halves swapped w
 // Geometry values of a cell.  Double: A_mk at 4 m + k, then (n dl / A)_m, x and y, at 16 + 2 m; a
 // triangle has no slot 3 and keeps the six normal components in the free places 3, 7, 11-14, so
 // that only 16 values are read.  Float: node positions relative to the centroid (8 values; face
-// m joins nodes m and m + 1), then the least-squares weights W_m.  Stored in 16-byte chunks,
+// m joins nodes m and m + 1), then the least-squares weights W_m; explicit Euler: the face offsets
+// r_m in place of the node positions (see k_fused_fv).  Stored in 16-byte chunks,
 // chunk c of 32 consecutive cells together, so that a warp's load of one chunk is contiguous
 // (a row per cell took 16 to 24 cache-line accesses a load, up to two fifths of all accesses to
 // L1 and shared memory).
@@ -332,10 +333,11 @@ __device__ __forceinline__ void fv_relax_to_row(float *f, float *sf, float *sf0,
 #define FV_END_Y(m) ((m) == 3 ? q[1] : ((m) == 2 && tri ? q[1] : q[2 * (m) + 3]))
 
 // Gradient (Step 2) and outgoing face values of item cell c, two pairs at a time (packed FMAs).
-// g: node positions q relative to the centroid, then least-squares weights W_m (x, y per face
-// slot); w: adjacency.
+// g: node positions q relative to the centroid (OFF: the face offsets r_m), then least-squares
+// weights W_m (x, y per face slot); w: adjacency.
 // Absent faces have weight 0 and the cell itself as datum, and values at faces without a neighbour
 // are formed but not read, so the only branch is the warp's on the fourth slot (quads).
+template <bool OFF>
 __device__ __forceinline__ void fv_cell(int c, const float *g, const unsigned *w, bool quads,
                                         const float *__restrict__ sf, float *__restrict__ sv) {
     using PV = FvPair<float>;
@@ -362,8 +364,8 @@ __device__ __forceinline__ void fv_cell(int c, const float *g, const unsigned *w
             }
         };
         auto face = [&](int m) {
-            const V rx = PV::bcast(0.5f * (q[2 * m] + FV_END_X(m)));
-            const V ry = PV::bcast(0.5f * (q[2 * m + 1] + FV_END_Y(m)));
+            const V rx = PV::bcast(OFF ? q[2 * m] : 0.5f * (q[2 * m] + FV_END_X(m)));
+            const V ry = PV::bcast(OFF ? q[2 * m + 1] : 0.5f * (q[2 * m + 1] + FV_END_Y(m)));
             float out[2];
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
@@ -496,8 +498,8 @@ __device__ __forceinline__ double2 fv_ghost_pair(int type, double rb, double ub,
 
 // Boundary values of a cell with staged row fc, f0 at ghost gh.  The face's type and values are read
 // kept in L2, like the item tables: a few hundred kB read once per launch by the items along the
-// boundaries.
-template <class T>
+// boundaries.  OFF: as in fv_cell.
+template <class T, bool OFF>
 __device__ __forceinline__ void fv_ghost(const Geo<T> &G, const T *__restrict__ bnrm, const T *__restrict__ geo,
                                          const int4 &gh, T rho0, const typename FvPair<T>::V *fc, T f0,
                                          typename FvPair<T>::V *out) {
@@ -505,11 +507,14 @@ __device__ __forceinline__ void fv_ghost(const Geo<T> &G, const T *__restrict__ 
     const unsigned long long keep = l2_keep_policy();
     const int bf = gh.y;
     const int type = ld_keep(G.btype + bf, keep);
-    if constexpr (sizeof(T) == 4) {  // boundary_values itself, the far field's normal from the owner's nodes
+    if constexpr (sizeof(T) == 4) {  // boundary_values itself, the far field's normal as the flux has it
         T bval[3], fcs[kQ], fb[kQ], dr, r, u, v, nx = T(0), ny = T(0);
 #pragma unroll
         for (int c = 0; c < 3; ++c) bval[c] = ld_keep(G.bval + static_cast<size_t>(c) * G.nbt + bf, keep);
-        if (type == FVLBM_BC_FARFIELD) {
+        if (type == FVLBM_BC_FARFIELD && OFF) {
+            nx = G.sn[static_cast<size_t>(2 * gh.w) * G.np + gh.z];
+            ny = G.sn[static_cast<size_t>(2 * gh.w + 1) * G.np + gh.z];
+        } else if (type == FVLBM_BC_FARFIELD) {
             const bool tri = G.nbr[3 * static_cast<size_t>(G.np) + gh.z] == kNone;
             const int m = gh.w, e = m == 3 || (m == 2 && tri) ? 0 : m + 1;
             nx = geo[fv_geo_at<T>(gh.z, 2 * e + 1)] - geo[fv_geo_at<T>(gh.z, 2 * m + 1)];
@@ -664,6 +669,13 @@ __host__ __device__ constexpr size_t fv_acc_at(size_t i, int alpha) {
 // writes f^{n+1}; geo: the geometry rows, cutc: the cut faces' coefficients.  STAGE 4 is the explicit
 // Euler step: fin f^n, fs_out f^{n+1} (structure of arrays, another buffer: neighbours read f^n).
 //
+// Geometry of the float Euler step: offsets and normals formed in FP64 on the host and rounded once, as
+// the two-pass kernels read them.  Formed in float from the nodes, the area of a slim rotated cell
+// cancels: on quads of aspect 1000 the largest error of f against FP64 was 6.2e-7 after 8 steps, 1.0e-7
+// now, which is what the two-pass kernels have (f comes out the same).  The normals are loaded
+// before the barrier, not with the other geometry: eight registers more would leave four 64-cell CTAs to
+// an SM instead of five.  40k-cell cavity: 5.0 us a step either way.
+//
 // What bounds it.  Float: the chain inside a CTA (ids, rows, face values, barrier, flux, algebra)
 // at 24 warps an SM, neither memory nor issue alone.  A 2.57M-cell batch takes 145 + 119 + 109 us
 // for the stages (2.9, 4.3 and 3.3 TB/s of state words; 47 % of the issue slots in stage 1), 217 +
@@ -681,6 +693,7 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
     using L = FvSmem<T, IT>;
     constexpr int NT = S::nt, HS = S::hs;
     constexpr bool SOA = STAGE == 1 || STAGE == 4;  // reads f^n
+    constexpr bool OFF = STAGE == 4 && sizeof(T) == 4;  // r_m and normals as formed in FP64 on the host
     extern __shared__ __align__(128) unsigned char smem_raw[];
     T *sf = reinterpret_cast<T *>(smem_raw + L::sf);
     T *sf0 = reinterpret_cast<T *>(smem_raw + L::sf0);
@@ -908,7 +921,7 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
             const int4 gh = W.ghost[hx.z + q];
             V f[4], b[4];
             fv_load_row(sf, gh.x, f);
-            fv_ghost<T>(G, bnrm, geo, gh, rho0, f, sf0[gh.x], b);
+            fv_ghost<T, OFF>(G, bnrm, geo, gh, rho0, f, sf0[gh.x], b);
             fv_store_row(sf, cnt + hx.x + q, b);
         }
         __syncthreads();
@@ -916,20 +929,25 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
 
     // 2. outgoing face values: item cells (thread t takes cell t) and cut faces
     const bool quads = __any_sync(0xffffffffu, w[3] < kFvNone);  // (a triangle has no fourth face)
-    if (mine) fv_cell(t, A, w, quads, sf, sv);
+    if (mine) {
+        if constexpr (sizeof(T) == 4)
+            fv_cell<OFF>(t, A, w, quads, sf, sv);
+        else
+            fv_cell(t, A, w, quads, sf, sv);
+    }
     if (cut0) fv_cut<T>(sv + 4 * (4 * IT + (cu >> 1)), cu & 1, cr, ca, sf);
     if (cu >= 0)
         for (int u = cu + CS; u < 2 * ncut; u += CS) {
             load_cut(u >> 1);
             fv_cut<T>(sv + 4 * (4 * IT + (u >> 1)), u & 1, cr, ca, sf);
         }
-    // the normals: float forms them from the node positions; double loads a quad's before the
-    // barrier (a triangle's came with its coefficients)
+    // the normals: float forms them from the node positions; explicit Euler loads them and double
+    // a quad's before the barrier (a triangle's came with its coefficients)
     T sn[8];
     if (mine) {
         if constexpr (sizeof(T) == 4) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k) sn[k] = A[k];
+            for (int k = 0; k < 8; ++k) sn[k] = OFF ? G.sn[k * np + i] : A[k];
         } else if (w[3] < kFvNone) {
             fv_load_geo4(geo, i, 16, sn);
             fv_load_geo4(geo, i, 20, sn + 4);
@@ -951,7 +969,7 @@ __global__ void __launch_bounds__(FvShape<IT>::nt, sizeof(T) == 4 ? (IT == 256 ?
             V ac[4], fr[4];
 #pragma unroll
             for (int k = 0; k < 8; ++k) q[k] = sn[k];
-            fv_normals(q, w[3] >= kFvNone, sn);
+            if (!OFF) fv_normals(q, w[3] >= kFvNone, sn);
             fv_flux<T>(t, sn, w, sf, sv, ac);
             fv_load_row(sf, t, fr);
             fi[0] = sf0[t];

@@ -1992,8 +1992,11 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
         T *nn = static_cast<T *>(h->nut[n]);
         T *sg = static_cast<T *>(h->sgrad), *f1 = static_cast<T *>(h->f1);
         const CompactGeo<T> CG{static_cast<const T *>(h->gq), static_cast<const T *>(h->dvec)};
+        // beside the one-kernel Euler step, where the SST would derive its geometry on chip, the
+        // kernels that read it as formed in FP64
+        const bool stored = h->scheme == 1 && (sizeof(T) == 4 || h->nonorth);
         if constexpr (kHasFused<T>) {
-            if (h->config != 2) {  // compact geometry, packed records
+            if (h->config != 2 && !stored) {  // compact geometry, packed records
                 T *r8 = static_cast<T *>(h->sst_rec8), *r2 = static_cast<T *>(h->sst_rec2);
                 if constexpr (std::is_same<T, double>::value) {
                     if (!h->nonorth) sst64(h, G, s, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau);
@@ -2025,7 +2028,7 @@ void enqueue_step(fvlbm_handle *h, bool stats) {
                 lean = true;
             }
         }
-        if (h->config == 2 && !lean) {
+        if ((h->config == 2 || stored) && !lean) {
             launch(h, K_SST_GRAD, "sst_grad", [&] { sst_grad_twopass<T>(h, mac, kc, wc, sg, f1, G, CG); });
             launch(h, K_SST_UPDATE, "sst_update", [&] {
                 sst_update_twopass<T>(h, mac, kc, wc, nc, sg, f1, kn, wn, nn, tau, G, CG);
@@ -2255,6 +2258,7 @@ int build_fv_items_it(fvlbm_handle *h, const std::vector<int> &nbr, const std::v
     std::vector<uint2> cut;
     std::vector<int4> ghost;
     std::vector<double> cutc;
+    const bool off = sizeof(T) == 4 && h->scheme == 1;  // see fv_cell
     // float: node positions minus centroid as the kernels read them, and the offset of face m
     // formed from them in float
     auto node = [&](size_t g, int m, int c) { return static_cast<float>(gq[(2 * m + c) * np + g]); };
@@ -2356,7 +2360,8 @@ int build_fv_items_it(fvlbm_handle *h, const std::vector<int> &nbr, const std::v
                             if constexpr (sizeof(T) == 4) {
                                 for (int k = 0; k < 8; ++k)
                                     cutc.push_back(nbr[k / 2 * np + o] == kNone ? 0.0 : lsq[k * np + o]);
-                                for (int k = 0; k < 2; ++k) cutc.push_back(mid(o, b, k));
+                                for (int k = 0; k < 2; ++k)
+                                    cutc.push_back(off ? rown[(2 * b + k) * np + o] : mid(o, b, k));
                                 cutc.resize(cutc.size() + 2, 0.0);
                             } else {
                                 for (int k = 0; k < 4; ++k)
@@ -2400,7 +2405,7 @@ int build_fv_items_it(fvlbm_handle *h, const std::vector<int> &nbr, const std::v
         auto at = [&](int v) -> double & { return geo[fv_geo_at<T>(g, v)]; };
         if constexpr (sizeof(T) == 4) {
             for (int c = 0; c < 8; ++c) {
-                at(c) = gq[c * np + g];
+                at(c) = off ? rown[c * np + g] : gq[c * np + g];
                 at(8 + c) = lsq[c * np + g];
             }
             continue;
