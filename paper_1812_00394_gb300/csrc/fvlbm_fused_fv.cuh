@@ -78,6 +78,9 @@ struct FvShape<64> {
     static constexpr int nt = 128, ecap = 224, hs = 128, ccap = 160;
 };
 
+// (an instance is a whole number of blocks: no item straddles two)
+static_assert(kBlock % 256 == 0 && kBlock % 64 == 0, "FvShape sizes");
+
 // Staged rows and value rows are named by the address of their first 16 bytes (float; doubles:
 // twice that), so that a gather takes one mask: a row address is the byte offset of half 0 of the
 // row within sf (half 1 is at that offset with bit 4 flipped), see fv_row_addr.
