@@ -955,7 +955,6 @@ int adjoint_impl(fvlbm_handle *h, int instance, int n_steps, const double *w, do
     std::vector<AdjState> snap(nsnap), st(K);
     std::vector<AdjStep> slot(K);
     AdjVars A{};
-    double *gsrc = nullptr;  // geometry adjoints of the instance, in input order
     const size_t nbt = std::max(h->nbt, 1);
     auto state = [&](AdjState &x) {
         x.f = M.get(nq);
@@ -1050,7 +1049,6 @@ int adjoint_impl(fvlbm_handle *h, int instance, int n_steps, const double *w, do
                 A.a_wd = M.get(np);
             }
             if (h->limit_f) A.a_area = M.get(np);
-            gsrc = M.get(38 * static_cast<size_t>(I.nc));
         }
     };
     carve();
@@ -1184,7 +1182,7 @@ int adjoint_impl(fvlbm_handle *h, int instance, int n_steps, const double *w, do
     std::vector<double> btab(3 * static_cast<size_t>(std::max(I.nb, 1)));
     if (dJ_dxy && I.nc > 0) {
         const size_t nc = I.nc;
-        double *d = gsrc;
+        double *d = slot[0].s1;  // in input order: 38 values a cell where the stage values were (54 and more)
         auto fetch = [&](const double *a, int runs, std::vector<double> *to) -> int {
             k_adj_gather_geo<<<(I.nc + 255) / 256, 256, 0, s>>>(a, h->d_perm + perm_offset(h, instance), I.cell_off,
                                                                I.nc, runs, np, d);
