@@ -2230,12 +2230,13 @@ std::vector<unsigned char> outgoing_bits(size_t np, const std::vector<int> &nbr,
 
 // Cells per item of the face-value kernels for a handle of np padded cells.  64-cell items spread
 // a small mesh over the 152 SMs, as long as (in float) all of them are resident at once, five to
-// an SM; beyond that 256-cell items, whose halo is smaller for their size, take over.  Both sides
-// measured, us per step, 64 against 256 cells: float cavities of 5k cells 10.7 / 12.4, 40k
-// 13.1 / 16.1, 59k 19.7 / 17.0, 199k 45 / 30; SST airfoils 40k 22.2 / 25.9, 60k 28.5 / 26.1; double
-// cavities 5k 45 / 70, 50k 116 / 120, 99k 214 / 201; SST airfoils 50k 239 / 243, 100k 387 / 379.
+// an SM by their 95 registers; beyond that 256-cell items, whose halo is smaller for their size, take
+// over.  Both sides measured, us per step, 64 against 256 cells: float cavities of 5k cells 10.0 / 11.0,
+// 48k 13.0 / 13.6, 50k 18.7 / 14.5, 198k 44 / 29; SST airfoils 40k 20.6 / 20.9, 50k 24.9 / 22.2; double
+// cavities 5k 45 / 70, 48k 116 / 122, 50k 132 / 135, 59k 140 / 121; SST airfoils 50k 162 / 169, 60k
+// 194 / 177.  (The line for double lies somewhere in 50k to 59k cells.)
 // Padded cells up to which FP64 handles take four threads per cell (fvlbm_lanes.cuh has both sides).
-constexpr size_t kLaneCells = 24576;
+constexpr size_t kLaneCells = 20480;
 template <class T>
 int fv_item_cells(size_t np) {
     return np <= (sizeof(T) == 4 ? 5 * 152 * 64 : 50000) ? 64 : 256;

@@ -15,9 +15,10 @@
 // the two kinds of kernels ran (a step with statistics runs the fused ones).  The price is the
 // part of the algebra that all four lanes repeat (a third more operations), so larger meshes,
 // which fill the schedulers anyway, keep one thread per cell.  Measured, us per step, one against
-// four threads per cell: quad cavities of 4k cells 48.7 / 33.7, 10k 54.9 / 45.1, 20k 70.6 / 68.3, 80k
-// 203 / 211; SST airfoils of 4k cells 79.6 / 54.3, 10k 84.5 / 63.8, 20k 92 / 89.  One warp a block: it is
-// placed on the emptiest scheduler, where blocks of two or four ran up to a third longer.
+// four threads per cell: quad cavities of 4k cells 49.1 / 33.8, 10k 55.2 / 44.4, 20k 71.0 / 68.5, 24k
+// 73.2 / 81.1, 80k 189 / 212; triangles 20k 64.6 / 65.1; SST airfoils of 4k cells 72.3 / 55.0, 10k
+// 73.7 / 64.4, 20k 89.1 / 88.7, 24k 94.3 / 97.7.  One warp a block: it is placed on the emptiest
+// scheduler, where blocks of two or four ran up to a third longer.
 constexpr int kLaneBlock = 32;
 
 // Layout of the stage values, B and C: pairs at [8 i + 2 p], f_0 at [8 np + i]; of the boundary
