@@ -583,6 +583,18 @@ void cell_geometry(const fvlbm_mesh &m, int i, const S *xy, const int *nbr, cons
     }
 }
 
+// One cell as a mesh of its own, whose nodes can be seeded one at a time: the cores that work on
+// geometry_adjoint need no copies of the whole mesh's nodes.
+struct SeedCell {
+    Dual xy[8];
+    int ptr[2];
+    const int nodes[4] = {0, 1, 2, 3};
+    fvlbm_mesh mesh;  // (its own node positions are not read: the functions above take xy)
+    SeedCell(const fvlbm_mesh &m, int i) : ptr{0, m.cell_ptr[i + 1] - m.cell_ptr[i]}, mesh{ptr[1], nullptr, 1, ptr, nodes} {
+        for (int k = 0; k < 2 * ptr[1]; ++k) xy[k] = Dual(m.xy[2 * m.cell_nodes[m.cell_ptr[i] + k / 2] + k % 2], 0.0);
+    }
+};
+
 }  // namespace
 
 int geometry_adjoint(const fvlbm_mesh &m, const fvlbm_bc &bc, const GeometryAdjoint &A, double *dxy,
@@ -622,16 +634,13 @@ int geometry_adjoint(const fvlbm_mesh &m, const fvlbm_bc &bc, const GeometryAdjo
         cell_area_centroid(m, i, m.xy, &ar, &cxv[i], &cyv[i]);
     }
     std::fill(dxy, dxy + 2 * static_cast<size_t>(nn), 0.0);
-    // Each cell's contributions are formed by all cores (every core seeds its own copy of the node
-    // positions), then added up in cell order, so that the sums do not depend on the cores.
+    // Each cell's contributions are formed by all cores, then added up in cell order, so that the sums do
+    // not depend on the cores.
     std::vector<double> gown(8 * static_cast<size_t>(nc)), gnbr(8 * static_cast<size_t>(nc));
-#pragma omp parallel
-    {
-    std::vector<Dual> xyd(2 * static_cast<size_t>(nn));
-    for (size_t k = 0; k < xyd.size(); ++k) xyd[k] = Dual(m.xy[k], 0.0);
-#pragma omp for schedule(static)
+#pragma omp parallel for schedule(static)
     for (int i = 0; i < nc; ++i) {
-        const int p0 = m.cell_ptr[i], nv = m.cell_ptr[i + 1] - p0;
+        SeedCell C(m, i);
+        const int nv = C.ptr[1];
         const int *nb = nbr.data() + 4 * static_cast<size_t>(i);
         Dual nbx[4], nby[4];
         for (int l = 0; l < nv; ++l)
@@ -658,25 +667,21 @@ int geometry_adjoint(const fvlbm_mesh &m, const fvlbm_bc &bc, const GeometryAdjo
             return s;
         };
         CellGeo<Dual> G;
-        for (int l = 0; l < nv; ++l) {  // own node coordinates
-            const int a = m.cell_nodes[p0 + l];
-            for (int c = 0; c < 2; ++c) {
-                xyd[2 * a + c].d = 1.0;
-                cell_geometry<Dual>(m, i, xyd.data(), nb, nbx, nby, &G);
-                xyd[2 * a + c].d = 0.0;
-                gown[8 * static_cast<size_t>(i) + 2 * l + c] = contract(G);
-            }
+        for (int k = 0; k < 2 * nv; ++k) {  // own node coordinates
+            C.xy[k].d = 1.0;
+            cell_geometry<Dual>(C.mesh, 0, C.xy, nb, nbx, nby, &G);
+            C.xy[k].d = 0.0;
+            gown[8 * static_cast<size_t>(i) + k] = contract(G);
         }
         for (int l = 0; l < nv; ++l) {  // neighbour centroids
             if (nb[l] < 0) continue;
             for (int c = 0; c < 2; ++c) {
                 (c == 0 ? nbx[l] : nby[l]).d = 1.0;
-                cell_geometry<Dual>(m, i, xyd.data(), nb, nbx, nby, &G);
+                cell_geometry<Dual>(C.mesh, 0, C.xy, nb, nbx, nby, &G);
                 (c == 0 ? nbx[l] : nby[l]).d = 0.0;
                 gnbr[8 * static_cast<size_t>(i) + 2 * l + c] = contract(G);
             }
         }
-    }
     }
     for (int i = 0; i < nc; ++i) {
         const int p0 = m.cell_ptr[i], nv = m.cell_ptr[i + 1] - p0;
@@ -734,24 +739,16 @@ int geometry_adjoint(const fvlbm_mesh &m, const fvlbm_bc &bc, const GeometryAdjo
         }
     }
     // centroid adjoints to the nodes of their cells
-#pragma omp parallel
-    {
-        std::vector<Dual> xyd(2 * static_cast<size_t>(nn));
-        for (size_t k = 0; k < xyd.size(); ++k) xyd[k] = Dual(m.xy[k], 0.0);
-#pragma omp for schedule(static)
-        for (int j = 0; j < nc; ++j) {
-            const int p0 = m.cell_ptr[j], nv = m.cell_ptr[j + 1] - p0;
-            for (int l = 0; l < nv; ++l) {
-                const int a = m.cell_nodes[p0 + l];
-                for (int c = 0; c < 2; ++c) {
-                    xyd[2 * a + c].d = 1.0;
-                    Dual ar, cx, cy;
-                    cell_area_centroid<Dual>(m, j, xyd.data(), &ar, &cx, &cy);
-                    xyd[2 * a + c].d = 0.0;
-                    gown[8 * static_cast<size_t>(j) + 2 * l + c] =
-                        dc[2 * static_cast<size_t>(j)] * cx.d + dc[2 * static_cast<size_t>(j) + 1] * cy.d;
-                }
-            }
+#pragma omp parallel for schedule(static)
+    for (int j = 0; j < nc; ++j) {
+        SeedCell C(m, j);
+        for (int k = 0; k < 2 * C.ptr[1]; ++k) {
+            C.xy[k].d = 1.0;
+            Dual ar, cx, cy;
+            cell_area_centroid<Dual>(C.mesh, 0, C.xy, &ar, &cx, &cy);
+            C.xy[k].d = 0.0;
+            gown[8 * static_cast<size_t>(j) + k] =
+                dc[2 * static_cast<size_t>(j)] * cx.d + dc[2 * static_cast<size_t>(j) + 1] * cy.d;
         }
     }
     for (int j = 0; j < nc; ++j) {
