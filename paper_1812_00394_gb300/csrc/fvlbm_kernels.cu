@@ -376,24 +376,18 @@ __device__ __forceinline__ void block_sum(double (&v)[N], double *out) {
 // f^(J) = (X + zJ f^eq) / (1 + zJ), dt Gamma^c(J) = dt/tau (f^eq - X) / (1 + zJ) exactly, so a
 // rounding of X or f^eq is multiplied by dt/tau / (1 + zJ) <= 1/m_JJ instead of dt/tau.
 // Store of a stage value f^(2) or f^(3): structure of arrays, or (ROWS) the cell-major rows of
-// the face-value stages: alpha = 1..8 in pair order (1,3)(2,4)(5,7)(6,8) at f[8 i] (the two
-// halves swapped where bit 2 of i is set), f_0 at f[8 np + i].
+// the face-value stages in float (fv_store_stage, from f in alpha order): alpha = 1..8 in pair order
+// (1,3)(2,4)(5,7)(6,8) at f[8 i] (the two halves swapped where bit 2 of i is set), f_0 at f[8 np + i].
 template <class T, bool ROWS>
 __device__ __forceinline__ void store_stage(T *__restrict__ f, size_t np, int i, const T *o) {
     if constexpr (!ROWS) {
         store9(f, np, i, o);
     } else {
+        static_assert(std::is_same<T, float>::value, "double stages work on pairs (fv_store_stage)");
         T *row = f + 8 * static_cast<size_t>(i);
         const int sw = (i & 4) ? 4 : 0;  // halves swapped where bit 2 of the cell index is set
-        if constexpr (std::is_same<T, float>::value) {
-            *reinterpret_cast<float4 *>(row + sw) = make_float4(o[1], o[3], o[2], o[4]);
-            *reinterpret_cast<float4 *>(row + (sw ^ 4)) = make_float4(o[5], o[7], o[6], o[8]);
-        } else {
-            *reinterpret_cast<double2 *>(row + sw) = make_double2(o[1], o[3]);
-            *reinterpret_cast<double2 *>(row + sw + 2) = make_double2(o[2], o[4]);
-            *reinterpret_cast<double2 *>(row + (sw ^ 4)) = make_double2(o[5], o[7]);
-            *reinterpret_cast<double2 *>(row + (sw ^ 4) + 2) = make_double2(o[6], o[8]);
-        }
+        *reinterpret_cast<float4 *>(row + sw) = make_float4(o[1], o[3], o[2], o[4]);
+        *reinterpret_cast<float4 *>(row + (sw ^ 4)) = make_float4(o[5], o[7], o[6], o[8]);
         f[8 * np + i] = o[0];
     }
 }
@@ -1165,11 +1159,11 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
 #include "fvlbm_tangent.cuh"
 
 // ------------------------------------------------------------------ state I/O kernels
-// Records of N values per cell pass between the caller's order and the kernels' arrays through
-// shared memory, kIoBlock records at a time, so that the records are read and written as whole
-// cache lines: a thread that walks its own record touches a line per value (a 36-byte record: nine
-// times the transactions).  Gathering 640k FP32 records took 31.5 us that way, 14.2 now; packing
-// 200k cells for an exchange 16.6 and 13.9.
+// Output: records of N values per cell go to the caller's order through shared memory, kIoBlock records
+// at a time, and are written as whole cache lines: a thread that walks its own record touches a line
+// per value (a 36-byte record: nine times the transactions).  Gathering 640k FP32 records took 31.5 us
+// that way, 14.2 now; packing 200k cells for an exchange 16.6 and 13.9.  (Input: each thread reads its
+// own record, and the arrays are written coalesced.)
 constexpr int kIoBlock = 128;
 template <class V, int N>
 __device__ __forceinline__ void io_put(const V *sm, V *__restrict__ out, int j0, int n) {
@@ -2497,7 +2491,7 @@ int allocate_state(fvlbm_handle *h, const std::vector<const Prepared *> &P,
         if ((rc = dalloc(h, &h->f1, np * ts))) return rc;
     }
     // geometry, concatenated over instances with neighbour / boundary ids offset
-    std::vector<int> nbr(4 * np, kNone), back(4 * np, -1), nface(np, 0);
+    std::vector<int> nbr(4 * np, kNone), back(4 * np, -1);
     std::vector<int> btype(h->nbt), bowner(h->nbt), perm;
     std::vector<double> gq(8 * np, 0), dvec(8 * np, 0);
     std::vector<double> sn(8 * np, 0), lsq(8 * np, 0), rown(8 * np, 0), rnbr(8 * np, 0);
@@ -2525,7 +2519,6 @@ int allocate_state(fvlbm_handle *h, const std::vector<const Prepared *> &P,
                 gq[c * np + o + k] = p.gq[c * pn + k];
                 dvec[c * np + o + k] = p.dvec[c * pn + k];
             }
-        for (size_t k = 0; k < pn; ++k) nface[o + k] = p.nface[k];
         for (size_t k = 0; k < pn; ++k) {
             area[o + k] = p.area[k];
             wdist[o + k] = p.wdist[k];

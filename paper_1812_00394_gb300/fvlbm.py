@@ -346,8 +346,8 @@ def fvlbm_autotune(h, trial_steps: int = 5):
     chosen = C.c_int()
     ms = np.zeros(4)
     _check(load().fvlbm_autotune(h, int(trial_steps), C.byref(chosen), _p(ms)), "fvlbm_autotune")
-    names = ("fused256", "fused128", "twopass", "facevalue")
-    return names[chosen.value], {names[k]: float(ms[k]) for k in range(4) if ms[k] >= 0}
+    names = {2: "twopass", 3: "facevalue"}   # 0 and 1 are numbers of forms that no longer exist
+    return names[chosen.value], {nm: float(ms[k]) for k, nm in names.items() if ms[k] >= 0}
 
 
 def fvlbm_tangent_seed(h, instance: int, dbedge_val: np.ndarray | None = None,
