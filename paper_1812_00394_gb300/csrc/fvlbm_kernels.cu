@@ -131,6 +131,13 @@ __device__ __forceinline__ bool nonneg(double x) {
 }
 __device__ __forceinline__ bool nonneg(const Dual &x) { return nonneg(x.v); }
 
+// Threads per block of the two-pass kernels (kTwoPassBlock; a tile with statistics), in float a constant.
+template <class T>
+__device__ __forceinline__ unsigned block_width() { return sizeof(T) == 4 ? kTile : blockDim.x; }
+// Tile of the cells of a block.
+template <class T>
+__device__ __forceinline__ int block_tile(unsigned block) { return static_cast<int>(block * block_width<T>() / kTile); }
+
 // ------------------------------------------------------------------ cell algebra
 // Quotient a / b in the collision and stage algebra and in the SST gradients (limiter, f1).
 // In float it is the fast form (within 2 ulp instead of correctly rounded): the FP32 path
@@ -233,9 +240,9 @@ __device__ __forceinline__ void relax9(T *f, T rho0, T dt, T tau_i, T *eq_out = 
 template <class T>
 __global__ void __launch_bounds__(kTile) k_stage1(const T *__restrict__ fn, T *__restrict__ fs,
                                                   const T *__restrict__ tau, Geo<T> G) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * block_width<T>() + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[i / kTile]];
+    const InstParam P = G.ip[G.tile_inst[block_tile<T>(blockIdx.x)]];
     T f[kQ];
     load9(fn, np, i, f);
     relax9(f, ipv<T>(P.rho0, P.rho0_f), cell_dt(G, P, i), tau[i]);
@@ -247,11 +254,11 @@ __global__ void __launch_bounds__(kTile) k_stage1(const T *__restrict__ fn, T *_
 template <class T>
 __global__ void __launch_bounds__(kTile) k_stage_macros(const T *__restrict__ fs, T *__restrict__ mac,
                                                         Geo<T> G) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * block_width<T>() + threadIdx.x;
     const size_t np = G.np;
     T f[kQ], dr, r, u, v;
     load9(fs, np, i, f);
-    const InstParam &P = G.ip[G.tile_inst[i / kTile]];
+    const InstParam &P = G.ip[G.tile_inst[block_tile<T>(blockIdx.x)]];
     moments(f, ipv<T>(P.rho0, P.rho0_f), dr, r, u, v);
     mac[i] = r;
     mac[np + i] = u;
@@ -264,9 +271,9 @@ __global__ void __launch_bounds__(kTile) k_stage_macros(const T *__restrict__ fs
 template <class T, bool LIMIT>
 __global__ void __launch_bounds__(kTile) k_grad(const T *__restrict__ f, T *__restrict__ g,
                                                 Geo<T> G) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * block_width<T>() + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[i / kTile]];
+    const InstParam P = G.ip[G.tile_inst[block_tile<T>(blockIdx.x)]];
     const T rho0 = ipv<T>(P.rho0, P.rho0_f);
     T fi[kQ], gx[kQ], gy[kQ], lo[kQ], hi[kQ];
     load9(f, np, i, fi);
@@ -538,9 +545,9 @@ __global__ void __launch_bounds__(kTile)
                  T *__restrict__ fn, T *__restrict__ Bacc, T *__restrict__ Cacc,
                  const T *__restrict__ tau, T *__restrict__ mac, double *__restrict__ partial,
                  Geo<T> G, const T *__restrict__ tau1 = nullptr) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * block_width<T>() + threadIdx.x;
     const size_t np = G.np;
-    const InstParam P = G.ip[G.tile_inst[i / kTile]];
+    const InstParam P = G.ip[G.tile_inst[block_tile<T>(blockIdx.x)]];
     const T rho0 = ipv<T>(P.rho0, P.rho0_f);
     T fi[kQ], acc[kQ];
     load9(fs, np, i, fi);
@@ -969,7 +976,8 @@ __global__ void __launch_bounds__(kTile)
     k_sst_grad(const T *mac, const T *kk, const T *ww, T *__restrict__ grads, T *__restrict__ f1out, Geo<T> G,
                CompactGeo<T> CG, const T *nut, T *__restrict__ rec8, T *__restrict__ rec2, bool inv_only,
                int tile0) {
-    const int i = tile0 * kTile + static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x), tile = i / kTile;
+    const int i = tile0 * kTile + static_cast<int>(blockIdx.x * block_width<T>() + threadIdx.x);
+    const int tile = tile0 + block_tile<T>(blockIdx.x);
     const size_t np = G.np;
     const InstParam P = G.ip[G.tile_inst[tile]];
     const T nu = ipv<T>(P.nu, P.nu_f);
@@ -1056,8 +1064,9 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
                  T *__restrict__ k_out, T *__restrict__ w_out, T *__restrict__ nut_out, T *__restrict__ tau,
                  Geo<T> G, CompactGeo<T> CG, const T *rec8, const T *rec2, int tile0) {
     // backwards: the records that k_sst_grad wrote last are still in L2
-    const int i = tile0 * kTile + static_cast<int>((gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x);
-    const int tile = i / kTile;
+    const unsigned block = gridDim.x - 1 - blockIdx.x;
+    const int i = tile0 * kTile + static_cast<int>(block * block_width<T>() + threadIdx.x);
+    const int tile = tile0 + block_tile<T>(block);
     const size_t np = G.np;
     const InstParam P = G.ip[G.tile_inst[tile]];
     const T nu = ipv<T>(P.nu, P.nu_f);
@@ -1892,12 +1901,23 @@ constexpr int kTwoPassBlock = sizeof(T) == 8 ? 32 : kTile;
 
 // The two SST kernels of the two-pass path (unpacked gradients, geometry read as stored), on
 // stream h->stream: gradients and f1 of the macros mac, then k, omega, nu_t and tau_out.
+// Float: dependent launches, for which these kernels order their loads (FP32 airfoils, us a step, plain
+// and so: 2k cells 46.6 / 45.5, 200k cells 100.8 / 99.4, SST at every stage 150 / 145).  Double: plain (20k-cell
+// step with explicit Euler 95.4 against 99.3: see dep_launch).
+template <class T, class... P, class... A>
+void launch_sst_twopass(const fvlbm_handle *h, dim3 tiles, void (*kernel)(P...), A... args) {
+    const dim3 grid(tiles.x * (kTile / kTwoPassBlock<T>)), block(kTwoPassBlock<T>);
+    if (sizeof(T) == 4)
+        launch_dep(kernel, grid, block, 0, h->stream, args...);
+    else
+        kernel<<<grid, block, 0, h->stream>>>(args...);
+}
 template <class T>
 void sst_grad_twopass(const fvlbm_handle *h, const T *mac, const T *kc, const T *wc, T *sg, T *f1,
                       const Geo<T> &G, const CompactGeo<T> &CG) {
     for_sst_runs(h, [&](dim3 g, int t0) {
-        k_sst_grad<T, false><<<g.x * (kTile / kTwoPassBlock<T>), kTwoPassBlock<T>, 0, h->stream>>>(mac, kc, wc, sg, f1, G, CG, nullptr, nullptr,
-                                                         nullptr, false, t0);
+        launch_sst_twopass<T>(h, g, k_sst_grad<T, false>, mac, kc, wc, sg, f1, G, CG, nullptr, nullptr, nullptr, false,
+                              t0);
     });
 }
 template <class T>
@@ -1905,12 +1925,8 @@ void sst_update_twopass(const fvlbm_handle *h, const T *mac, const T *kc, const 
                         const T *sg, const T *f1, T *kn, T *wn, T *nn, T *tau_out, const Geo<T> &G,
                         const CompactGeo<T> &CG) {
     for_sst_runs(h, [&](dim3 g, int t0) {
-        if (h->nonorth)
-            k_sst_update<T, false, true><<<g.x * (kTile / kTwoPassBlock<T>), kTwoPassBlock<T>, 0, h->stream>>>(mac, kc, wc, nc, sg, f1, kn, wn, nn, tau_out,
-                                                                     G, CG, nullptr, nullptr, t0);
-        else
-            k_sst_update<T, false, false><<<g.x * (kTile / kTwoPassBlock<T>), kTwoPassBlock<T>, 0, h->stream>>>(mac, kc, wc, nc, sg, f1, kn, wn, nn, tau_out,
-                                                                      G, CG, nullptr, nullptr, t0);
+        launch_sst_twopass<T>(h, g, h->nonorth ? k_sst_update<T, false, true> : k_sst_update<T, false, false>, mac, kc,
+                              wc, nc, sg, f1, kn, wn, nn, tau_out, G, CG, nullptr, nullptr, t0);
     });
 }
 
