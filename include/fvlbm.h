@@ -198,7 +198,8 @@ int fvlbm_check_mesh(const fvlbm_mesh *mesh, const fvlbm_bc *bc, const fvlbm_par
                      double *dt, char *why, int why_len);
 
 /* Advance n_steps time steps (Steps 1-7 of Sec. 3.2 each), asynchronously on the handle's
- * stream.  Runs of 16 steps are replayed from a captured CUDA graph, the rest are launches.  On a
+ * stream.  Runs of 16 steps are replayed from a captured CUDA graph, the rest are launches (graphs of one
+ * step for laminar handles on the two-pass kernels).  On a
  * stream that the caller captures, laminar handles, runs of 16 steps and statistics return
  * FVLBM_ERR_CUDA and change nothing (so do fvlbm_profile_kernels and fvlbm_autotune).  Fewer steps
  * of an SST handle may be captured and replayed any number of times (an odd number copies k, omega
@@ -477,9 +478,9 @@ int fvlbm_set_adjoint_budget(fvlbm_handle *h, long long bytes);
 /* ---------------------------------------------------------------------------------------------
  * Checkpoint / resume and divergence rollback (no counterpart in the paper).
  *
- * The state of a handle -- f^n, f^(1) of the coming step, the macros, tau, k / omega / nu_t and
- * their ping-pong parity, and the step count -- as one opaque host blob in the handle's internal
- * cell order.  fvlbm_state_bytes gives its size; fvlbm_save_state writes it into buf (bytes at
+ * The state of a handle -- f^n, the macros, tau, k / omega / nu_t and their ping-pong parity, and
+ * the step count -- as one opaque host blob in the handle's internal cell order (blobs of version 1,
+ * which also hold f^(1) of the coming step, are read too).  fvlbm_state_bytes gives its size; fvlbm_save_state writes it into buf (bytes at
  * least that size); fvlbm_load_state restores it into this handle or into any handle created
  * from the same meshes and parameters (the preprocessing is deterministic).  The blob's header
  * carries the precision, the sizes and a checksum of the cell order; a blob of another

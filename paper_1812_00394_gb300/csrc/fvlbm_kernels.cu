@@ -1064,9 +1064,8 @@ __global__ void __launch_bounds__(kTile, sizeof(T) == 4 ? 5 : 1)
                  T *__restrict__ k_out, T *__restrict__ w_out, T *__restrict__ nut_out, T *__restrict__ tau,
                  Geo<T> G, CompactGeo<T> CG, const T *rec8, const T *rec2, int tile0) {
     // backwards: the records that k_sst_grad wrote last are still in L2
-    const unsigned block = gridDim.x - 1 - blockIdx.x;
-    const int i = tile0 * kTile + static_cast<int>(block * block_width<T>() + threadIdx.x);
-    const int tile = tile0 + block_tile<T>(block);
+    const int i = tile0 * kTile + static_cast<int>((gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x);
+    const int tile = i / kTile;  // (by thread: with the tile of the block 87.5 us against 82.6 on that batch)
     const size_t np = G.np;
     const InstParam P = G.ip[G.tile_inst[tile]];
     const T nu = ipv<T>(P.nu, P.nu_f);
